@@ -5,12 +5,20 @@
 //  - prefill_tc_kernel (this file): one CTA owns TWO query tiles of 128 rows of one (sequence, query head) and walks
 //    the KV cache in tiles of 128 keys, every K/V tile serving both query tiles:
 //      loader warp : TMA (tiled, 128-byte swizzle) Q once, then K/V tiles into 2-stage rings
-//      MMA warp    : one thread issues tcgen05.mma  S = Q K^T  and  O += P V, accumulators in TMEM
+//      MMA warps   : one thread issues the tcgen05.mma of S = Q K^T, another those of O += P V, accumulators in TMEM
 //      softmax WGs : one warpgroup per query tile, one thread per row holding the row's 128 scores in registers:
-//                    row maximum, P = exp2(...) with fp32-pair arithmetic written back over S as bf16 and released
-//                    to the MMA issuer in two parts; lazy rescale of O only when the maximum grew by > 2^8
-//    TMEM (512 columns): S_A | S_B | O_A | O_B (128 each).  For grids that cannot fill the SMs a cluster of 4 CTAs
-//    shares the pair of query tiles and splits the KV walk (template parameter CL).
+//                    row maximum, P = exp2(...) with fp32-pair arithmetic written to TMEM as bf16 and released to the
+//                    MMA issuer in two parts; lazy rescale of O only when the maximum grew by > 2^8
+//    TMEM (512 columns): O_A | O_B (128 each) | S (128) | P_A | P_B (64 each).  The one S buffer goes back and forth
+//    between the query tiles: a softmax holds it only while it reads its scores into registers, so the next tile's
+//    scores are computed during the softmax and not after O += P V has read P.  What bounds it: the softmax warps (two
+//    per scheduler, 2720 cycles per pair of tiles for 2048 of the special-function unit and as many of the tensor pipe), and the
+//    clock, which falls with the tensor pipe's use (about 1.5 GHz here).  Measured on four 8192-token prompts with 32 / 8
+//    heads in chunks of 512 (us a prompt set, in a burst / back to back), from P written over S and one issuing thread:
+//    2188 / 2390; P in its own columns and S shared, one issuer 2460 / 2613; two issuers 2024 / 2277; the PV
+//    issuer standing back for the scores 1963 / 2225; named barriers 1986 / 2223 (2720 against 3140 cycles per pair of
+//    tiles).  For grids that cannot fill the SMs a cluster of 4 CTAs shares the pair of query tiles and splits the KV
+//    walk (template parameter CL).
 //  - prefill_frag_kernel (prefill_tc_frag.cuh): one query tile per CTA, both warpgroups on it.
 // All mbarrier waits are bounded; on expiry the CTA sets the status word, drains its own copies and MMAs, frees
 // TMEM and returns.
@@ -56,13 +64,14 @@ struct TcCfg {
   static constexpr int KV_STAGES = 2;
   static constexpr int SOFTMAX_WARPS = 4 * TC_NQ;
   static constexpr int LOADER_WARP = SOFTMAX_WARPS;
-  static constexpr int MMA_WARP = SOFTMAX_WARPS + 1;
-  // Three full warpgroups (the third: loader, MMA issuer, two idle warps) so that the register file can be
+  static constexpr int QK_WARP = SOFTMAX_WARPS + 1, PV_WARP = SOFTMAX_WARPS + 2;
+  // Three full warpgroups (the third: loader, two MMA issuers, an idle warp) so that the register file can be
   // re-divided: a softmax thread holds a whole score row (REGS_SOFTMAX), the third warpgroup gives its share back
   // (REGS_OTHER); 2 x 128 x 208 + 128 x 88 = 384 x 168, the registers the CTA starts with.
   static constexpr int THREADS = 384;
   static constexpr int REGS_SOFTMAX = 208, REGS_OTHER = 88;
-  static constexpr int O_COL0 = 256;
+  // TMEM columns: O_0 | O_1 | S | P_0 | P_1
+  static constexpr int O_COL0 = 0, S_COL = 256, P_COL0 = 384;
   // shared memory: [Q tiles][K ring][V ring][barriers]
   static constexpr int SMEM_Q = 0;
   static constexpr int SMEM_K = TC_NQ * TC_TILE_BYTES;
@@ -80,11 +89,21 @@ enum {
   BAR_V_FULL = 6,    // [2]
   BAR_V_EMPTY = 8,   // [2]
   BAR_S_FULL = 10,   // [2] one per query tile
-  BAR_P_FULL = 12,   // [2]
-  BAR_O_READY = 14,  // [2]
-  BAR_P_EARLY = 16,  // [2] the first 96 columns of P are in TMEM
-  BAR_DRAIN = 18,
-  BAR_COUNT = 19
+  BAR_O_READY = 12,  // [2]
+  BAR_DRAIN = 14,    // [2] one per issuing thread
+  BAR_COUNT = 16
+};
+// Named barriers (hardware, not in shared memory): what a softmax warpgroup tells an issuing warp.  While the tensor
+// cores stream their operands an access to shared memory takes 100 to 200 cycles, and so does either side of an
+// mbarrier; a named barrier does not.  It cannot give up, so every thread passes every one of them whatever happened:
+// after a failed wait the tiles are walked on without meaning (and a softmax warp then waits instead of only
+// arriving, so that it cannot arrive twice at one phase).
+enum {
+  NB_STORE = 1,    // [2] the 128 threads of a query tile in the epilogue
+  NB_MERGE = 3,
+  NB_S_FREE = 4,   // [2] the softmax of query tile x has read its scores: the S buffer may be written again
+  NB_P_EARLY = 6,  // [2] the first 96 columns of P are in TMEM
+  NB_P_FULL = 8,   // [2]
 };
 
 constexpr int TC_BOX_FLOATS = TC_BM * 32;  // 16 KB
@@ -109,6 +128,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   const uint32_t sBar = smem_base + Cfg::SMEM_BAR;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + Cfg::SMEM_BAR + 8 * BAR_COUNT);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + Cfg::SMEM_BAR + 8 * BAR_COUNT + 8);
+  const uint32_t qk_turn = sBar + 8u * BAR_COUNT + 16u;  // odd while a batch of scores is being issued
+  static_assert(8 * BAR_COUNT + 20 <= 256, "barrier block");
   auto bar = [&](int i) { return sBar + 8u * i; };
 
   // a CTA of a cluster can meet rows that see none of a tile, and ends with unnormalised partials
@@ -146,11 +167,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 
   // ---- set-up
   if (threadIdx.x == 0) {
-    for (int i = 0; i < BAR_COUNT; ++i) mbar_init(bar(i), (i == BAR_P_FULL || i == BAR_P_FULL + 1 || i == BAR_P_EARLY || i == BAR_P_EARLY + 1) ? 128u : 1u);
+    for (int i = 0; i < BAR_COUNT; ++i) mbar_init(bar(i), 1u);
     *abort_flag = 0;
+    count_publish(qk_turn, 0);
     mbar_fence_init();
   }
-  if (warp == Cfg::MMA_WARP) {
+  if (warp == Cfg::QK_WARP) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
     tmem_relinquish();
   } else if (warp == Cfg::LOADER_WARP && lane == 0) {
@@ -248,99 +270,92 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       }
     }
     __syncwarp();
-  } else if (warp == Cfg::MMA_WARP) {
-    // =============================================================== MMA issuer
+  } else if (warp == Cfg::QK_WARP) {
+    // =============================================================== issuer of S = Q K^T
+    // Two threads issue the MMAs, one the scores and one the products with V: an issuing thread is held up while the
+    // tensor pipe works through what it has queued, so the barrier tests and commits between two batches of a single
+    // thread leave the pipe idle; with two threads the pipe works on one batch while the other thread prepares its
+    // next.  The issue loops are kept to an integer addition or two per MMA (descriptor halves, see tc_desc_lo).
     reg_dec<Cfg::REGS_OTHER>();
-    if (lane == 0) {
-      constexpr uint32_t idesc_qk = tc_idesc_bf16(TC_BM, TC_BN, false, false);
-      constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, TC_D, false, true);
-      auto s_col = [&](int x) { return tmem + x * 128; };
-      auto o_col = [&](int x) { return tmem + Cfg::O_COL0 + x * 128; };
-      // The issue loops are kept to an integer addition or two per MMA (descriptor halves, see tc_desc_lo): this
-      // thread shares its scheduler with two softmax warps, and a longer chain of address arithmetic per MMA
-      // made the issue, not the tensor pipe, the limit.
-      auto issue_qk = [&](int x, int g) {  // S(x) = Q(x) K^T, K of load sequence number g
-        const uint32_t q_lo = tc_desc_lo(sQ + x * TC_TILE_BYTES, 16);
-        const uint32_t k_lo = tc_desc_lo(sK + (g % KV_STAGES) * TC_TILE_BYTES, 16);
-        const uint32_t d = s_col(x);
-#pragma unroll
-        for (int ks = 0; ks < TC_D / 16; ++ks) {
-          const uint32_t off = ((ks >> 2) * TC_PANEL_BYTES + (ks & 3) * 32) >> 4;
-          tc_mma_ss_lo(d, q_lo + off, k_lo + off, idesc_qk, ks > 0);
-        }
-      };
-      // O(x) (+)= P(x) V over the keys [16 ks0, 16 ks1) of the tile, V of load sequence number g
-      auto issue_pv = [&](int x, int g, bool first, int ks0, int ks1) {
-        const uint32_t v_lo = tc_desc_lo(sV + (g % KV_STAGES) * TC_TILE_BYTES, TC_PANEL_BYTES);
-        const uint32_t d = o_col(x), a = s_col(x);
-#pragma unroll
-        for (int ks = ks0; ks < ks1; ++ks)
-          tc_mma_ts_lo(d, a + ks * 8, v_lo + ks * (2048 >> 4), idesc_pv, (!first || ks > 0));
-      };
-      auto last_user = [&](int g) {  // the last query tile (in issue order) that uses the tile of sequence number g
-        int r = -1;
-#pragma unroll
-        for (int x = 0; x < NQ; ++x)
-          if (g < T[x]) r = x;
-        return r;
-      };
-      bool ok = true;
-      int k_waited = -1, v_waited = -1;
-      auto need_k = [&](int j) {
-        if (k_waited < j) {
-          ok = ok && mbar_wait(bar(BAR_K_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
-          k_waited = j;
-          tc_fence_after();
-        }
-      };
-      auto need_v = [&](int j) {
-        if (v_waited < j) {
-          ok = ok && mbar_wait(bar(BAR_V_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
-          v_waited = j;
-          tc_fence_after();
-        }
-      };
-      // prologue: S(x, 0)
+    constexpr uint32_t idesc_qk = tc_idesc_bf16(TC_BM, TC_BN, false, false);
+    const uint32_t s_col = tmem + Cfg::S_COL;
+    bool ok = true;
+    // One S buffer serves both query tiles: it may be written once the softmax that got the previous scores has
+    // read them (a fraction of a tile's time), long before that tile's P V is due, so the scores are complete when
+    // the softmax comes for them and only its own work is on a tile's critical path.
+    int prev_x = -1;  // owner of the scores written last
+    int turn = 0;
+    for (int j = 0; j < Tall; ++j) {
+      const uint32_t k_lo = tc_desc_lo(sK + (j % KV_STAGES) * TC_TILE_BYTES, 16);
+      if (lane == 0) ok = ok && mbar_wait(bar(BAR_K_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
-        if (T[x] == 0 || !ok) continue;
-        ok = ok && mbar_wait(bar(BAR_Q_FULL + x), 0, abort_flag, p.status);
-        need_k(0);
-        if (!ok) break;
-        issue_qk(x, 0);
-        tc_commit(bar(BAR_S_FULL + x));
-        if (x == last_user(0)) tc_commit(bar(BAR_K_EMPTY + 0));
-      }
-      for (int j = 0; j < Tall && ok; ++j) {
+        if (j >= T[x]) continue;
+        if (j == 0 && lane == 0) ok = ok && mbar_wait(bar(BAR_Q_FULL + x), 0, abort_flag, p.status);
+        if (prev_x >= 0) named_sync(NB_S_FREE + prev_x, 160);
+        prev_x = x;
+        if (lane == 0 && ok) {
+          flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
+          tc_fence_after();
+          const uint32_t q_lo = tc_desc_lo(sQ + x * TC_TILE_BYTES, 16);
 #pragma unroll
-        for (int x = 0; x < NQ; ++x) {
-          if (j >= T[x] || !ok) continue;
-          const int g = j, gn = j + 1;  // load sequence numbers
-          need_v(g);
-          ok = ok && mbar_wait(bar(BAR_P_EARLY + x), j & 1, abort_flag, p.status);
-          if (!ok) break;
-          tc_fence_after();
-          issue_pv(x, g, j == 0, 0, 6);  // the first 96 keys while the softmax finishes the last 32
-          ok = ok && mbar_wait(bar(BAR_P_FULL + x), j & 1, abort_flag, p.status);
-          if (!ok) break;
-          tc_fence_after();
-          issue_pv(x, g, j == 0, 6, 8);
-          tc_commit(bar(BAR_O_READY + x));
-          if (x == last_user(g)) tc_commit(bar(BAR_V_EMPTY + g % KV_STAGES));
-          if (j + 1 < T[x]) {
-            need_k(gn);
-            if (!ok) break;
-            issue_qk(x, gn);
-            tc_commit(bar(BAR_S_FULL + x));
-            if (x == last_user(gn)) tc_commit(bar(BAR_K_EMPTY + gn % KV_STAGES));
+          for (int ks = 0; ks < TC_D / 16; ++ks) {
+            const uint32_t off = ((ks >> 2) * TC_PANEL_BYTES + (ks & 3) * 32) >> 4;
+            tc_mma_ss_lo(s_col, q_lo + off, k_lo + off, idesc_qk, ks > 0);
           }
+          tc_commit(bar(BAR_S_FULL + x));
+          flag_write(qk_turn, ++turn);
         }
+        __syncwarp();
       }
-      if (!ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
-        int dummy = 0;
-        tc_commit(bar(BAR_DRAIN));
-        mbar_wait(bar(BAR_DRAIN), 0, &dummy, nullptr);
+      if (lane == 0 && ok) tc_commit(bar(BAR_K_EMPTY + j % KV_STAGES));
+    }
+    if (prev_x >= 0) named_sync(NB_S_FREE + prev_x, 160);
+    if (lane == 0 && !ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
+      int dummy = 0;
+      tc_commit(bar(BAR_DRAIN));
+      mbar_wait(bar(BAR_DRAIN), 0, &dummy, nullptr);
+    }
+    __syncwarp();
+  } else if (warp == Cfg::PV_WARP) {
+    // =============================================================== issuer of O += P V
+    // The pipe serves the two threads' MMAs in turn, which would double the time to the next scores, and those are
+    // what everybody waits for: this thread stands back while a batch of scores is being issued.  (Looked at once per
+    // batch: the shared-memory read takes longer than an MMA.)
+    reg_dec<Cfg::REGS_OTHER>();
+    constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, TC_D, false, true);
+    bool ok = true;
+    for (int j = 0; j < Tall; ++j) {
+      const uint32_t v_lo = tc_desc_lo(sV + (j % KV_STAGES) * TC_TILE_BYTES, TC_PANEL_BYTES);
+      if (lane == 0) ok = ok && mbar_wait(bar(BAR_V_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
+#pragma unroll
+      for (int x = 0; x < NQ; ++x) {
+        if (j >= T[x]) continue;
+        const uint32_t o_col = tmem + Cfg::O_COL0 + x * 128, p_col = tmem + Cfg::P_COL0 + x * 64;
+        named_sync(NB_P_EARLY + x, 160);  // the first 96 keys while the softmax finishes the last 32
+        if (lane == 0 && ok) {
+          for (int it = 0; it < 4096 && (flag_read(qk_turn) & 1); ++it) {}
+          tc_fence_after();
+#pragma unroll
+          for (int ks = 0; ks < 6; ++ks)
+            tc_mma_ts_lo(o_col, p_col + ks * 8, v_lo + ks * (2048 >> 4), idesc_pv, (j > 0 || ks > 0));
+        }
+        __syncwarp();
+        named_sync(NB_P_FULL + x, 160);
+        if (lane == 0 && ok) {
+          tc_fence_after();
+#pragma unroll
+          for (int ks = 6; ks < 8; ++ks) tc_mma_ts_lo(o_col, p_col + ks * 8, v_lo + ks * (2048 >> 4), idesc_pv, 1);
+          tc_commit(bar(BAR_O_READY + x));
+        }
+        __syncwarp();
       }
+      if (lane == 0 && ok) tc_commit(bar(BAR_V_EMPTY + j % KV_STAGES));
+    }
+    if (lane == 0 && !ok) {
+      int dummy = 0;
+      tc_commit(bar(BAR_DRAIN + 1));
+      mbar_wait(bar(BAR_DRAIN + 1), 0, &dummy, nullptr);
     }
     __syncwarp();
   } else if (warp < Cfg::SOFTMAX_WARPS) {
@@ -357,28 +372,30 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
     const int Tx = T[x];
-    for (int j = 0; j < Tx && ok; ++j) {
-      const uint32_t tS = tmem + lane_base + x * 128;
-      ok = mbar_wait(bar(BAR_S_FULL + x), j & 1, abort_flag, p.status);
-      if (!ok) break;
+    auto signal = [&](int id) {
+      tc_fence_before();
+      if (ok) named_arrive(id + x, 160);
+      else named_sync(id + x, 160);
+    };
+    for (int j = 0; j < Tx; ++j) {
+      const uint32_t tS = tmem + lane_base + Cfg::S_COL, tP = tmem + lane_base + Cfg::P_COL0 + x * 64;
+      // (ok is the same in all lanes of a warp: the barriers and the tcgen05 operations are warp-collective)
+      ok = __all_sync(0xffffffffu, ok && mbar_spin_wait(bar(BAR_S_FULL + x), j & 1, abort_flag, p.status));
       tc_fence_after();
       // columns >= nvalid are masked: the end of the prefix in its last tile, the causal limit afterwards
       const int g = tile_of_seq(j);
       const int nvalid = g < Tp ? p.prefix_len - g * TC_BN : lim - (g - Tp) * TC_BN;
-      // warp-uniform flag, so the warp stays converged for the collective tcgen05 operations
       const bool masked = __any_sync(0xffffffffu, nvalid < TC_BN);
-      // (the accumulator's barrier is only consulted when O has to be rescaled: phase j - 1 cannot be overtaken,
-      // because PV(j) needs this thread's P(j))
-      ok = softmax_tile_row<PARTIAL>(
-          tS, tO, j, masked, ColumnLimit{nvalid}, c, m_ref, l,
-          [&] { return mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
+      softmax_tile_row<PARTIAL>(
+          tS, tP, tO, j, masked, ColumnLimit{nvalid}, c, m_ref, l,
+          [&] { return mbar_test_wait(bar(BAR_O_READY + x), (j - 1) & 1); },
+          [&] { ok = ok && mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
+          [&] { signal(NB_S_FREE); },
           [&] {
-            tc_fence_before();
-            mbar_arrive(bar(BAR_P_EARLY + x));
+            ok = __all_sync(0xffffffffu, ok);
+            signal(NB_P_EARLY);
           });
-      if (!ok) break;
-      tc_fence_before();
-      mbar_arrive(bar(BAR_P_FULL + x));
+      signal(NB_P_FULL);
     }
     pdl_launch_dependents();  // the next kernel of the stream may start its own set-up now
     if constexpr (CL > 1) {
@@ -410,7 +427,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
           stage_box_row(stage + q2 * TC_BOX_FLOATS, row_in_tile, v);
         }
         fence_proxy_async();
-        asm volatile("bar.sync %0, 128;\n" ::"r"(1 + x) : "memory");
+        named_sync(NB_STORE + x, 128);
         if (tid_t == 0) {
           if (ok) {
             tma_store_4d(&tm_o, stage_addr, hh * 64, h, tile_row0, b);
@@ -419,7 +436,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
           }
           tma_store_wait_read();  // the boxes are rewritten next / shared memory is released at the end of the kernel
         }
-        if (hh == 0) asm volatile("bar.sync %0, 128;\n" ::"r"(1 + x) : "memory");
+        if (hh == 0) named_sync(NB_STORE + x, 128);
       }
       if (ok && p.lse && row_valid)
         p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row] =
@@ -428,7 +445,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   }
 
   else {
-    reg_dec<Cfg::REGS_OTHER>();  // the idle warps of the third warpgroup: the re-division is a warpgroup's decision
+    reg_dec<Cfg::REGS_OTHER>();  // the idle warp of the third warpgroup: the re-division is a warpgroup's decision
   }
 
   if constexpr (CL > 1) {
@@ -468,7 +485,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
               make_float4(__uint_as_float(o[4 * cc]), __uint_as_float(o[4 * cc + 1]), __uint_as_float(o[4 * cc + 2]),
                           __uint_as_float(o[4 * cc + 3]));
       }
-      asm volatile("bar.sync 3, 256;\n" ::: "memory");
+      named_sync(NB_MERGE, 256);
       const float4* src = reinterpret_cast<const float4*>(part);
       float4* dst = reinterpret_cast<float4*>(gpart + crank * TC_PART_FLOATS);
 #pragma unroll 8
@@ -551,7 +568,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   // ---- tear-down
   tc_fence_before();
   __syncthreads();
-  if (warp == Cfg::MMA_WARP) {
+  if (warp == Cfg::QK_WARP) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }

@@ -109,6 +109,15 @@ __device__ __forceinline__ int count_read(uint32_t addr) {
   asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
+// The same word without ordering, for hints.
+__device__ __forceinline__ void flag_write(uint32_t addr, int value) {
+  asm volatile("st.relaxed.cta.shared::cta.b32 [%0], %1;\n" ::"r"(addr), "r"(value) : "memory");
+}
+__device__ __forceinline__ int flag_read(uint32_t addr) {
+  int v;
+  asm volatile("ld.relaxed.cta.shared::cta.b32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
 // Bounded wait until the counter reaches `need`; gives up like mbar_wait.
 __device__ __forceinline__ bool count_wait(uint32_t addr, int need, volatile int* abort_flag, int* status,
                                            long long limit_cycles) {
@@ -179,6 +188,14 @@ struct PollGuard {
     return false;
   }
 };
+
+// Named barriers: the calling warp (all lanes, converged) arrives, or arrives and waits; `threads` counts both kinds.
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
 
 // ---------------------------------------------------------------- thread-block cluster, distributed shared memory
 __device__ __forceinline__ uint32_t cluster_ctarank() {

@@ -1,12 +1,12 @@
 // The online-softmax steps of the tcgen05 attention kernels, three forms of the same arithmetic -- P = exp2(s c - m)
-// with fp32-pair instructions, written back over S in TMEM as bf16 pairs (P column k holds keys 2k and 2k + 1, so the
-// writes stay behind the reads), a lazy reference maximum m that only moves when the tile's maximum outgrew it by more
+// with fp32-pair instructions, written to TMEM as bf16 pairs (P column k holds keys 2k and 2k + 1; over S in two of the
+// forms, where the writes stay behind the reads), a lazy reference maximum m that only moves when the tile's maximum outgrew it by more
 // than 2^8 (then the row sum and the accumulator O are scaled by exp2(m_old - m_new); with well-behaved scores that
 // happens in a row's first tile and almost never again):
 //   softmax_tile_step : a thread per row, the row's 128 scores walked once in four chunks of 32 columns with the next
 //                       chunk in flight (about 160 registers; the branch kernel)
-//   softmax_tile_row  : a thread per row holding the whole row (about 200 registers), P released in two parts (the
-//                       two-tile prefill kernel)
+//   softmax_tile_row  : a thread per row holding the whole row (about 200 registers), S given back as soon as it is
+//                       read, P in columns of its own and released in two parts (the two-tile prefill kernel)
 //   frag_*            : 16 rows per warp in the 16x256b fragment layout, in pieces that a kernel interleaves across
 //                       consecutive tiles (the one-tile prefill kernel)
 #pragma once
@@ -143,20 +143,25 @@ __device__ __forceinline__ bool softmax_tile_step(uint32_t tS, uint32_t tO, int 
   return true;
 }
 
-// The same step with the whole score row in registers (needs about 200 registers per thread): one load of the 128
-// scores, the row maximum, at most one move of the reference per tile (decided before any P is written, so no P
-// chunk is ever corrected), then P in four chunks of 32 columns.  After the third chunk is in TMEM (tcgen05.wait::st
-// done) release_early() runs: the caller signals the MMA issuer, which starts O += P V on the first 96 keys while
-// this thread still computes the last 32.  wait_o() is only called when the accumulator has to be rescaled
-// (j > 0); it waits until O(j-1) is complete and returns false if the wait gave up, and then so does this function.
+// The same step with the whole score row in registers (needs about 200 registers per thread) and P in columns of its
+// own (tP), so that the S buffer is free as soon as the scores have been read: loaded() runs then, and the caller
+// passes the buffer on to the MMA issuer before anything is computed.  At most one move of the reference per tile
+// (decided before any P is written, so no P chunk is ever corrected); P in four chunks of 32 columns.  After the third
+// chunk is in TMEM (tcgen05.wait::st done) release_early() runs: the caller signals the MMA issuer, which starts
+// O += P V on the first 96 keys while this thread still computes the last 32.  Before the accumulator is rescaled or the
+// previous P overwritten, O += P V of the stream's previous tile must be complete: test_o() tests that without
+// waiting, under the latency of the score load (it nearly always is), and wait_o() waits otherwise (j > 0 only).
 // On return P is complete in TMEM; the caller fences and signals the second half.
-template <bool PARTIAL, class Allow, class WaitO, class Release>
-__device__ __forceinline__ bool softmax_tile_row(uint32_t tS, uint32_t tO, int j, bool masked, const Allow& allow, float c,
-                                                 float& m_ref, float& l, WaitO&& wait_o, Release&& release_early) {
+template <bool PARTIAL, class Allow, class TestO, class WaitO, class Loaded, class Release>
+__device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint32_t tO, int j, bool masked,
+                                                 const Allow& allow, float c, float& m_ref, float& l, TestO&& test_o,
+                                                 WaitO&& wait_o, Loaded&& loaded, Release&& release_early) {
   uint32_t sv[128];
 #pragma unroll
   for (int q4 = 0; q4 < 4; ++q4) tmem_ld32(tS + q4 * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[q4 * 32]));
+  const bool o_here = j == 0 || test_o();
   tc_wait_ld();
+  loaded();
   if (masked) {
 #pragma unroll
     for (int i = 0; i < 128; ++i)
@@ -182,13 +187,13 @@ __device__ __forceinline__ bool softmax_tile_row(uint32_t tS, uint32_t tO, int j
   // lazy reference: it only moves when the maximum outgrew it by 2^8 (a row that has seen nothing keeps -inf,
   // and its first visible score moves it because -inf + 8 is still -inf)
   const bool grow = mxs > m_ref + TC_RESCALE_THRESHOLD;
+  if (!o_here) wait_o();
+  tc_fence_after();
   if (__any_sync(0xffffffffu, grow)) {
     const float alpha = grow ? fast_exp2(m_ref - mxs) : 1.f;
     l *= alpha;
     if (grow) m_ref = mxs;
-    if (j > 0) {  // O(j-1) must be complete before it is rescaled
-      if (!wait_o()) return false;
-      tc_fence_after();
+    if (j > 0) {
 #pragma unroll
       for (int q4 = 0; q4 < 4; ++q4) {
         uint32_t o[32];
@@ -219,7 +224,7 @@ __device__ __forceinline__ bool softmax_tile_row(uint32_t tS, uint32_t tO, int j
       lacc[i & 3] = add2(lacc[i & 3], pack2(p0, p1));
       pk[i] = pack_bf16(p0, p1);
     }
-    tmem_st16(tS + q4 * 16, pk);
+    tmem_st16(tP + q4 * 16, pk);
     if (q4 == 2) {
       tc_wait_st();
       release_early();
@@ -232,7 +237,6 @@ __device__ __forceinline__ bool softmax_tile_row(uint32_t tS, uint32_t tO, int j
     l += (a0 + a1) + (b0 + b1);
   }
   tc_wait_st();
-  return true;
 }
 
 // ---------------------------------------------------------------- fragment form

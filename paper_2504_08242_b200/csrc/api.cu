@@ -304,14 +304,13 @@ static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const ju
   // to the tensor-core kernel (which adapts to the scratch it is given); the rest to the split-KV kernel, the only one that can find the
   // scratch too small
   DeviceGuard guard(ctx->device);
-  const bool tc_ok = jup::branch_tc_supported(sfx, prefix_len, max_suffix_len, n_branches, q_heads, q_len, scale,
-                                              ctx->sm_count);
+  const bool tc_ok = jup::branch_tc_supported(sfx, n_branches, q_heads, q_len, scale);
   bool use_stream, use_tc;
   switch (ctx->branch_kernel) {
     case JUPITER_BRANCH_STREAM: use_stream = true, use_tc = false; break;
     case JUPITER_BRANCH_SPLIT_KV: use_stream = use_tc = false; break;
     case JUPITER_BRANCH_TENSOR_CORE:
-      if (!tc_ok) return JUPITER_ERR_UNSUPPORTED;
+      if (!tc_ok || sfx.head_dim != 128) return JUPITER_ERR_UNSUPPORTED;
       use_stream = false, use_tc = true;
       break;
     default:
@@ -329,11 +328,13 @@ static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const ju
                                   max_suffix_len, n_branches, q_heads, q_len, scale, out, lse,
                                   static_cast<cudaStream_t>(stream), li, static_cast<const bf16*>(k_new),
                                   static_cast<const bf16*>(v_new));
-  else if (use_tc)
-    e = jup::launch_branch_tc(static_cast<const bf16*>(q), pfx, prefix_len, sfx, d_suffix_len, d_tree_mask,
-                              max_suffix_len, n_branches, q_heads, q_len, scale, out, lse, ctx->d_status,
-                              ctx->wait_limit, ctx->workspace, ctx->workspace_bytes, static_cast<cudaStream_t>(stream),
-                              li, static_cast<const bf16*>(k_new), static_cast<const bf16*>(v_new));
+  else if (use_tc) {
+    const jup::BranchLayerTensors t{static_cast<const bf16*>(q), static_cast<const bf16*>(k_new),
+                                    static_cast<const bf16*>(v_new), pfx.k, pfx.v, sfx.k, sfx.v, out, lse};
+    e = jup::launch_branch_tc_layers(&t, 1, pfx, prefix_len, sfx, d_suffix_len, d_tree_mask, max_suffix_len, n_branches,
+                                     q_heads, q_len, scale, ctx->d_status, ctx->wait_limit, ctx->workspace,
+                                     ctx->workspace_bytes, static_cast<cudaStream_t>(stream), li);
+  }
   else
     e = jup::launch_branch(static_cast<const bf16*>(q), pfx, prefix_len, sfx, d_suffix_len, d_tree_mask,
                            max_suffix_len, n_branches, q_heads, q_len, scale, out, lse, ctx->workspace,
@@ -383,13 +384,19 @@ jupiter_status jupiter_branch_append_attn_layers(jupiter_ctx* ctx, const jupiter
     t[l] = jup::BranchLayerTensors{static_cast<const bf16*>(L.q), static_cast<const bf16*>(L.k_new),
                                    static_cast<const bf16*>(L.v_new), pfx.k, pfx.v, sfx.k, sfx.v, L.out, L.lse};
   }
+  const bool stream_kernel = jup::branch_stream_preferred(n_branches, q_heads, sfx0.kv_heads, q_len, ctx->sm_count);
   if (ctx->branch_kernel == JUPITER_BRANCH_AUTO &&
-      jup::branch_stream_preferred(n_branches, q_heads, sfx0.kv_heads, q_len, ctx->sm_count)) {
+      (stream_kernel || jup::branch_tc_supported(sfx0, n_branches, q_heads, q_len, scale))) {
     DeviceGuard guard(ctx->device);
     jup::LaunchInfo li{ctx->sm_count, 0};
-    cudaError_t e = jup::launch_branch_stream_layers(t.data(), n_layers, pfx0, prefix_len, sfx0, d_suffix_len,
-                                                     max_suffix_len, n_branches, q_heads, q_len, scale,
-                                                     static_cast<cudaStream_t>(stream), li);
+    cudaError_t e;
+    if (stream_kernel)
+      e = jup::launch_branch_stream_layers(t.data(), n_layers, pfx0, prefix_len, sfx0, d_suffix_len, max_suffix_len,
+                                           n_branches, q_heads, q_len, scale, static_cast<cudaStream_t>(stream), li);
+    else
+      e = jup::launch_branch_tc_layers(t.data(), n_layers, pfx0, prefix_len, sfx0, d_suffix_len, nullptr, max_suffix_len,
+                                       n_branches, q_heads, q_len, scale, ctx->d_status, ctx->wait_limit, ctx->workspace,
+                                       ctx->workspace_bytes, static_cast<cudaStream_t>(stream), li);
     ctx->launches += li.launches;
     return e == cudaSuccess ? JUPITER_OK : cuda_fail(ctx, e, "branch_append_attn_layers");
   }

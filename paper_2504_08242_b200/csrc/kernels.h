@@ -88,36 +88,7 @@ cudaError_t launch_branch(const bf16* q, const CacheView& prefix, int prefix_len
                           int q_heads, int q_len, float scale, float* out, float* lse, void* workspace,
                           cudaStream_t st, LaunchInfo& li, const bf16* k_new = nullptr, const bf16* v_new = nullptr);
 
-// Streaming form of branch attention: clusters walk prefix + suffixes with one softmax state per row and merge
-// through distributed shared memory; no scratch.  Preferred when all stacked rows of a kv head fit one 16-row tile, or
-// when the (kv head, 16-row tile) units all run at once.
-bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_len, int sm_count);
-cudaError_t launch_branch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,
-                                 const int32_t* d_suffix_len, const uint32_t* d_tree_mask, int max_suffix_len,
-                                 int n_branches, int q_heads, int q_len, float scale, float* out, float* lse,
-                                 cudaStream_t st, LaunchInfo& li, const bf16* k_new = nullptr,
-                                 const bf16* v_new = nullptr);
-
-// Branch attention on tcgen05 / TMEM for many stacked rows per kv head (head_dim 128, positive finite scale; a
-// branch's q_len x group rows must fit a 128-row tile or the group size must divide 128): units of (kv head, row
-// tile) walk prefix + suffixes with one softmax state per row; the CTAs that share a unit form a thread-block
-// cluster and exchange their partials through the scratch (with too little of it a unit is walked by one CTA, so
-// the call never fails for lack of scratch).  Both calls need the target device current.
-bool branch_tc_supported(const CacheView& suffix, int prefix_len, int max_suffix_len, int n_branches, int q_heads,
-                         int q_len, float scale, int sm_count);
-cudaError_t launch_branch_tc(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,
-                             const int32_t* d_suffix_len, const uint32_t* d_tree_mask, int max_suffix_len,
-                             int n_branches, int q_heads, int q_len, float scale, float* out, float* lse, int* status,
-                             long long wait_limit, void* workspace, size_t workspace_bytes, cudaStream_t st,
-                             LaunchInfo& li, const bf16* k_new = nullptr, const bf16* v_new = nullptr);
-
-// One CTA that waits, for at most limit_cycles SM clocks, on a barrier nobody arrives at, then reports through the
-// status word like any kernel whose bounded wait ran out.
-cudaError_t launch_wait_probe(int* status, long long limit_cycles, cudaStream_t st, LaunchInfo& li);
-
-// The same step for several decoder layers in one launch of the streaming kernel (at most
-// kBranchMaxLayersPerLaunch per launch; more layers take further launches): every layer has its own tensors, all
-// share the geometry of `prefix` / `suffix` (whose own k / v are ignored), the lengths and the scale.
+// One layer of a branch-attention step; a launch takes at most kBranchMaxLayersPerLaunch of them.
 constexpr int kBranchMaxLayersPerLaunch = 16;
 struct BranchLayerTensors {
   const bf16* q;
@@ -130,6 +101,37 @@ struct BranchLayerTensors {
   float* out;
   float* lse;  // nullable
 };
+
+// Streaming form of branch attention: clusters walk prefix + suffixes with one softmax state per row and merge
+// through distributed shared memory; no scratch.  Preferred when all stacked rows of a kv head fit one 16-row tile, or
+// when the (kv head, 16-row tile) units all run at once.
+bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_len, int sm_count);
+cudaError_t launch_branch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,
+                                 const int32_t* d_suffix_len, const uint32_t* d_tree_mask, int max_suffix_len,
+                                 int n_branches, int q_heads, int q_len, float scale, float* out, float* lse,
+                                 cudaStream_t st, LaunchInfo& li, const bf16* k_new = nullptr,
+                                 const bf16* v_new = nullptr);
+
+// Branch attention on tcgen05 / TMEM for many stacked rows per kv head (positive finite scale; a
+// branch's q_len x group rows must fit a 128-row tile or the group size must divide 128): units of (kv head, row
+// tile) walk prefix + suffixes with one softmax state per row; the CTAs that share a unit form a thread-block
+// cluster and exchange their partials through the scratch (with too little of it a unit is walked by one CTA, so
+// the call never fails for lack of scratch).  Both calls need the target device current.
+bool branch_tc_supported(const CacheView& suffix, int n_branches, int q_heads, int q_len, float scale);
+// Several layers of the same geometry (prefix / suffix, whose own k / v are ignored) share a launch.
+cudaError_t launch_branch_tc_layers(const BranchLayerTensors* layers, int n_layers, const CacheView& prefix, int prefix_len,
+                                    const CacheView& suffix, const int32_t* d_suffix_len, const uint32_t* d_tree_mask,
+                                    int max_suffix_len, int n_branches, int q_heads, int q_len, float scale, int* status,
+                                    long long wait_limit, void* workspace, size_t workspace_bytes, cudaStream_t st,
+                                    LaunchInfo& li);
+
+// One CTA that waits, for at most limit_cycles SM clocks, on a barrier nobody arrives at, then reports through the
+// status word like any kernel whose bounded wait ran out.
+cudaError_t launch_wait_probe(int* status, long long limit_cycles, cudaStream_t st, LaunchInfo& li);
+
+// The same step for several decoder layers in one launch of the streaming kernel (at most
+// kBranchMaxLayersPerLaunch per launch; more layers take further launches): every layer has its own tensors, all
+// share the geometry of `prefix` / `suffix` (whose own k / v are ignored), the lengths and the scale.
 cudaError_t launch_branch_stream_layers(const BranchLayerTensors* layers, int n_layers, const CacheView& prefix,
                                         int prefix_len, const CacheView& suffix, const int32_t* d_suffix_len,
                                         int max_suffix_len, int n_branches, int q_heads, int q_len, float scale,

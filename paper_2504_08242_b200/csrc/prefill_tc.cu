@@ -93,19 +93,6 @@ enum {
   BAR_DRAIN = 14,    // [2] one per issuing thread
   BAR_COUNT = 16
 };
-// Named barriers (hardware, not in shared memory): what a softmax warpgroup tells an issuing warp.  While the tensor
-// cores stream their operands an access to shared memory takes 100 to 200 cycles, and so does either side of an
-// mbarrier; a named barrier does not.  It cannot give up, so every thread passes every one of them whatever happened:
-// after a failed wait the tiles are walked on without meaning (and a softmax warp then waits instead of only
-// arriving, so that it cannot arrive twice at one phase).
-enum {
-  NB_STORE = 1,    // [2] the 128 threads of a query tile in the epilogue
-  NB_MERGE = 3,
-  NB_S_FREE = 4,   // [2] the softmax of query tile x has read its scores: the S buffer may be written again
-  NB_P_EARLY = 6,  // [2] the first 96 columns of P are in TMEM
-  NB_P_FULL = 8,   // [2]
-};
-
 constexpr int TC_BOX_FLOATS = TC_BM * 32;  // 16 KB
 constexpr int NQ = TC_NQ;
 
@@ -386,8 +373,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       const int g = tile_of_seq(j);
       const int nvalid = g < Tp ? p.prefix_len - g * TC_BN : lim - (g - Tp) * TC_BN;
       const bool masked = __any_sync(0xffffffffu, nvalid < TC_BN);
-      softmax_tile_row<PARTIAL>(
-          tS, tP, tO, j, masked, ColumnLimit{nvalid}, c, m_ref, l,
+      softmax_tile_row<PARTIAL, TC_D>(
+          tS, tP, tO, j, 4, masked, ColumnLimit{nvalid}, c, m_ref, l,
           [&] { return mbar_test_wait(bar(BAR_O_READY + x), (j - 1) & 1); },
           [&] { ok = ok && mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
           [&] { signal(NB_S_FREE); },

@@ -118,30 +118,8 @@ __device__ __forceinline__ int flag_read(uint32_t addr) {
   asm volatile("ld.relaxed.cta.shared::cta.b32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-// Bounded wait until the counter reaches `need`; gives up like mbar_wait.
-__device__ __forceinline__ bool count_wait(uint32_t addr, int need, volatile int* abort_flag, int* status,
-                                           long long limit_cycles) {
-  if (count_read(addr) >= need) return true;
-  const long long t0 = clock64();
-  for (uint32_t it = 1;; ++it) {
-    if (count_read(addr) >= need) return true;
-    __nanosleep(32);  // leave the issue slots to the warps that compute
-    if ((it & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (status && *reinterpret_cast<volatile int*>(status) != 0) {
-        *abort_flag = 1;
-        return false;
-      }
-      if (clock64() - t0 > limit_cycles) break;
-    }
-  }
-  *abort_flag = 1;
-  if (status) atomicExch(status, 1);
-  return false;
-}
-
-// The same wait for a thread on a latency-critical path that has a warp to itself: it polls without sleeping.
-// Returns the count it read (>= need), or -1 when it gave up.
+// Bounded wait until the counter reaches `need`, for a thread on a latency-critical path that has a warp to itself: it
+// polls without sleeping.  Returns the count it read (>= need), or -1 when it gave up (like mbar_wait).
 __device__ __forceinline__ int count_spin_wait(uint32_t addr, int need, volatile int* abort_flag, int* status,
                                                long long limit_cycles = kWaitLimitCycles) {
   int v = count_read(addr);
@@ -189,7 +167,19 @@ struct PollGuard {
   }
 };
 
-// Named barriers: the calling warp (all lanes, converged) arrives, or arrives and waits; `threads` counts both kinds.
+// Named barriers (hardware, not in shared memory): what a softmax warpgroup tells an issuing warp.  While the tensor
+// cores stream their operands an access to shared memory takes 100 to 200 cycles, and so does either side of an
+// mbarrier; a named barrier does not.  It cannot give up, so every thread passes every one of them whatever happened:
+// after a failed wait the tiles are walked on without meaning (and a softmax warp then waits instead of only
+// arriving, so that it cannot arrive twice at one phase).
+enum {
+  NB_STORE = 1,    // [2] the 128 threads of a query tile in the epilogue
+  NB_MERGE = 3,    // the 256 softmax threads
+  NB_S_FREE = 4,   // [2] the softmax of query tile (stream) x has read its scores: the S buffer may be written again
+  NB_P_EARLY = 6,  // [2] the first 96 columns of P are in TMEM
+  NB_P_FULL = 8,   // [2]
+};
+// The calling warp (all lanes, converged) arrives, or arrives and waits; `threads` counts both kinds.
 __device__ __forceinline__ void named_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
 }

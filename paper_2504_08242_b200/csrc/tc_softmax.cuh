@@ -1,14 +1,12 @@
-// The online-softmax steps of the tcgen05 attention kernels, three forms of the same arithmetic -- P = exp2(s c - m)
-// with fp32-pair instructions, written to TMEM as bf16 pairs (P column k holds keys 2k and 2k + 1; over S in two of the
-// forms, where the writes stay behind the reads), a lazy reference maximum m that only moves when the tile's maximum outgrew it by more
-// than 2^8 (then the row sum and the accumulator O are scaled by exp2(m_old - m_new); with well-behaved scores that
-// happens in a row's first tile and almost never again):
-//   softmax_tile_step : a thread per row, the row's 128 scores walked once in four chunks of 32 columns with the next
-//                       chunk in flight (about 160 registers; the branch kernel)
+// The online-softmax steps of the tcgen05 attention kernels, two forms of the same arithmetic -- P = exp2(s c - m)
+// with fp32-pair instructions, written to TMEM as bf16 pairs (P column k holds keys 2k and 2k + 1), a lazy reference
+// maximum m that only moves when the tile's maximum outgrew it by more than 2^8 (then the row sum and the accumulator O
+// are scaled by exp2(m_old - m_new); with well-behaved scores that happens in a row's first tile and almost never again):
 //   softmax_tile_row  : a thread per row holding the whole row (about 200 registers), S given back as soon as it is
-//                       read, P in columns of its own and released in two parts (the two-tile prefill kernel)
-//   frag_*            : 16 rows per warp in the 16x256b fragment layout, in pieces that a kernel interleaves across
-//                       consecutive tiles (the one-tile prefill kernel)
+//                       read, P in columns of its own and released in two parts (the two-tile prefill kernel, the
+//                       branch kernel)
+//   frag_*            : 16 rows per warp in the 16x256b fragment layout, P written over S, in pieces that a kernel
+//                       interleaves across consecutive tiles (the one-tile prefill kernel)
 #pragma once
 #include "tc_common.cuh"
 
@@ -26,124 +24,7 @@ struct ColumnBits {  // bit (col & 31) of w[col >> 5] set: visible
   __device__ __forceinline__ bool operator()(int col) const { return (w[col >> 5] >> (col & 31)) & 1u; }
 };
 
-__device__ __forceinline__ uint32_t scale_bf16_pair(uint32_t pair, float a) {
-  const float lo = __uint_as_float(pair << 16), hi = __uint_as_float(pair & 0xffff0000u);
-  return pack_bf16(lo * a, hi * a);
-}
-
-// tS / tO: TMEM addresses (lane base included) of the row's 128 scores and of its 128 accumulator columns.
-// j: number of tiles this stream has processed before (0: O holds nothing yet).
-// masked: warp-uniform; when false every column is visible and `allow` is not consulted.
-// PARTIAL: the stream may meet rows that see none of a tile (their reference maximum stays -inf and P is 0);
-// otherwise every row sees column 0 of its first tile.
-// wait_o(): waits until O(j-1) is complete (called exactly once when j > 0); returns false if the wait gave up,
-// and then so does this function.  On return P is complete in TMEM (tcgen05.wait::st done); the caller fences
-// and signals the MMA issuer.
-template <bool PARTIAL, class Allow, class WaitO>
-__device__ __forceinline__ bool softmax_tile_step(uint32_t tS, uint32_t tO, int j, bool masked, const Allow& allow,
-                                                  float c, float& m_ref, float& l, WaitO&& wait_o) {
-  const uint64_t c2 = pack2(c, c);
-  uint64_t lacc[4];  // this tile's row sum, four chains
-#pragma unroll
-  for (int k = 0; k < 4; ++k) lacc[k] = pack2(0.f, 0.f);
-  float alpha_total = 1.f;  // what the sum and the accumulator of the tiles before this one must be scaled by
-  bool moved = false;       // warp-uniform: some row's reference moved during this tile
-  uint32_t sb[2][32];
-  tmem_ld32(tS, sb[0]);
-#pragma unroll
-  for (int q4 = 0; q4 < 4; ++q4) {
-    tc_wait_ld();
-    if (q4 < 3) tmem_ld32(tS + (q4 + 1) * 32, sb[(q4 + 1) & 1]);
-    uint32_t(&sv)[32] = sb[q4 & 1];
-    if (masked) {
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (!allow(q4 * 32 + i)) sv[i] = 0xff800000u;  // -inf
-    }
-    // ---- chunk maximum (eight chains of 3-input max)
-    float a[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      a[k] = fmax3(__uint_as_float(sv[4 * k]), __uint_as_float(sv[4 * k + 1]), __uint_as_float(sv[4 * k + 2]));
-    const float mx = fmax3(fmax3(fmax3(a[0], a[1], a[2]), fmax3(a[3], a[4], a[5]), fmaxf(a[6], a[7])),
-                           fmax3(__uint_as_float(sv[3]), __uint_as_float(sv[7]), __uint_as_float(sv[11])),
-                           fmax3(fmax3(__uint_as_float(sv[15]), __uint_as_float(sv[19]), __uint_as_float(sv[23])),
-                                 __uint_as_float(sv[27]), __uint_as_float(sv[31])));
-    const float mxs = mx * c;
-    // lazy reference: it only moves when the maximum outgrew it by 2^8 (a row that has seen nothing keeps -inf,
-    // and its first visible score moves it because -inf + 8 is still -inf)
-    const bool grow = mxs > m_ref + TC_RESCALE_THRESHOLD;
-    if (__any_sync(0xffffffffu, grow)) {
-      const float alpha = grow ? fast_exp2(m_ref - mxs) : 1.f;
-      const uint64_t al2 = pack2(alpha, alpha);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) lacc[k] = mul2(lacc[k], al2);
-      if (q4 > 0) {  // the P chunks of this tile written so far were relative to the old reference
-        tc_wait_st();
-#pragma unroll
-        for (int qq = 0; qq < 3; ++qq) {
-          if (qq >= q4) break;
-          uint32_t pk[16];
-          tmem_ld16(tS + qq * 16, pk);
-          tc_wait_ld();  // (also completes the load of the next chunk, which is consumed later anyway)
-#pragma unroll
-          for (int i = 0; i < 16; ++i) pk[i] = scale_bf16_pair(pk[i], alpha);
-          tmem_st16(tS + qq * 16, pk);
-        }
-      }
-      alpha_total *= alpha;
-      moved = true;
-      if (grow) m_ref = mxs;
-    }
-    // ---- P
-    const float nm = (PARTIAL && m_ref == -INFINITY) ? 0.f : -m_ref;
-    const uint64_t nm2 = pack2(nm, nm);
-    uint32_t pk[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const uint64_t x = fma2(pack2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), c2, nm2);
-      float x0, x1;
-      unpack2(x, x0, x1);
-      const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-      lacc[i & 3] = add2(lacc[i & 3], pack2(p0, p1));
-      pk[i] = pack_bf16(p0, p1);
-    }
-    tmem_st16(tS + q4 * 16, pk);
-  }
-  float l_tile;
-  {
-    float a0, a1, b0, b1;
-    unpack2(add2(lacc[0], lacc[1]), a0, a1);
-    unpack2(add2(lacc[2], lacc[3]), b0, b1);
-    l_tile = (a0 + a1) + (b0 + b1);
-  }
-  bool o_waited = false;
-  if (moved) {
-    l *= alpha_total;
-    if (j > 0) {  // O(j-1) must be complete before it is rescaled
-      if (!wait_o()) return false;
-      o_waited = true;
-      tc_fence_after();
-#pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
-        uint32_t o[32];
-        tmem_ld32(tO + q4 * 32, o);
-        tc_wait_ld();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha_total);
-        tmem_st32(tO + q4 * 32, o);
-      }
-    }
-  }
-  l += l_tile;
-  tc_wait_st();
-  // every phase of the O-complete barrier is waited on exactly once, in order, so a parity never aliases;
-  // PV(j) queues behind PV(j-1) in the tensor pipe anyway, so this costs no overlap
-  if (j > 0 && !o_waited && !wait_o()) return false;
-  return true;
-}
-
-// The same step with the whole score row in registers (needs about 200 registers per thread) and P in columns of its
+// A thread per row, the whole score row in registers (needs about 200 registers per thread) and P in columns of its
 // own (tP), so that the S buffer is free as soon as the scores have been read: loaded() runs then, and the caller
 // passes the buffer on to the MMA issuer before anything is computed.  At most one move of the reference per tile
 // (decided before any P is written, so no P chunk is ever corrected); P in four chunks of 32 columns.  After the third
@@ -152,8 +33,14 @@ __device__ __forceinline__ bool softmax_tile_step(uint32_t tS, uint32_t tO, int 
 // previous P overwritten, O += P V of the stream's previous tile must be complete: test_o() tests that without
 // waiting, under the latency of the score load (it nearly always is), and wait_o() waits otherwise (j > 0 only).
 // On return P is complete in TMEM; the caller fences and signals the second half.
-template <bool PARTIAL, class Allow, class TestO, class WaitO, class Loaded, class Release>
-__device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint32_t tO, int j, bool masked,
+// tS / tP / tO: TMEM addresses (lane base included) of the row's 128 scores, of P and of its D accumulator columns.
+// j: number of tiles this stream has processed before (0: O holds nothing yet).
+// chunks: P is wanted for the first `chunks` blocks of 32 columns only; masked: warp-uniform, when false every column
+// is visible and `allow` is not consulted.
+// PARTIAL: the stream may meet rows that see none of a tile (their reference maximum stays -inf and P is 0);
+// otherwise every row sees column 0 of its first tile.
+template <bool PARTIAL, int D, class Allow, class TestO, class WaitO, class Loaded, class Release>
+__device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint32_t tO, int j, int chunks, bool masked,
                                                  const Allow& allow, float c, float& m_ref, float& l, TestO&& test_o,
                                                  WaitO&& wait_o, Loaded&& loaded, Release&& release_early) {
   uint32_t sv[128];
@@ -195,7 +82,7 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
     if (grow) m_ref = mxs;
     if (j > 0) {
 #pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
+      for (int q4 = 0; q4 < D / 32; ++q4) {
         uint32_t o[32];
         tmem_ld32(tO + q4 * 32, o);
         tc_wait_ld();
@@ -213,18 +100,20 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
   for (int k = 0; k < 4; ++k) lacc[k] = pack2(0.f, 0.f);
 #pragma unroll
   for (int q4 = 0; q4 < 4; ++q4) {
-    uint32_t pk[16];
+    if (q4 < chunks) {
+      uint32_t pk[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const uint64_t x =
-          fma2(pack2(__uint_as_float(sv[q4 * 32 + 2 * i]), __uint_as_float(sv[q4 * 32 + 2 * i + 1])), c2, nm2);
-      float x0, x1;
-      unpack2(x, x0, x1);
-      const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-      lacc[i & 3] = add2(lacc[i & 3], pack2(p0, p1));
-      pk[i] = pack_bf16(p0, p1);
+      for (int i = 0; i < 16; ++i) {
+        const uint64_t x =
+            fma2(pack2(__uint_as_float(sv[q4 * 32 + 2 * i]), __uint_as_float(sv[q4 * 32 + 2 * i + 1])), c2, nm2);
+        float x0, x1;
+        unpack2(x, x0, x1);
+        const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+        lacc[i & 3] = add2(lacc[i & 3], pack2(p0, p1));
+        pk[i] = pack_bf16(p0, p1);
+      }
+      tmem_st16(tP + q4 * 16, pk);
     }
-    tmem_st16(tP + q4 * 16, pk);
     if (q4 == 2) {
       tc_wait_st();
       release_early();

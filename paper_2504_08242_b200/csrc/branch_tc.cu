@@ -464,40 +464,35 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       // the tensor cores still compute the tile's scores
       const BtTile e = tile_at(2 * j + x, cursor);
       const int key0 = e.tile * BT_BN;
-      ColumnBits allow;
-      auto first_columns = [&](int cnt) {
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const int k = cnt - 32 * w;
-          allow.w[w] = k >= 32 ? 0xffffffffu : (k <= 0 ? 0u : (1u << k) - 1u);
+      ColumnBits allow = {0u, 0u, 0u, 0u};
+      bool warp_sees = (warp & 3) * 32 < rows_here, masked = false;  // a whole prefix tile is seen by every row there is
+      if (e.seg != BT_PREFIX || e.valid < BT_BN) {
+        // by 32-column words: the first `cnt` columns, and the block's rows by the mask from column `col` on (which may
+        // lie outside the tile)
+        auto word = [&](int w, int cnt, int col) {
+          const int k = cnt - 32 * w, c0 = col - 32 * w;
+          const uint32_t before = k >= 32 ? 0xffffffffu : (k <= 0 ? 0u : (1u << k) - 1u);
+          const uint32_t block = c0 >= 32 ? 0u : (c0 >= 0 ? tm << c0 : (c0 > -32 ? tm >> (-c0) : 0u));
+          return before | block;
+        };
+        // shared prefix: up to its end; the step's block: the rows of this row's branch; the row's own branch: the rows
+        // before the block, then (without the fused write) the block; another branch's suffix: nothing
+        constexpr int NONE = 0x100000;
+        int cnt = 0, col = NONE;
+        if (e.seg == BT_PREFIX) {
+          cnt = e.valid;
+        } else if (e.seg == BT_NEW) {
+          col = rj * n;
+        } else if (e.seg == rj) {
+          cnt = len_s[rj] - n - key0;
+          col = fused ? NONE : cnt;
         }
-      };
-      auto add_block = [&](int col) {  // the block's rows by the mask, from column `col` (which may lie outside the tile) on
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const int k = col - 32 * w;
-          allow.w[w] |= k >= 32 ? 0u : (k >= 0 ? tm << k : (k > -32 ? tm >> (-k) : 0u));
-        }
-      };
-      bool full = true;  // (also for a row beyond the tile's rows, which sees nothing and whose scores nobody uses)
-      if (e.seg == BT_PREFIX && row_valid) {  // shared prefix: up to its end
-        first_columns(e.valid);
-        full = e.valid == BT_BN;
-      } else if (e.seg == BT_NEW && row_valid) {  // the step's block of every branch of the tile
-        first_columns(0);
-        add_block(rj * n);
-        full = false;
-      } else if (e.seg >= 0 && e.seg == rj) {  // the row's own branch: rows before the block, then the block by the mask
-        const int hist = len_s[rj] - n - key0;  // column of the block's first row
-        first_columns(hist);
-        if (!fused) add_block(hist);
-        full = hist >= BT_BN;
-      } else {  // another branch's suffix
-        first_columns(0);
-        full = !row_valid;
+        if (!row_valid) cnt = 0, col = NONE;
+        allow = ColumnBits{word(0, cnt, col), word(1, cnt, col), word(2, cnt, col), word(3, cnt, col)};
+        warp_sees = __any_sync(0xffffffffu, (allow.w0 | allow.w1 | allow.w2 | allow.w3) != 0u);
+        // (a row beyond the tile's rows sees nothing and nobody uses its scores)
+        masked = !__all_sync(0xffffffffu, !row_valid || (allow.w0 & allow.w1 & allow.w2 & allow.w3) == 0xffffffffu);
       }
-      const bool warp_sees = __any_sync(0xffffffffu, (allow.w[0] | allow.w[1] | allow.w[2] | allow.w[3]) != 0u);
-      const bool masked = !__all_sync(0xffffffffu, full);
       // (ok is the same in all lanes of a warp: the barriers and the tcgen05 operations are warp-collective)
       ok = __all_sync(0xffffffffu, ok && mbar_spin_wait(bar(BT_S_FULL + x), j & 1, abort_flag, p.status, wl));
       tc_fence_after();
@@ -517,7 +512,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         uint32_t z[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) z[i] = 0u;
-#pragma unroll
+#pragma unroll 1
         for (int q4 = 0; q4 < 4; ++q4) tmem_st16(tP + q4 * 16, z);
         tc_wait_st();
         release_early();

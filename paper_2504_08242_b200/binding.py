@@ -124,13 +124,13 @@ lib = _load()
 
 
 def _ptr(t):
-    return None if t is None else c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    if stream is None:  # torch's current stream of the current device, without the Python object (3 us) around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def cache_desc(k: torch.Tensor, v: torch.Tensor) -> jupiter_kv_cache:
@@ -164,7 +164,7 @@ class Context:
             pass
 
     def _check(self, st: int):
-        if st != OK:
+        if st:
             detail = lib.jupiter_last_cuda_error(self._h).decode() if st == ERR_CUDA else ""
             raise JupiterError(st, detail)
 

@@ -158,9 +158,10 @@ jupiter_status jupiter_chunk_prefill_attn(jupiter_ctx* ctx, const void* q, const
  *   jupiter_chunk_prefill_attn(ctx, q, cache, q_heads, q_len, pos, scale, out, lse, stream):
  * k_new / v_new ([batch][q_len][kv_heads][D] bf16, dense, device) are copied bit-exactly into cache
  * rows [pos, pos+q_len) of every (sequence, head) and nothing else in the cache is written; row i
- * of head h attends cache rows 0..pos-1 and the chunk's own rows 0..i.  With head_dim 128 and
- * scale > 0 this is one kernel launch (the attention reads the chunk's K/V from k_new / v_new, so
- * no thread waits for the copy); otherwise it enqueues the two kernels of the separate calls.
+ * of head h attends cache rows 0..pos-1 and the chunk's own rows 0..i.  With scale > 0 and
+ * head_dim 128, or head_dim 64 and more than 64 rows, this is one kernel launch (the attention reads
+ * the chunk's K/V from k_new / v_new, so no thread waits for the copy); otherwise it enqueues the two
+ * kernels of the separate calls.
  * Precondition: cache rows [0, pos) are valid.  Arguments and errors as for the two calls. */
 jupiter_status jupiter_chunk_prefill_append_attn(jupiter_ctx* ctx, const void* q, const void* k_new,
                                                  const void* v_new, const jupiter_kv_cache* cache,

@@ -209,7 +209,7 @@ jupiter_status jupiter_chunk_prefill_attn(jupiter_ctx* ctx, const void* q, const
   if (jup::prefill_tc_supported(c, scale))
     e = jup::launch_prefill_tc(static_cast<const bf16*>(q), c, nullptr, 0, q_heads, q_len, pos, scale, out, lse,
                                ctx->d_status, ctx->workspace, ctx->workspace_bytes, static_cast<cudaStream_t>(stream), li);
-  else  // head_dim 64, or a non-positive scale: the general mma.sync kernel
+  else  // a non-positive scale: the general mma.sync kernel
     e = jup::launch_prefill_mma(static_cast<const bf16*>(q), c, q_heads, q_len, pos, scale, out, lse,
                                 static_cast<cudaStream_t>(stream), li);
   ctx->launches += li.launches;
@@ -231,14 +231,18 @@ jupiter_status jupiter_chunk_prefill_append_attn(jupiter_ctx* ctx, const void* q
   jup::LaunchInfo li{ctx->sm_count, 0};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  if (jup::prefill_tc_supported(c, scale)) {
+  const bool tc = jup::prefill_tc_supported(c, scale);
+  if (tc && (c.head_dim == 128 || q_len > 64)) {
     e = jup::launch_prefill_tc_fused(static_cast<const bf16*>(q), c, static_cast<const bf16*>(k_new),
                                      static_cast<const bf16*>(v_new), q_heads, q_len, pos, scale, out, lse,
                                      ctx->d_status, ctx->workspace, ctx->workspace_bytes, st, li);
-  } else {  // head_dim 64, or a non-positive scale: the append kernel, then the general mma.sync kernel
+  } else {  // the append kernel, then the attention on the cache
     e = jup::launch_kv_append(c, static_cast<const bf16*>(k_new), static_cast<const bf16*>(v_new), q_len, pos, nullptr,
                               st, li);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && tc)
+      e = jup::launch_prefill_tc(static_cast<const bf16*>(q), c, nullptr, 0, q_heads, q_len, pos, scale, out, lse,
+                                 ctx->d_status, ctx->workspace, ctx->workspace_bytes, st, li);
+    else if (e == cudaSuccess)
       e = jup::launch_prefill_mma(static_cast<const bf16*>(q), c, q_heads, q_len, pos, scale, out, lse, st, li);
   }
   ctx->launches += li.launches;
@@ -265,7 +269,7 @@ jupiter_status jupiter_branch_prefill_attn(jupiter_ctx* ctx, const void* q, cons
   if (!jup::scale_ok(scale)) return JUPITER_ERR_INVALID_ARG;
   if (pos < 0 || static_cast<int64_t>(pos) + q_len > c.capacity) return JUPITER_ERR_OUT_OF_RANGE;
   if (!aligned16(q) || !aligned16(out)) return JUPITER_ERR_ALIGNMENT;
-  if (!jup::prefill_tc_supported(c, scale)) return JUPITER_ERR_UNSUPPORTED;  // head_dim 128 and scale > 0 only
+  if (c.head_dim != 128 || !jup::prefill_tc_supported(c, scale)) return JUPITER_ERR_UNSUPPORTED;  // head_dim 128 and scale > 0 only
   DeviceGuard guard(ctx->device);
   jup::LaunchInfo li{ctx->sm_count, 0};
   cudaError_t e = jup::launch_prefill_tc(static_cast<const bf16*>(q), c, prefix_len > 0 ? &pfx : nullptr, prefix_len,

@@ -61,7 +61,7 @@ cudaError_t launch_kv_append(const CacheView& c, const bf16* k_new, const bf16* 
 cudaError_t launch_prefill_mma(const bf16* q, const CacheView& c, int q_heads, int q_len, int pos, float scale,
                                float* out, float* lse, cudaStream_t st, LaunchInfo& li);
 
-// tcgen05 / TMEM prefill kernel (head_dim 128, positive finite scale, TMA-encodable strides).
+// tcgen05 / TMEM prefill kernels (positive finite scale, TMA-encodable strides).
 bool prefill_tc_supported(const CacheView& c, float scale);
 // prefix (nullable) / prefix_len: a shared cache (batch 1) whose rows [0, prefix_len) every query row attends
 // before the sequence's own rows.
@@ -70,7 +70,7 @@ cudaError_t launch_prefill_tc(const bf16* q, const CacheView& c, const CacheView
                               int q_heads, int q_len, int pos, float scale, float* out, float* lse, int* status,
                               void* workspace, size_t workspace_bytes, cudaStream_t st, LaunchInfo& li);
 
-// Fused KVCache write + attention: the chunk's K/V (k_new / v_new, [batch][q_len][kv_heads][128] token-major) go into
+// Fused KVCache write + attention: the chunk's K/V (k_new / v_new, [batch][q_len][kv_heads][D] token-major) go into
 // cache rows [pos, pos + q_len) and the chunk attends cache rows [0, pos) plus itself, in one launch.
 cudaError_t launch_prefill_tc_fused(const bf16* q, const CacheView& c, const bf16* k_new, const bf16* v_new,
                                     int q_heads, int q_len, int pos, float scale, float* out, float* lse, int* status,

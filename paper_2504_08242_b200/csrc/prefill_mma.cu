@@ -1,6 +1,7 @@
 // Chunked-prefill attention on mma.sync (paper Sec. IV-A, Fig. 5(b)): the chunk's
-// rows at positions pos..pos+n-1 attend to cache rows 0..pos+i.  General-shape
-// path: any head_dim in {64,128}, any pos / q_len.  One CTA = 64 chunk rows of
+// rows at positions pos..pos+n-1 attend to cache rows 0..pos+i.  Takes what the
+// tcgen05 kernels do not: non-positive scales (they take the row maximum before scaling), strides a tensor map cannot
+// carry.  Any head_dim in {64,128}, any pos / q_len.  One CTA = 64 chunk rows of
 // one (sequence, query head); heaviest row tiles are scheduled first.
 #include "attn_mma.cuh"
 #include "host_checks.h"

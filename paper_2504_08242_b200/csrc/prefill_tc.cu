@@ -1,5 +1,5 @@
 // Chunked-prefill attention on the 5th-generation tensor cores (paper Sec. IV-A, Fig. 5(b)):
-// chunk rows at positions pos..pos+n-1 attend causally to cache rows 0..pos+i.  head_dim 128.
+// chunk rows at positions pos..pos+n-1 attend causally to cache rows 0..pos+i.
 //
 // Two kernels, chosen by the size of the grid (see launch_tc):
 //  - prefill_tc_kernel (this file): one CTA owns TWO query tiles of 128 rows of one (sequence, query head) and walks
@@ -20,6 +20,10 @@
 //    tiles).  For grids that cannot fill the SMs a cluster of 4 CTAs shares the pair of query tiles and splits the KV
 //    walk (template parameter CL).
 //  - prefill_frag_kernel (prefill_tc_frag.cuh): one query tile per CTA, both warpgroups on it.
+// head_dim 64 runs the same kernels with half as many operand slices and accumulator columns.  Measured against the
+// mma.sync kernel that took it before (us a call, append included, 32 / 8 heads): 16 rows at position 0 4.9 : 6.6, 448
+// rows at position 0 8.1 : 14.8, at position 2048 23 : 60, four prompts at once 65 : 171 -- never slower, so that kernel
+// is left with the non-positive scales.
 // All mbarrier waits are bounded; on expiry the CTA sets the status word, drains its own copies and MMAs, frees
 // TMEM and returns.
 #include "host_checks.h"
@@ -32,11 +36,9 @@
 
 namespace jup {
 
-constexpr int TC_D = 128;
 constexpr int TC_BM = 128;              // query rows per tile
 constexpr int TC_BN = 128;              // keys per KV tile
-constexpr int TC_TILE_BYTES = 32768;    // 128 x 128 bf16
-constexpr int TC_PANEL_BYTES = 16384;   // 128 rows x 64 elements
+constexpr int TC_PANEL_BYTES = 16384;   // 128 rows x 64 elements of bf16: a Q, K or V tile is D / 64 of them
 constexpr int TC_CLUSTER_MIN_TILES = 18;     // shortest KV walk (in tiles) that a cluster of 4 CTAs shares
 
 struct TcParams {
@@ -56,11 +58,15 @@ struct TcParams {
   int fused_write;
   int copy_pos;
 };
-constexpr int TC_PART_FLOATS = 2 * TC_BM * TC_D;  // one CTA's partial accumulators (both query tiles)
+template <int D>
+constexpr int TC_PART_FLOATS = 2 * TC_BM * D;  // one CTA's partial accumulators (both query tiles)
 constexpr int TC_ML_FLOATS = 2 * TC_BM * 2;       // one CTA's (m, l) pairs
 
 constexpr int TC_NQ = 2;  // query tiles per CTA
+template <int D>
 struct TcCfg {
+  static constexpr int TILE_BYTES = TC_BM * D * 2;
+  static constexpr int PANELS = D / 64;
   static constexpr int KV_STAGES = 2;
   static constexpr int SOFTMAX_WARPS = 4 * TC_NQ;
   static constexpr int LOADER_WARP = SOFTMAX_WARPS;
@@ -74,9 +80,9 @@ struct TcCfg {
   static constexpr int O_COL0 = 0, S_COL = 256, P_COL0 = 384;
   // shared memory: [Q tiles][K ring][V ring][barriers]
   static constexpr int SMEM_Q = 0;
-  static constexpr int SMEM_K = TC_NQ * TC_TILE_BYTES;
-  static constexpr int SMEM_V = SMEM_K + KV_STAGES * TC_TILE_BYTES;
-  static constexpr int SMEM_BAR = SMEM_V + KV_STAGES * TC_TILE_BYTES;
+  static constexpr int SMEM_K = TC_NQ * TILE_BYTES;
+  static constexpr int SMEM_V = SMEM_K + KV_STAGES * TILE_BYTES;
+  static constexpr int SMEM_BAR = SMEM_V + KV_STAGES * TILE_BYTES;
   static constexpr int SMEM_BYTES = SMEM_BAR + 256 + 1024;  // + slack for 1024-byte alignment
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
 };
@@ -100,13 +106,14 @@ constexpr int NQ = TC_NQ;
 // r, r + CL, r + 2 CL, ... and the partial (O, m, l) are exchanged through global scratch (L2) around one
 // cluster barrier: distributed shared memory moved them at about 20 GB/s per SM when measured, L2 is
 // several times faster.  CTA r then finishes the output columns [128 r / CL, 128 (r + 1) / CL).
-template <int CL>
-__global__ void __launch_bounds__(TcCfg::THREADS, 1)
+template <int D, int CL>
+__global__ void __launch_bounds__(TcCfg<D>::THREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
                   const __grid_constant__ CUtensorMap tm_pv, const __grid_constant__ CUtensorMap tm_o,
                   const __grid_constant__ CUtensorMap tm_ck, const __grid_constant__ CUtensorMap tm_cv, TcParams p) {
-  using Cfg = TcCfg;
+  using Cfg = TcCfg<D>;
+  constexpr int TILE_BYTES = Cfg::TILE_BYTES;
   constexpr int KV_STAGES = Cfg::KV_STAGES;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -193,9 +200,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       for (int x = 0; x < NQ; ++x) {
         if (T[x] == 0) continue;
         const int r0 = (qblk * NQ + x) * TC_BM;
-        mbar_expect_tx(bar(BAR_Q_FULL + x), TC_TILE_BYTES);
-        tma_load_4d(sQ + x * TC_TILE_BYTES, &tm_q, bar(BAR_Q_FULL + x), 0, h, r0, b);
-        tma_load_4d(sQ + x * TC_TILE_BYTES + TC_PANEL_BYTES, &tm_q, bar(BAR_Q_FULL + x), 64, h, r0, b);
+        mbar_expect_tx(bar(BAR_Q_FULL + x), TILE_BYTES);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c)
+          tma_load_4d(sQ + x * TILE_BYTES + c * TC_PANEL_BYTES, &tm_q, bar(BAR_Q_FULL + x), c * 64, h, r0, b);
       }
       int issued = 0;
       bool ok = true;
@@ -212,10 +220,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         ok = ok && mbar_wait(bar(BAR_V_FULL + s), u & 1, abort_flag, p.status);
         if (!ok) return;
         const int row = p.copy_pos + t * TC_BN;  // rows beyond copy_pos + q_len are clipped by the tensor maps
-        tma_store_4d(&tm_ck, sK + s * TC_TILE_BYTES, 0, row, hk, b);
-        tma_store_4d(&tm_ck, sK + s * TC_TILE_BYTES + TC_PANEL_BYTES, 64, row, hk, b);
-        tma_store_4d(&tm_cv, sV + s * TC_TILE_BYTES, 0, row, hk, b);
-        tma_store_4d(&tm_cv, sV + s * TC_TILE_BYTES + TC_PANEL_BYTES, 64, row, hk, b);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c) {
+          tma_store_4d(&tm_ck, sK + s * TILE_BYTES + c * TC_PANEL_BYTES, c * 64, row, hk, b);
+          tma_store_4d(&tm_cv, sV + s * TILE_BYTES + c * TC_PANEL_BYTES, c * 64, row, hk, b);
+        }
         tma_store_commit();
         tma_store_wait_read();
       };
@@ -225,21 +234,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         if (!ok) break;
         if (u > 0) ok = mbar_wait(bar(BAR_K_EMPTY + s), (u - 1) & 1, abort_flag, p.status);
         if (!ok) break;
-        mbar_expect_tx(bar(BAR_K_FULL + s), TC_TILE_BYTES);
+        mbar_expect_tx(bar(BAR_K_FULL + s), TILE_BYTES);
         const int g = tile_of_seq(j);
         const CUtensorMap* mk = g < Tp ? &tm_pk : &tm_k;
         const int krow = (g < Tp ? g : g - Tp) * TC_BN, kb = (g < Tp && !p.prefix_batched) ? 0 : b;
-        tma_load_4d(sK + s * TC_TILE_BYTES, mk, bar(BAR_K_FULL + s), 0, krow, hk, kb);
-        tma_load_4d(sK + s * TC_TILE_BYTES + TC_PANEL_BYTES, mk, bar(BAR_K_FULL + s), 64, krow, hk, kb);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c)
+          tma_load_4d(sK + s * TILE_BYTES + c * TC_PANEL_BYTES, mk, bar(BAR_K_FULL + s), c * 64, krow, hk, kb);
         if (u > 0) ok = mbar_wait(bar(BAR_V_EMPTY + s), (u - 1) & 1, abort_flag, p.status);
         if (!ok) {
           issued = 2 * j + 1;
           break;
         }
-        mbar_expect_tx(bar(BAR_V_FULL + s), TC_TILE_BYTES);
+        mbar_expect_tx(bar(BAR_V_FULL + s), TILE_BYTES);
         const CUtensorMap* mv = g < Tp ? &tm_pv : &tm_v;
-        tma_load_4d(sV + s * TC_TILE_BYTES, mv, bar(BAR_V_FULL + s), 0, krow, hk, kb);
-        tma_load_4d(sV + s * TC_TILE_BYTES + TC_PANEL_BYTES, mv, bar(BAR_V_FULL + s), 64, krow, hk, kb);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c)
+          tma_load_4d(sV + s * TILE_BYTES + c * TC_PANEL_BYTES, mv, bar(BAR_V_FULL + s), c * 64, krow, hk, kb);
         issued = 2 * j + 2;
       }
       for (int j = max(0, Tall - KV_STAGES); j < Tall && ok; ++j) store_own_tile(j);
@@ -273,7 +284,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     int prev_x = -1;  // owner of the scores written last
     int turn = 0;
     for (int j = 0; j < Tall; ++j) {
-      const uint32_t k_lo = tc_desc_lo(sK + (j % KV_STAGES) * TC_TILE_BYTES, 16);
+      const uint32_t k_lo = tc_desc_lo(sK + (j % KV_STAGES) * TILE_BYTES, 16);
       if (lane == 0) ok = ok && mbar_wait(bar(BAR_K_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
@@ -284,9 +295,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         if (lane == 0 && ok) {
           flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
           tc_fence_after();
-          const uint32_t q_lo = tc_desc_lo(sQ + x * TC_TILE_BYTES, 16);
+          const uint32_t q_lo = tc_desc_lo(sQ + x * TILE_BYTES, 16);
 #pragma unroll
-          for (int ks = 0; ks < TC_D / 16; ++ks) {
+          for (int ks = 0; ks < D / 16; ++ks) {
             const uint32_t off = ((ks >> 2) * TC_PANEL_BYTES + (ks & 3) * 32) >> 4;
             tc_mma_ss_lo(s_col, q_lo + off, k_lo + off, idesc_qk, ks > 0);
           }
@@ -310,10 +321,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     // what everybody waits for: this thread stands back while a batch of scores is being issued.  (Looked at once per
     // batch: the shared-memory read takes longer than an MMA.)
     reg_dec<Cfg::REGS_OTHER>();
-    constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, TC_D, false, true);
+    constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, D, false, true);
     bool ok = true;
     for (int j = 0; j < Tall; ++j) {
-      const uint32_t v_lo = tc_desc_lo(sV + (j % KV_STAGES) * TC_TILE_BYTES, TC_PANEL_BYTES);
+      const uint32_t v_lo = tc_desc_lo(sV + (j % KV_STAGES) * TILE_BYTES, TC_PANEL_BYTES);
       if (lane == 0) ok = ok && mbar_wait(bar(BAR_V_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
@@ -373,7 +384,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       const int g = tile_of_seq(j);
       const int nvalid = g < Tp ? p.prefix_len - g * TC_BN : lim - (g - Tp) * TC_BN;
       const bool masked = __any_sync(0xffffffffu, nvalid < TC_BN);
-      softmax_tile_row<PARTIAL, TC_D>(
+      softmax_tile_row<PARTIAL, D>(
           tS, tP, tO, j, 4, masked, ColumnLimit{nvalid}, c, m_ref, l,
           [&] { return mbar_test_wait(bar(BAR_O_READY + x), (j - 1) & 1); },
           [&] { ok = ok && mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
@@ -395,18 +406,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       ok = ok && mbar_wait(bar(BAR_O_READY + x), (Tx - 1) & 1, abort_flag, p.status);
       tc_fence_after();
       // O / l goes out through shared memory (this tile's Q buffer, free now) and tiled stores: two rounds of
-      // two boxes of 128 rows x 32 columns; rows at or beyond q_len are clipped by the tensor map.
+      // D / 64 boxes of 128 rows x 32 columns; rows at or beyond q_len are clipped by the tensor map.
       const float inv = 1.f / l;
-      float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_Q + x * TC_TILE_BYTES);
-      const uint32_t stage_addr = sQ + x * TC_TILE_BYTES;
+      float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_Q + x * TILE_BYTES);
+      const uint32_t stage_addr = sQ + x * TILE_BYTES;
       const int tid_t = threadIdx.x & 127;
       const int tile_row0 = (qblk * NQ + x) * TC_BM;
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
 #pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2) {
+        for (int q2 = 0; q2 < Cfg::PANELS; ++q2) {
           uint32_t o[32];
-          tmem_ld32(tO + hh * 64 + q2 * 32, o);
+          tmem_ld32(tO + hh * (D / 2) + q2 * 32, o);
           tc_wait_ld();
           float v[32];
 #pragma unroll
@@ -417,8 +428,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         named_sync(NB_STORE + x, 128);
         if (tid_t == 0) {
           if (ok) {
-            tma_store_4d(&tm_o, stage_addr, hh * 64, h, tile_row0, b);
-            tma_store_4d(&tm_o, stage_addr + TC_BOX_FLOATS * 4, hh * 64 + 32, h, tile_row0, b);
+#pragma unroll
+            for (int c = 0; c < Cfg::PANELS; ++c)
+              tma_store_4d(&tm_o, stage_addr + c * TC_BOX_FLOATS * 4, hh * (D / 2) + c * 32, h, tile_row0, b);
             tma_store_commit();
           }
           tma_store_wait_read();  // the boxes are rewritten next / shared memory is released at the end of the kernel
@@ -442,20 +454,20 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    constexpr int W = TC_D / CL;  // output columns this CTA finishes
+    constexpr int W = D / CL;  // output columns this CTA finishes
     // Partial accumulators, unnormalised fp32: [column slice CL][query tile 2][row 128][W], the 16-byte chunks
     // of a row XOR-swizzled by the row (bank conflicts); staged in the K/V rings, copied as they are to the
     // cluster's scratch.  (m, l) per row: [query tile 2][row 128].
     float* part = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);
-    static_assert(TC_PART_FLOATS * 4 <= 2 * KV_STAGES * TC_TILE_BYTES, "partials fit in the K/V rings");
-    float* gpart = p.scratch + static_cast<size_t>(work) * CL * (TC_PART_FLOATS + TC_ML_FLOATS);
-    float* gml = gpart + CL * TC_PART_FLOATS;
+    static_assert(TC_PART_FLOATS<D> * 4 <= 2 * KV_STAGES * TILE_BYTES, "partials fit in the K/V rings");
+    float* gpart = p.scratch + static_cast<size_t>(work) * CL * (TC_PART_FLOATS<D> + TC_ML_FLOATS);
+    float* gml = gpart + CL * TC_PART_FLOATS<D>;
     if (warp < Cfg::SOFTMAX_WARPS) {
       const int x = warp >> 2, row_in_tile = (warp & 3) * 32 + lane;
       const uint32_t tO = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + Cfg::O_COL0 + x * 128;
       reinterpret_cast<float2*>(gml + crank * TC_ML_FLOATS)[x * TC_BM + row_in_tile] = make_float2(part_m, part_l);
 #pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
+      for (int q4 = 0; q4 < D / 32; ++q4) {
         uint32_t o[32];
         if (T[x] > 0) {  // warpgroup-uniform; a stream without tiles never wrote its accumulator
           tmem_ld32(tO + q4 * 32, o);
@@ -464,19 +476,20 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
           for (int i = 0; i < 32; ++i) o[i] = 0u;
         }
-        const int slice = (q4 * 32) / W, chunk0 = ((q4 * 32) % W) / 4;
-        float* dst = part + ((slice * 2 + x) * TC_BM + row_in_tile) * W;
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc)
-          *reinterpret_cast<float4*>(dst + (((chunk0 + cc) ^ (row_in_tile & 7)) << 2)) =
+        for (int cc = 0; cc < 8; ++cc) {
+          const int slice = (q4 * 32 + cc * 4) / W, chunk = ((q4 * 32 + cc * 4) % W) / 4;
+          *reinterpret_cast<float4*>(part + ((slice * 2 + x) * TC_BM + row_in_tile) * W +
+                                     ((chunk ^ (row_in_tile & (W / 4 - 1))) << 2)) =
               make_float4(__uint_as_float(o[4 * cc]), __uint_as_float(o[4 * cc + 1]), __uint_as_float(o[4 * cc + 2]),
                           __uint_as_float(o[4 * cc + 3]));
+        }
       }
       named_sync(NB_MERGE, 256);
       const float4* src = reinterpret_cast<const float4*>(part);
-      float4* dst = reinterpret_cast<float4*>(gpart + crank * TC_PART_FLOATS);
+      float4* dst = reinterpret_cast<float4*>(gpart + crank * TC_PART_FLOATS<D>);
 #pragma unroll 8
-      for (int i = 0; i < TC_PART_FLOATS / 4 / 256; ++i) dst[i * 256 + threadIdx.x] = src[i * 256 + threadIdx.x];
+      for (int i = 0; i < TC_PART_FLOATS<D> / 4 / 256; ++i) dst[i * 256 + threadIdx.x] = src[i * 256 + threadIdx.x];
       __threadfence();
     }
     cluster_sync_all();  // release / acquire over the cluster: the partials of every CTA are visible
@@ -526,10 +539,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
           for (int k = 0; k < BATCH; ++k) {
             const int r = row_of(it0 + k);
-            const int off = ((crank * 2 + x) * TC_BM + r) * W + ((chunk ^ (r & 7)) << 2);
+            const int off = ((crank * 2 + x) * TC_BM + r) * W + ((chunk ^ (r & (W / 4 - 1))) << 2);
 #pragma unroll
             for (int cr = 0; cr < CL; ++cr)
-              v[k][cr] = __ldcg(reinterpret_cast<const float4*>(gpart + cr * TC_PART_FLOATS + off));
+              v[k][cr] = __ldcg(reinterpret_cast<const float4*>(gpart + cr * TC_PART_FLOATS<D> + off));
           }
 #pragma unroll
           for (int k = 0; k < BATCH; ++k) {
@@ -544,7 +557,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             }
             const int row = (qblk * NQ + x) * TC_BM + row_of(it0 + k);
             if (cta_ok && row < p.q_len)
-              *reinterpret_cast<float4*>(p.out + ((static_cast<int64_t>(b) * p.q_len + row) * p.q_heads + h) * TC_D +
+              *reinterpret_cast<float4*>(p.out + ((static_cast<int64_t>(b) * p.q_len + row) * p.q_heads + h) * D +
                                          crank * W + chunk * 4) = acc;
           }
         }
@@ -569,55 +582,56 @@ namespace jup {
 
 // ---------------------------------------------------------------- host side
 
+template <int D>
 static cudaError_t launch_frag(int64_t ctas, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
                                const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
                                const CUtensorMap& tck, const CUtensorMap& tcv, const TcParams& p) {
   static PerDeviceOnce done;
   if (!done.done()) {
     cudaError_t e =
-        cudaFuncSetAttribute(prefill_frag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FragCfg::SMEM_BYTES);
+        cudaFuncSetAttribute(prefill_frag_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, FragCfg<D>::SMEM_BYTES);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(prefill_frag_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+      e = cudaFuncSetAttribute(prefill_frag_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     done.set();
   }
-  return launch_pdl_cluster(prefill_frag_kernel, dim3(static_cast<unsigned>(ctas)), dim3(FragCfg::THREADS),
-                            FragCfg::SMEM_BYTES, st, 1u, tq, tk, tv, tpk, tpv, tck, tcv, p);
+  return launch_pdl_cluster(prefill_frag_kernel<D>, dim3(static_cast<unsigned>(ctas)), dim3(FragCfg<D>::THREADS),
+                            FragCfg<D>::SMEM_BYTES, st, 1u, tq, tk, tv, tpk, tpv, tck, tcv, p);
 }
 
-template <int CL>
+template <int D, int CL>
 static cudaError_t launch_variant(int64_t ctas, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
                                   const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
                                   const CUtensorMap& to, const CUtensorMap& tck, const CUtensorMap& tcv,
                                   const TcParams& p) {
-  using Cfg = TcCfg;
+  using Cfg = TcCfg<D>;
   static PerDeviceOnce done;
   if (!done.done()) {
     cudaError_t e =
-        cudaFuncSetAttribute(prefill_tc_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+        cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(prefill_tc_kernel<CL>, cudaFuncAttributePreferredSharedMemoryCarveout,
+      e = cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     done.set();
   }
-  return launch_pdl_cluster(prefill_tc_kernel<CL>, dim3(static_cast<unsigned>(ctas * CL)),
+  return launch_pdl_cluster(prefill_tc_kernel<D, CL>, dim3(static_cast<unsigned>(ctas * CL)),
                             dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, static_cast<unsigned>(CL), tq, tk, tv, tpk, tpv, to, tck,
                             tcv, p);
 }
 
 // How many clusters of CL CTAs of the cluster-mode kernel can be resident at once (0 if the query fails).
-template <int CL>
+template <int D, int CL>
 static int max_resident_clusters() {
   static std::atomic<int> cache[64];  // per device: 0 = not asked yet, else answer + 1
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   const int cached = cache[dev].load(std::memory_order_acquire);
   if (cached > 0) return cached - 1;
-  using Cfg = TcCfg;
+  using Cfg = TcCfg<D>;
   int n = 0;
-  if (cudaFuncSetAttribute(prefill_tc_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            Cfg::SMEM_BYTES) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CL * 64);
@@ -631,7 +645,7 @@ static int max_resident_clusters() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, prefill_tc_kernel<CL>, &cfg) == cudaSuccess) n = got;
+    if (cudaOccupancyMaxActiveClusters(&got, prefill_tc_kernel<D, CL>, &cfg) == cudaSuccess) n = got;
     else (void)cudaGetLastError();
   } else {
     (void)cudaGetLastError();
@@ -641,48 +655,49 @@ static int max_resident_clusters() {
 }
 
 bool prefill_tc_supported(const CacheView& c, float scale) {
-  // head_dim 128, a positive finite scale, and strides a tensor map can carry (multiples of 16 bytes below 2^40;
+  // a positive finite scale, and strides a tensor map can carry (multiples of 16 bytes below 2^40;
   // the 16-byte rule is part of every cache descriptor already)
   auto encodable = [](int64_t elems) { return static_cast<uint64_t>(elems) * 2 < (1ull << 40); };
-  return c.head_dim == TC_D && scale > 0.f && scale < INFINITY && encode_fn() != nullptr && encodable(c.sr) &&
+  return scale > 0.f && scale < INFINITY && encode_fn() != nullptr && encodable(c.sr) &&
          encodable(c.sh) && encodable(c.sb);
 }
 
 // c: the attention's own segment (rows [0, pos + q_len) of every sequence); prefix (nullable): the segment in front
 // of it, shared by all sequences or one per sequence (prefix_batched); copy_dst (nullable): cache that receives the
 // own segment's rows at copy_pos (the own segment is then the chunk's token-major K/V).
+template <int D>
 static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView* prefix, int prefix_len,
                              bool prefix_batched, const CacheView* copy_dst, int copy_pos, int q_heads, int q_len,
                              int pos, float scale, float* out, float* lse, int* status, void* workspace,
                              size_t workspace_bytes, cudaStream_t st, LaunchInfo& li) {
   CUtensorMap tq, tk, tv, tpk, tpv, to, tck, tcv;
   if (!encode_fn()) return cudaErrorInvalidValue;
-  {  // out: [batch][q_len][q_heads][128] fp32, boxes of 128 rows x 32 columns
-    const uint64_t d[4] = {TC_D, static_cast<uint64_t>(q_heads), static_cast<uint64_t>(q_len),
+  {  // out: [batch][q_len][q_heads][D] fp32, boxes of 128 rows x 32 columns
+    const uint64_t d[4] = {D, static_cast<uint64_t>(q_heads), static_cast<uint64_t>(q_len),
                            static_cast<uint64_t>(c.batch)};
-    const uint64_t s[3] = {TC_D * 4ull, static_cast<uint64_t>(q_heads) * TC_D * 4ull,
-                           static_cast<uint64_t>(q_len) * q_heads * TC_D * 4ull};
+    const uint64_t s[3] = {D * 4ull, static_cast<uint64_t>(q_heads) * D * 4ull,
+                           static_cast<uint64_t>(q_len) * q_heads * D * 4ull};
     const uint32_t bx[4] = {32, 1, TC_BM, 1};
     if (!make_map_f32(&to, out, d, s, bx)) return cudaErrorInvalidValue;
   }
   const uint64_t rows_valid = static_cast<uint64_t>(pos) + q_len;  // rows above are dead: TMA zero-fills them
   {
-    const uint64_t d[4] = {TC_D, static_cast<uint64_t>(q_heads), static_cast<uint64_t>(q_len),
+    const uint64_t d[4] = {D, static_cast<uint64_t>(q_heads), static_cast<uint64_t>(q_len),
                            static_cast<uint64_t>(c.batch)};
-    const uint64_t s[3] = {TC_D * 2ull, static_cast<uint64_t>(q_heads) * TC_D * 2ull,
-                           static_cast<uint64_t>(q_len) * q_heads * TC_D * 2ull};
+    const uint64_t s[3] = {D * 2ull, static_cast<uint64_t>(q_heads) * D * 2ull,
+                           static_cast<uint64_t>(q_len) * q_heads * D * 2ull};
     const uint32_t bx[4] = {64, 1, TC_BM, 1};
     if (!make_map_bf16(&tq, q, d, s, bx)) return cudaErrorInvalidValue;
   }
   {
-    const uint64_t d[4] = {TC_D, rows_valid, static_cast<uint64_t>(c.kv_heads), static_cast<uint64_t>(c.batch)};
+    const uint64_t d[4] = {D, rows_valid, static_cast<uint64_t>(c.kv_heads), static_cast<uint64_t>(c.batch)};
     const uint64_t s[3] = {static_cast<uint64_t>(c.sr) * 2, static_cast<uint64_t>(c.sh) * 2,
                            static_cast<uint64_t>(c.sb) * 2};
     const uint32_t bx[4] = {64, TC_BN, 1, 1};
     if (!make_map_bf16(&tk, c.k, d, s, bx) || !make_map_bf16(&tv, c.v, d, s, bx)) return cudaErrorInvalidValue;
   }
   if (prefix && prefix_len > 0) {  // rows at or beyond prefix_len are zero-filled by TMA
-    const uint64_t d[4] = {TC_D, static_cast<uint64_t>(prefix_len), static_cast<uint64_t>(prefix->kv_heads),
+    const uint64_t d[4] = {D, static_cast<uint64_t>(prefix_len), static_cast<uint64_t>(prefix->kv_heads),
                            static_cast<uint64_t>(prefix_batched ? prefix->batch : 1)};
     const uint64_t s[3] = {static_cast<uint64_t>(prefix->sr) * 2, static_cast<uint64_t>(prefix->sh) * 2,
                            static_cast<uint64_t>(prefix->sb) * 2};
@@ -707,7 +722,7 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   tck = tk;  // never dereferenced without a fused write
   tcv = tv;
   if (copy_dst) {  // destination rows [0, copy_pos + q_len) of every sequence's cache; stores beyond are clipped
-    const uint64_t d[4] = {TC_D, static_cast<uint64_t>(copy_pos) + q_len, static_cast<uint64_t>(copy_dst->kv_heads),
+    const uint64_t d[4] = {D, static_cast<uint64_t>(copy_pos) + q_len, static_cast<uint64_t>(copy_dst->kv_heads),
                            static_cast<uint64_t>(copy_dst->batch)};
     const uint64_t s[3] = {static_cast<uint64_t>(copy_dst->sr) * 2, static_cast<uint64_t>(copy_dst->sh) * 2,
                            static_cast<uint64_t>(copy_dst->sb) * 2};
@@ -729,23 +744,23 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   if (ctas2 < li.sm_count && q_len > TC_BM) {
     // scratch for the partials behind the counter block at the head of the workspace
     auto fits = [&](int n) {
-      return workspace && SCRATCH_COUNTER_BYTES + static_cast<size_t>(ctas2) * n * (TC_PART_FLOATS + TC_ML_FLOATS) * 4 <=
+      return workspace && SCRATCH_COUNTER_BYTES + static_cast<size_t>(ctas2) * n * (TC_PART_FLOATS<D> + TC_ML_FLOATS) * 4 <=
                               workspace_bytes;
     };
-    if (ctas2 * 4 <= li.sm_count && kv_tiles >= TC_CLUSTER_MIN_TILES && fits(4) && max_resident_clusters<4>() >= ctas2)
+    if (ctas2 * 4 <= li.sm_count && kv_tiles >= TC_CLUSTER_MIN_TILES && fits(4) && max_resident_clusters<D, 4>() >= ctas2)
       cl = 4;
   }
   p.scratch = cl > 1 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES) : nullptr;
   cudaError_t e;
   if (ctas2 >= li.sm_count) {
     p.q_blocks = (q_len + 255) / 256;
-    e = launch_variant<1>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
+    e = launch_variant<D, 1>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
   } else if (cl == 4) {
     p.q_blocks = (q_len + 255) / 256;
-    e = launch_variant<4>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
+    e = launch_variant<D, 4>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
   } else {
     p.q_blocks = (q_len + 127) / 128;
-    e = launch_frag(ctas1, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
+    e = launch_frag<D>(ctas1, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
   }
   li.launches += 1;
   return e;
@@ -754,8 +769,8 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
 cudaError_t launch_prefill_tc(const bf16* q, const CacheView& c, const CacheView* prefix, int prefix_len,
                               int q_heads, int q_len, int pos, float scale, float* out, float* lse, int* status,
                               void* workspace, size_t workspace_bytes, cudaStream_t st, LaunchInfo& li) {
-  return launch_tc(q, c, prefix, prefix_len, false, nullptr, 0, q_heads, q_len, pos, scale, out, lse, status, workspace,
-                   workspace_bytes, st, li);
+  return (c.head_dim == 128 ? launch_tc<128> : launch_tc<64>)(q, c, prefix, prefix_len, false, nullptr, 0, q_heads, q_len, pos,
+                                                              scale, out, lse, status, workspace, workspace_bytes, st, li);
 }
 
 cudaError_t launch_prefill_tc_fused(const bf16* q, const CacheView& c, const bf16* k_new, const bf16* v_new,
@@ -773,8 +788,9 @@ cudaError_t launch_prefill_tc_fused(const bf16* q, const CacheView& c, const bf1
   own.sr = static_cast<int64_t>(c.kv_heads) * c.head_dim;
   own.sh = c.head_dim;
   own.sb = static_cast<int64_t>(q_len) * own.sr;
-  return launch_tc(q, own, pos > 0 ? &c : nullptr, pos, true, &c, pos, q_heads, q_len, 0, scale, out, lse, status,
-                   workspace, workspace_bytes, st, li);
+  return (c.head_dim == 128 ? launch_tc<128> : launch_tc<64>)(q, own, pos > 0 ? &c : nullptr, pos, true, &c, pos, q_heads,
+                                                              q_len, 0, scale, out, lse, status, workspace,
+                                                              workspace_bytes, st, li);
 }
 
 }  // namespace jup

@@ -18,16 +18,19 @@
 
 namespace jup {
 
+template <int D>
 struct FragCfg {
+  static constexpr int TILE_BYTES = TC_BM * D * 2;
+  static constexpr int PANELS = D / 64;
   static constexpr int STAGES = 3;  // K slots = V slots = S buffers
   static constexpr int SOFTMAX_WARPS = 8, LOADER_WARP = 8, MMA_WARP = 9, WATCH_WARP = 10;
   static constexpr int THREADS = 384;
   static constexpr int REGS_SOFTMAX = 216, REGS_OTHER = 72;  // 2 x 128 x 216 + 128 x 72 = 384 x 168
   static constexpr int O_COL0 = 384;
   static constexpr int SMEM_Q = 0;
-  static constexpr int SMEM_K = TC_TILE_BYTES;
-  static constexpr int SMEM_V = SMEM_K + STAGES * TC_TILE_BYTES;
-  static constexpr int SMEM_BAR = SMEM_V + STAGES * TC_TILE_BYTES;
+  static constexpr int SMEM_K = TILE_BYTES;
+  static constexpr int SMEM_V = SMEM_K + STAGES * TILE_BYTES;
+  static constexpr int SMEM_BAR = SMEM_V + STAGES * TILE_BYTES;
   static constexpr int SMEM_BYTES = SMEM_BAR + 256 + 1024;  // + slack for 1024-byte alignment
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
 };
@@ -43,12 +46,14 @@ enum {
   FB_COUNT = 17
 };
 
-__global__ void __launch_bounds__(FragCfg::THREADS, 1)
+template <int D>
+__global__ void __launch_bounds__(FragCfg<D>::THREADS, 1)
 prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
                     const __grid_constant__ CUtensorMap tm_pv, const __grid_constant__ CUtensorMap tm_ck,
                     const __grid_constant__ CUtensorMap tm_cv, TcParams p) {
-  using Cfg = FragCfg;
+  using Cfg = FragCfg<D>;
+  constexpr int TILE_BYTES = Cfg::TILE_BYTES;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -111,20 +116,20 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     reg_dec<Cfg::REGS_OTHER>();
     if (lane == 0) {
       const int r0 = qblk * TC_BM;
-      mbar_expect_tx(bar(FB_Q_FULL), TC_TILE_BYTES);
-      tma_load_4d(sQ, &tm_q, bar(FB_Q_FULL), 0, h, r0, b);
-      tma_load_4d(sQ + TC_PANEL_BYTES, &tm_q, bar(FB_Q_FULL), 64, h, r0, b);
+      mbar_expect_tx(bar(FB_Q_FULL), TILE_BYTES);
+#pragma unroll
+      for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(sQ + c * TC_PANEL_BYTES, &tm_q, bar(FB_Q_FULL), c * 64, h, r0, b);
       bool ok = true;
       int k_issued = 0, v_issued = 0;
       auto load = [&](bool is_v, int j) {
         const int s = j % STAGES;
         const uint32_t full = bar3(is_v ? FB_V_FULL : FB_K_FULL, j);
-        const uint32_t dst = (is_v ? sV : sK) + s * TC_TILE_BYTES;
+        const uint32_t dst = (is_v ? sV : sK) + s * TILE_BYTES;
         const CUtensorMap* m = j < Tp ? (is_v ? &tm_pv : &tm_pk) : (is_v ? &tm_v : &tm_k);
         const int krow = (j < Tp ? j : j - Tp) * TC_BN, kb = (j < Tp && !p.prefix_batched) ? 0 : b;
-        mbar_expect_tx(full, TC_TILE_BYTES);
-        tma_load_4d(dst, m, full, 0, krow, hk, kb);
-        tma_load_4d(dst + TC_PANEL_BYTES, m, full, 64, krow, hk, kb);
+        mbar_expect_tx(full, TILE_BYTES);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(dst + c * TC_PANEL_BYTES, m, full, c * 64, krow, hk, kb);
         if (is_v) v_issued = j + 1;
         else k_issued = j + 1;
       };
@@ -135,11 +140,11 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       auto store_own = [&](bool is_v) {
         ok = ok && mbar_wait(bar3(is_v ? FB_V_FULL : FB_K_FULL, j_own), par3(j_own), abort_flag, p.status);
         if (!ok) return;
-        const uint32_t src = (is_v ? sV : sK) + (j_own % STAGES) * TC_TILE_BYTES;
+        const uint32_t src = (is_v ? sV : sK) + (j_own % STAGES) * TILE_BYTES;
         const CUtensorMap* m = is_v ? &tm_cv : &tm_ck;
         const int row = p.copy_pos + qblk * TC_BN;
-        tma_store_4d(m, src, 0, row, hk, b);
-        tma_store_4d(m, src + TC_PANEL_BYTES, 64, row, hk, b);
+#pragma unroll
+        for (int c = 0; c < Cfg::PANELS; ++c) tma_store_4d(m, src + c * TC_PANEL_BYTES, c * 64, row, hk, b);
         tma_store_commit();
         tma_store_wait_read();
       };
@@ -177,21 +182,21 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     reg_dec<Cfg::REGS_OTHER>();
     if (lane == 0) {
       constexpr uint32_t idesc_qk = tc_idesc_bf16(TC_BM, TC_BN, false, false);
-      constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, TC_D, false, true);
+      constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, D, false, true);
       const uint32_t q_lo = tc_desc_lo(sQ, 16), k_lo0 = tc_desc_lo(sK, 16), v_lo0 = tc_desc_lo(sV, TC_PANEL_BYTES);
       const uint32_t o_col = tmem + Cfg::O_COL0;
       // slot of K and V and S buffer are all j mod 3
       auto issue_qk = [&](int s) {  // S[s] = Q K[s]^T
-        const uint32_t k_lo = k_lo0 + s * (TC_TILE_BYTES >> 4);
+        const uint32_t k_lo = k_lo0 + s * (TILE_BYTES >> 4);
         const uint32_t d = tmem + s * 128;
 #pragma unroll
-        for (int ks = 0; ks < TC_D / 16; ++ks) {
+        for (int ks = 0; ks < D / 16; ++ks) {
           const uint32_t off = ((ks >> 2) * TC_PANEL_BYTES + (ks & 3) * 32) >> 4;
           tc_mma_ss_lo(d, q_lo + off, k_lo + off, idesc_qk, ks > 0);
         }
       };
       auto issue_pv = [&](int s, bool first) {  // O (+)= P[s] V[s]
-        const uint32_t v_lo = v_lo0 + s * (TC_TILE_BYTES >> 4);
+        const uint32_t v_lo = v_lo0 + s * (TILE_BYTES >> 4);
         const uint32_t a = tmem + s * 128;
 #pragma unroll
         for (int ks = 0; ks < TC_BN / 16; ++ks)
@@ -298,7 +303,7 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // One tile: cur holds its masked scores and mxs its maxima; nxt is the next tile's fetch in flight, whose maxima
     // are worked out between this tile's exponentials; afterwards the fetch of the tile after that goes into cur.
     auto tile = [&](int j, uint32_t (&cur)[64], uint32_t (&nxt)[64]) {
-      if (!frag_decide(mxs, m_ref, l, tO, j, [&] { return wait_o_before(j); })) {
+      if (!frag_decide<D>(mxs, m_ref, l, tO, j, [&] { return wait_o_before(j); })) {
         ok = false;
         return;
       }
@@ -340,14 +345,14 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       inv[e] = 1.f / l[e];
     }
 #pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
+    for (int hh = 0; hh < Cfg::PANELS; ++hh) {
       uint32_t o[32];
       tmem_ld_16x256b_x8(tO + hh * 64, o);
       tc_wait_ld();
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         if (!ok || row[e] >= p.q_len) continue;
-        float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row[e]) * p.q_heads + h) * TC_D + hh * 64 + col0;
+        float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row[e]) * p.q_heads + h) * D + hh * 64 + col0;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
           *reinterpret_cast<float2*>(dst + 8 * k) =

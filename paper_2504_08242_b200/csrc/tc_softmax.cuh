@@ -193,7 +193,7 @@ __device__ __forceinline__ void frag_mask_max(uint32_t (&sv)[64], bool masked, c
 
 // Lazy reference: moves m_ref[e] to the tile's maximum when that outgrew it by 2^8 and scales l and, from the second
 // tile on, the accumulator rows (wait_o(): bounded wait until O holds the tiles before this one; false: gave up).
-template <class WaitO>
+template <int D, class WaitO>
 __device__ __forceinline__ bool frag_decide(const float (&mxs)[2], float (&m_ref)[2], float (&l)[2], uint32_t tO, int j,
                                             WaitO&& wait_o) {
   bool grow[2];
@@ -211,7 +211,7 @@ __device__ __forceinline__ bool frag_decide(const float (&mxs)[2], float (&m_ref
       if (!wait_o()) return false;
       tc_fence_after();
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
+      for (int hh = 0; hh < D / 64; ++hh) {
         uint32_t o[32];
         tmem_ld_16x256b_x8(tO + hh * 64, o);
         tc_wait_ld();

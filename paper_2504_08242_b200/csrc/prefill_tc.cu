@@ -1,7 +1,7 @@
 // Chunked-prefill attention on the 5th-generation tensor cores (paper Sec. IV-A, Fig. 5(b)):
 // chunk rows at positions pos..pos+n-1 attend causally to cache rows 0..pos+i.
 //
-// Two kernels, chosen by the size of the grid (see launch_tc):
+// Two kernels, see choose_form:
 //  - prefill_tc_kernel (this file): one CTA owns TWO query tiles of 128 rows of one (sequence, query head) and walks
 //    the KV cache in tiles of 128 keys, every K/V tile serving both query tiles:
 //      loader warp : TMA (tiled, 128-byte swizzle) Q once, then K/V tiles into 2-stage rings
@@ -17,9 +17,9 @@
 //    heads in chunks of 512 (us a prompt set, in a burst / back to back), from P written over S and one issuing thread:
 //    2188 / 2390; P in its own columns and S shared, one issuer 2460 / 2613; two issuers 2024 / 2277; the PV
 //    issuer standing back for the scores 1963 / 2225; named barriers 1986 / 2223 (2720 against 3140 cycles per pair of
-//    tiles).  For grids that cannot fill the SMs a cluster of 4 CTAs shares the pair of query tiles and splits the KV
-//    walk (template parameter CL).
-//  - prefill_frag_kernel (prefill_tc_frag.cuh): one query tile per CTA, both warpgroups on it.
+//    tiles).
+//  - prefill_frag_kernel (prefill_tc_frag.cuh): one query tile per CTA, both warpgroups on it; on small grids a cluster of
+//    2, 4 or 8 CTAs shares a query tile and splits its KV walk.
 // head_dim 64 runs the same kernels with half as many operand slices and accumulator columns.  Measured against the
 // mma.sync kernel that took it before (us a call, append included, 32 / 8 heads): 16 rows at position 0 4.9 : 6.6, 448
 // rows at position 0 8.1 : 14.8, at position 2048 23 : 60, four prompts at once 65 : 171 -- never slower, so that kernel
@@ -39,7 +39,6 @@ namespace jup {
 constexpr int TC_BM = 128;              // query rows per tile
 constexpr int TC_BN = 128;              // keys per KV tile
 constexpr int TC_PANEL_BYTES = 16384;   // 128 rows x 64 elements of bf16: a Q, K or V tile is D / 64 of them
-constexpr int TC_CLUSTER_MIN_TILES = 18;     // shortest KV walk (in tiles) that a cluster of 4 CTAs shares
 
 struct TcParams {
   int q_heads, group, q_len, pos, batch;
@@ -49,7 +48,7 @@ struct TcParams {
   float* out;
   float* lse;
   int* status;
-  float* scratch;  // cluster mode: per cluster, CL x (partial accumulators 2 x 128 x 128, then (m, l) 2 x 128 x 2)
+  float* scratch;  // fragment form with several CTAs per query tile: their partial results
   int prefix_batched;  // 1: the front segment has one cache per sequence (fused form), 0: one cache shared by all
   // Fused KVCache write (fused_write != 0).  The chunk's K/V rows, token-major [batch][q_len][kv_heads][128], are
   // the attention's own segment; the CTAs of each group's first query head also write them, bit-exactly, into rows
@@ -58,9 +57,6 @@ struct TcParams {
   int fused_write;
   int copy_pos;
 };
-template <int D>
-constexpr int TC_PART_FLOATS = 2 * TC_BM * D;  // one CTA's partial accumulators (both query tiles)
-constexpr int TC_ML_FLOATS = 2 * TC_BM * 2;       // one CTA's (m, l) pairs
 
 constexpr int TC_NQ = 2;  // query tiles per CTA
 template <int D>
@@ -102,11 +98,7 @@ enum {
 constexpr int TC_BOX_FLOATS = TC_BM * 32;  // 16 KB
 constexpr int NQ = TC_NQ;
 
-// CL > 1: a thread-block cluster of CL CTAs shares one pair of query tiles; CTA r takes the KV tiles
-// r, r + CL, r + 2 CL, ... and the partial (O, m, l) are exchanged through global scratch (L2) around one
-// cluster barrier: distributed shared memory moved them at about 20 GB/s per SM when measured, L2 is
-// several times faster.  CTA r then finishes the output columns [128 r / CL, 128 (r + 1) / CL).
-template <int D, int CL>
+template <int D>
 __global__ void __launch_bounds__(TcCfg<D>::THREADS, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
@@ -126,38 +118,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   static_assert(8 * BAR_COUNT + 20 <= 256, "barrier block");
   auto bar = [&](int i) { return sBar + 8u * i; };
 
-  // a CTA of a cluster can meet rows that see none of a tile, and ends with unnormalised partials
-  constexpr bool PARTIAL = CL > 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int crank = CL > 1 ? static_cast<int>(cluster_ctarank()) : 0;
 
   // ---- work assignment: heaviest query blocks first
   const int nbh = p.batch * p.q_heads;
-  const int work = blockIdx.x / CL;
-  const int bh = work % nbh;
-  const int qblk = p.q_blocks - 1 - work / nbh;
+  const int bh = blockIdx.x % nbh;
+  const int qblk = p.q_blocks - 1 - blockIdx.x / nbh;
   const int b = bh / p.q_heads, h = bh % p.q_heads, hk = h / p.group;
   // KV tiles 0..Tp-1 come from the shared prefix (every row sees them, no causal limit), the rest from
   // the sequence's own cache
   const int Tp = (p.prefix_len + TC_BN - 1) / TC_BN;
-  // T[x]: KV tiles of query tile x; Tall: KV tiles the CTA loads (its load sequence 0..Tall-1).  CTA r of a
-  // cluster loads KV tile r + CL n as its n-th.
+  // T[x]: KV tiles of query tile x; Tall: KV tiles the CTA loads
   int T[2] = {0, 0};
-  int Tg[2] = {0, 0};  // cluster mode: tiles of the query tile over the whole cluster
 #pragma unroll
   for (int x = 0; x < NQ; ++x) {
     const int r0 = (qblk * NQ + x) * TC_BM;
     if (r0 < p.q_len) T[x] = Tp + (p.pos + min(p.q_len, r0 + TC_BM) + TC_BN - 1) / TC_BN;
   }
-  if constexpr (CL > 1) {
-#pragma unroll
-    for (int x = 0; x < NQ; ++x) {
-      Tg[x] = T[x];
-      T[x] = T[x] > crank ? (T[x] - crank + CL - 1) / CL : 0;
-    }
-  }
   const int Tall = max(T[0], T[1]);
-  auto tile_of_seq = [&](int n) { return CL > 1 ? crank + CL * n : n; };  // KV tile of a sequence number
 
   // ---- set-up
   if (threadIdx.x == 0) {
@@ -174,7 +152,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     tma_prefetch_desc(&tm_q);
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
-    if (CL == 1) tma_prefetch_desc(&tm_o);
+    tma_prefetch_desc(&tm_o);
     if (Tp > 0) {
       tma_prefetch_desc(&tm_pk);
       tma_prefetch_desc(&tm_pv);
@@ -189,8 +167,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();  // everything above overlapped the previous kernel's tail; global memory is touched from here on
-
-  float part_m = -INFINITY, part_l = 0.f;  // cluster mode: a softmax thread's (m, l) after its last tile
 
   if (warp == Cfg::LOADER_WARP) {
     // =============================================================== loader
@@ -208,12 +184,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       int issued = 0;
       bool ok = true;
       // Fused KVCache write: the chunk's own K/V tiles are loaded for the attention anyway; the tiles that hold
-      // the query rows of this CTA (of this cluster: the CTA that loads them) go from their slots to the cache with
+      // the query rows of this CTA go from their slots to the cache with
       // tiled stores, as soon as they have landed.  A slot is refilled only after its store has read it.
-      constexpr int QT = NQ;  // query tiles of the chunk per CTA (cluster)
+      constexpr int QT = NQ;  // query tiles of the chunk per CTA
       const bool writer = p.fused_write != 0 && h % p.group == 0;
       auto store_own_tile = [&](int j) {  // j: load sequence number
-        const int t = tile_of_seq(j) - Tp;  // tile of the chunk
+        const int t = j - Tp;  // tile of the chunk
         if (!writer || t < 0 || t / QT != qblk || t * TC_BN >= p.q_len) return;
         const int s = j % KV_STAGES, u = j / KV_STAGES;
         ok = ok && mbar_wait(bar(BAR_K_FULL + s), u & 1, abort_flag, p.status);
@@ -235,9 +211,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         if (u > 0) ok = mbar_wait(bar(BAR_K_EMPTY + s), (u - 1) & 1, abort_flag, p.status);
         if (!ok) break;
         mbar_expect_tx(bar(BAR_K_FULL + s), TILE_BYTES);
-        const int g = tile_of_seq(j);
-        const CUtensorMap* mk = g < Tp ? &tm_pk : &tm_k;
-        const int krow = (g < Tp ? g : g - Tp) * TC_BN, kb = (g < Tp && !p.prefix_batched) ? 0 : b;
+        const CUtensorMap* mk = j < Tp ? &tm_pk : &tm_k;
+        const int krow = (j < Tp ? j : j - Tp) * TC_BN, kb = (j < Tp && !p.prefix_batched) ? 0 : b;
 #pragma unroll
         for (int c = 0; c < Cfg::PANELS; ++c)
           tma_load_4d(sK + s * TILE_BYTES + c * TC_PANEL_BYTES, mk, bar(BAR_K_FULL + s), c * 64, krow, hk, kb);
@@ -247,7 +222,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
           break;
         }
         mbar_expect_tx(bar(BAR_V_FULL + s), TILE_BYTES);
-        const CUtensorMap* mv = g < Tp ? &tm_pv : &tm_v;
+        const CUtensorMap* mv = j < Tp ? &tm_pv : &tm_v;
 #pragma unroll
         for (int c = 0; c < Cfg::PANELS; ++c)
           tma_load_4d(sV + s * TILE_BYTES + c * TC_PANEL_BYTES, mv, bar(BAR_V_FULL + s), c * 64, krow, hk, kb);
@@ -381,10 +356,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       ok = __all_sync(0xffffffffu, ok && mbar_spin_wait(bar(BAR_S_FULL + x), j & 1, abort_flag, p.status));
       tc_fence_after();
       // columns >= nvalid are masked: the end of the prefix in its last tile, the causal limit afterwards
-      const int g = tile_of_seq(j);
-      const int nvalid = g < Tp ? p.prefix_len - g * TC_BN : lim - (g - Tp) * TC_BN;
+      const int nvalid = j < Tp ? p.prefix_len - j * TC_BN : lim - (j - Tp) * TC_BN;
       const bool masked = __any_sync(0xffffffffu, nvalid < TC_BN);
-      softmax_tile_row<PARTIAL, D>(
+      softmax_tile_row<false, D>(
           tS, tP, tO, j, 4, masked, ColumnLimit{nvalid}, c, m_ref, l,
           [&] { return mbar_test_wait(bar(BAR_O_READY + x), (j - 1) & 1); },
           [&] { ok = ok && mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
@@ -396,13 +370,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       signal(NB_P_FULL);
     }
     pdl_launch_dependents();  // the next kernel of the stream may start its own set-up now
-    if constexpr (CL > 1) {
-      // the accumulator is complete; the merge over the cluster follows the role branches
-      if (Tx > 0) ok = mbar_wait(bar(BAR_O_READY + x), (Tx - 1) & 1, abort_flag, p.status) && ok;
-      part_m = m_ref;
-      part_l = l;
-    } else if (Tx > 0) {  // warpgroup-uniform: every thread of the tile reaches the named barriers below, even
-                          // one that gave up on a wait (it only skips its global stores)
+    if (Tx > 0) {  // warpgroup-uniform: every thread of the tile reaches the named barriers below, even one that gave
+                   // up on a wait (it only skips its global stores)
       ok = ok && mbar_wait(bar(BAR_O_READY + x), (Tx - 1) & 1, abort_flag, p.status);
       tc_fence_after();
       // O / l goes out through shared memory (this tile's Q buffer, free now) and tiled stores: two rounds of
@@ -447,124 +416,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     reg_dec<Cfg::REGS_OTHER>();  // the idle warp of the third warpgroup: the re-division is a warpgroup's decision
   }
 
-  if constexpr (CL > 1) {
-    // ---- merge over the cluster.  Every thread of every CTA comes through here, whatever happened above.
-    // Each softmax thread has seen its stream's last accumulator, so after this barrier every MMA of the
-    // CTA is complete and every copy has landed: the K/V rings are free.
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    constexpr int W = D / CL;  // output columns this CTA finishes
-    // Partial accumulators, unnormalised fp32: [column slice CL][query tile 2][row 128][W], the 16-byte chunks
-    // of a row XOR-swizzled by the row (bank conflicts); staged in the K/V rings, copied as they are to the
-    // cluster's scratch.  (m, l) per row: [query tile 2][row 128].
-    float* part = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);
-    static_assert(TC_PART_FLOATS<D> * 4 <= 2 * KV_STAGES * TILE_BYTES, "partials fit in the K/V rings");
-    float* gpart = p.scratch + static_cast<size_t>(work) * CL * (TC_PART_FLOATS<D> + TC_ML_FLOATS);
-    float* gml = gpart + CL * TC_PART_FLOATS<D>;
-    if (warp < Cfg::SOFTMAX_WARPS) {
-      const int x = warp >> 2, row_in_tile = (warp & 3) * 32 + lane;
-      const uint32_t tO = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + Cfg::O_COL0 + x * 128;
-      reinterpret_cast<float2*>(gml + crank * TC_ML_FLOATS)[x * TC_BM + row_in_tile] = make_float2(part_m, part_l);
-#pragma unroll
-      for (int q4 = 0; q4 < D / 32; ++q4) {
-        uint32_t o[32];
-        if (T[x] > 0) {  // warpgroup-uniform; a stream without tiles never wrote its accumulator
-          tmem_ld32(tO + q4 * 32, o);
-          tc_wait_ld();
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] = 0u;
-        }
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
-          const int slice = (q4 * 32 + cc * 4) / W, chunk = ((q4 * 32 + cc * 4) % W) / 4;
-          *reinterpret_cast<float4*>(part + ((slice * 2 + x) * TC_BM + row_in_tile) * W +
-                                     ((chunk ^ (row_in_tile & (W / 4 - 1))) << 2)) =
-              make_float4(__uint_as_float(o[4 * cc]), __uint_as_float(o[4 * cc + 1]), __uint_as_float(o[4 * cc + 2]),
-                          __uint_as_float(o[4 * cc + 3]));
-        }
-      }
-      named_sync(NB_MERGE, 256);
-      const float4* src = reinterpret_cast<const float4*>(part);
-      float4* dst = reinterpret_cast<float4*>(gpart + crank * TC_PART_FLOATS<D>);
-#pragma unroll 8
-      for (int i = 0; i < TC_PART_FLOATS<D> / 4 / 256; ++i) dst[i * 256 + threadIdx.x] = src[i * 256 + threadIdx.x];
-      __threadfence();
-    }
-    cluster_sync_all();  // release / acquire over the cluster: the partials of every CTA are visible
-    if (warp < Cfg::SOFTMAX_WARPS) {
-      constexpr int LPR = W / 4;     // lanes per row (one 16-byte chunk each)
-      constexpr int RPI = 32 / LPR;  // rows per warp iteration
-      const int chunk = lane % LPR, sub = lane / LPR;
-      const int x = warp >> 2;
-      // a CTA of the cluster that gave up on a wait has set the status word (before the barrier): its partials are
-      // incomplete, so nobody writes rows merged from them
-      const bool cta_ok = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;
-      if (Tg[x] > 0) {  // the query tile exists
-        // This lane finishes one 16-byte chunk of the rows (warp & 3) * 32 + it * RPI + sub, it = 0..LPR-1.
-        // Loads go to L2 (the lines were written by other SMs) and are issued in batches before their first use.
-        auto row_of = [&](int it) { return (warp & 3) * 32 + it * RPI + sub; };
-        float2 ml[LPR][CL];
-#pragma unroll
-        for (int it = 0; it < LPR; ++it)
-#pragma unroll
-          for (int cr = 0; cr < CL; ++cr)
-            ml[it][cr] = __ldcg(reinterpret_cast<const float2*>(gml + cr * TC_ML_FLOATS) + x * TC_BM + row_of(it));
-        float wgt[LPR][CL];  // weight of CTA cr's partial in row it, normalisation included
-#pragma unroll
-        for (int it = 0; it < LPR; ++it) {
-          float m = -INFINITY;
-#pragma unroll
-          for (int cr = 0; cr < CL; ++cr)
-            if (ml[it][cr].y > 0.f) m = fmaxf(m, ml[it][cr].x);  // a CTA whose tiles were all hidden from the row has l = 0
-          float lsum = 0.f;
-#pragma unroll
-          for (int cr = 0; cr < CL; ++cr) {
-            wgt[it][cr] = ml[it][cr].y > 0.f ? fast_exp2(ml[it][cr].x - m) : 0.f;
-            lsum = fmaf(wgt[it][cr], ml[it][cr].y, lsum);
-          }
-          const float inv = 1.f / lsum;
-#pragma unroll
-          for (int cr = 0; cr < CL; ++cr) wgt[it][cr] *= inv;
-          const int row = (qblk * NQ + x) * TC_BM + row_of(it);
-          if (cta_ok && crank == 0 && chunk == 0 && p.lse && row < p.q_len)
-            p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row] =
-                (m + log2f(lsum)) * 0.69314718055994530942f;
-        }
-        constexpr int BATCH = 4;
-#pragma unroll
-        for (int it0 = 0; it0 < LPR; it0 += BATCH) {
-          float4 v[BATCH][CL];
-#pragma unroll
-          for (int k = 0; k < BATCH; ++k) {
-            const int r = row_of(it0 + k);
-            const int off = ((crank * 2 + x) * TC_BM + r) * W + ((chunk ^ (r & (W / 4 - 1))) << 2);
-#pragma unroll
-            for (int cr = 0; cr < CL; ++cr)
-              v[k][cr] = __ldcg(reinterpret_cast<const float4*>(gpart + cr * TC_PART_FLOATS<D> + off));
-          }
-#pragma unroll
-          for (int k = 0; k < BATCH; ++k) {
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int cr = 0; cr < CL; ++cr) {
-              const float w = wgt[it0 + k][cr];
-              acc.x = fmaf(w, v[k][cr].x, acc.x);
-              acc.y = fmaf(w, v[k][cr].y, acc.y);
-              acc.z = fmaf(w, v[k][cr].z, acc.z);
-              acc.w = fmaf(w, v[k][cr].w, acc.w);
-            }
-            const int row = (qblk * NQ + x) * TC_BM + row_of(it0 + k);
-            if (cta_ok && row < p.q_len)
-              *reinterpret_cast<float4*>(p.out + ((static_cast<int64_t>(b) * p.q_len + row) * p.q_heads + h) * D +
-                                         crank * W + chunk * 4) = acc;
-          }
-        }
-      }
-    }
-  }
-
   // ---- tear-down
   tc_fence_before();
   __syncthreads();
@@ -582,70 +433,51 @@ namespace jup {
 
 // ---------------------------------------------------------------- host side
 
-template <int D>
-static cudaError_t launch_frag(int64_t ctas, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
+template <int D, int C>
+static cudaError_t frag_set_attributes() {
+  static PerDeviceOnce done;
+  if (done.done()) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(prefill_frag_kernel<D, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       FragCfg<D>::SMEM_BYTES);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(prefill_frag_kernel<D, C>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) done.set();
+  return e;
+}
+template <int D, int C>
+static cudaError_t launch_frag(int64_t units, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
                                const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
                                const CUtensorMap& tck, const CUtensorMap& tcv, const TcParams& p) {
-  static PerDeviceOnce done;
-  if (!done.done()) {
-    cudaError_t e =
-        cudaFuncSetAttribute(prefill_frag_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, FragCfg<D>::SMEM_BYTES);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(prefill_frag_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    done.set();
-  }
-  return launch_pdl_cluster(prefill_frag_kernel<D>, dim3(static_cast<unsigned>(ctas)), dim3(FragCfg<D>::THREADS),
-                            FragCfg<D>::SMEM_BYTES, st, 1u, tq, tk, tv, tpk, tpv, tck, tcv, p);
+  cudaError_t e = frag_set_attributes<D, C>();
+  if (e != cudaSuccess) return e;
+  return launch_pdl_cluster(prefill_frag_kernel<D, C>, dim3(static_cast<unsigned>(units * C)), dim3(FragCfg<D>::THREADS),
+                            FragCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(C), tq, tk, tv, tpk, tpv, tck, tcv, p);
 }
 
-template <int D, int CL>
-static cudaError_t launch_variant(int64_t ctas, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
-                                  const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
-                                  const CUtensorMap& to, const CUtensorMap& tck, const CUtensorMap& tcv,
-                                  const TcParams& p) {
-  using Cfg = TcCfg<D>;
-  static PerDeviceOnce done;
-  if (!done.done()) {
-    cudaError_t e =
-        cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    done.set();
-  }
-  return launch_pdl_cluster(prefill_tc_kernel<D, CL>, dim3(static_cast<unsigned>(ctas * CL)),
-                            dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, static_cast<unsigned>(CL), tq, tk, tv, tpk, tpv, to, tck,
-                            tcv, p);
-}
-
-// How many clusters of CL CTAs of the cluster-mode kernel can be resident at once (0 if the query fails).
-template <int D, int CL>
-static int max_resident_clusters() {
+// How many clusters of C CTAs of the fragment form can be resident at once on the current device (0 if the query fails).
+template <int D, int C>
+static int frag_resident_clusters() {
   static std::atomic<int> cache[64];  // per device: 0 = not asked yet, else answer + 1
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   const int cached = cache[dev].load(std::memory_order_acquire);
   if (cached > 0) return cached - 1;
-  using Cfg = TcCfg<D>;
   int n = 0;
-  if (cudaFuncSetAttribute(prefill_tc_kernel<D, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           Cfg::SMEM_BYTES) == cudaSuccess) {
+  if (frag_set_attributes<D, C>() == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL * 64);
-    cfg.blockDim = dim3(Cfg::THREADS);
-    cfg.dynamicSmemBytes = Cfg::SMEM_BYTES;
+    cfg.gridDim = dim3(C * 64);
+    cfg.blockDim = dim3(FragCfg<D>::THREADS);
+    cfg.dynamicSmemBytes = FragCfg<D>::SMEM_BYTES;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL;
+    attr[0].val.clusterDim.x = C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, prefill_tc_kernel<D, CL>, &cfg) == cudaSuccess) n = got;
+    if (cudaOccupancyMaxActiveClusters(&got, prefill_frag_kernel<D, C>, &cfg) == cudaSuccess) n = got;
     else (void)cudaGetLastError();
   } else {
     (void)cudaGetLastError();
@@ -654,12 +486,75 @@ static int max_resident_clusters() {
   return n;
 }
 
+template <int D>
+static cudaError_t launch_pairs(int64_t ctas, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
+                                  const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
+                                  const CUtensorMap& to, const CUtensorMap& tck, const CUtensorMap& tcv,
+                                  const TcParams& p) {
+  using Cfg = TcCfg<D>;
+  static PerDeviceOnce done;
+  if (!done.done()) {
+    cudaError_t e =
+        cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                               cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    done.set();
+  }
+  return launch_pdl_cluster(prefill_tc_kernel<D>, dim3(static_cast<unsigned>(ctas)),
+                            dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, 1u, tq, tk, tv, tpk, tpv, to, tck,
+                            tcv, p);
+}
+
 bool prefill_tc_supported(const CacheView& c, float scale) {
   // a positive finite scale, and strides a tensor map can carry (multiples of 16 bytes below 2^40;
   // the 16-byte rule is part of every cache descriptor already)
   auto encodable = [](int64_t elems) { return static_cast<uint64_t>(elems) * 2 < (1ull << 40); };
   return scale > 0.f && scale < INFINITY && encode_fn() != nullptr && encodable(c.sr) &&
          encodable(c.sh) && encodable(c.sb);
+}
+
+// How a call is laid out: which kernel, how many CTAs share a query tile's KV walk.
+struct TcForm {
+  bool pairs;  // two query tiles per CTA (prefill_tc_kernel), else one (prefill_frag_kernel)
+  int split;
+};
+
+// The layout with the shortest estimated time, in cycles of a CTA.
+//  - A KV tile takes a CTA 2720 cycles with a pair of query tiles and 1700 with one (head_dim 128 and 64 alike); a CTA's
+//    fixed time is about 6000.
+//  - Several CTAs per query tile (a cluster) when all of them run at once: the walk shrinks by the split, the exchange of the
+//    partial results costs 2.8 / 3.7 / 4.6 us with 2 / 4 / 8 CTAs at head_dim 128 and about 2.0 / 2.1 / 2.4 at 64.  Measured
+//    (us a call, 1 : 2 : 4 : 8 CTAs, 8 heads x 100 rows): at position 192 8.1 : 10.0 : 9.4 : 10.4, at 960 13.5 : 12.6 :
+//    11.2 : 11.6, at 3968 33.6 : 22.1 : 15.6 : 13.7.  (A cluster of four CTAs sharing a PAIR of query tiles, which this
+//    replaced, took 29.6 us for 32 heads x 256 rows at position 3968 against 26.9 with two CTAs per query tile.)
+template <int D>
+static TcForm choose_form(int64_t rows_of_heads, int q_len, int kv_tiles, size_t workspace_bytes, int sm_count) {
+  constexpr int64_t PAIR = 2720, ONE = 1700, FIXED = 6000;
+  TcForm best = {false, 1};
+  int64_t best_est = -1;
+  for (int pairs = 0; pairs < 2; ++pairs) {
+    const int64_t units = rows_of_heads * (pairs ? (q_len + 255) / 256 : (q_len + 127) / 128);
+    auto consider = [&](int split, int64_t at_once, int64_t exchange) {
+      if (split > 1 && (at_once < units || kv_tiles < split ||
+                        SCRATCH_COUNTER_BYTES + static_cast<size_t>(units) * split * FRAG_PART_F4<D> * 16 > workspace_bytes))
+        return;
+      const int64_t waves = (units + at_once - 1) / at_once;
+      const int64_t est = waves * ((kv_tiles + split - 1) / split * (pairs ? PAIR : ONE) + FIXED + exchange);
+      if (best_est < 0 || est < best_est) {
+        best_est = est;
+        best = TcForm{pairs != 0, split};
+      }
+    };
+    consider(1, sm_count, 0);
+    if (!pairs && 2 * units <= sm_count) {
+      consider(2, frag_resident_clusters<D, 2>(), D == 128 ? 5200 : 3800);
+      consider(4, frag_resident_clusters<D, 4>(), D == 128 ? 7000 : 4000);
+      consider(8, frag_resident_clusters<D, 8>(), D == 128 ? 8500 : 4500);
+    }
+  }
+  return best;
 }
 
 // c: the attention's own segment (rows [0, pos + q_len) of every sequence); prefix (nullable): the segment in front
@@ -732,36 +627,20 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   p.out = out;
   p.lse = lse;
   p.status = status;
-  // Two query tiles per CTA when that still fills the machine (every K/V tile then serves two query tiles).  A
-  // grid that leaves SMs idle is latency-bound on the walk over the KV tiles: with few pairs of query tiles and a
-  // long walk, a cluster of 4 CTAs shares a pair and splits the walk; the exchange of the partials costs about
-  // 10 us, so the cluster pays from about 18 KV tiles on (measured on chunk 256 x 32 heads), and only while all
-  // clusters are resident at once.  Otherwise one query tile per CTA (fragment form).
-  const int64_t ctas2 = static_cast<int64_t>((q_len + 255) / 256) * c.batch * q_heads;
-  const int64_t ctas1 = static_cast<int64_t>((q_len + 127) / 128) * c.batch * q_heads;
   const int kv_tiles = (prefix_len + TC_BN - 1) / TC_BN + (pos + q_len + TC_BN - 1) / TC_BN;
-  int cl = 1;
-  if (ctas2 < li.sm_count && q_len > TC_BM) {
-    // scratch for the partials behind the counter block at the head of the workspace
-    auto fits = [&](int n) {
-      return workspace && SCRATCH_COUNTER_BYTES + static_cast<size_t>(ctas2) * n * (TC_PART_FLOATS<D> + TC_ML_FLOATS) * 4 <=
-                              workspace_bytes;
-    };
-    if (ctas2 * 4 <= li.sm_count && kv_tiles >= TC_CLUSTER_MIN_TILES && fits(4) && max_resident_clusters<D, 4>() >= ctas2)
-      cl = 4;
-  }
-  p.scratch = cl > 1 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES) : nullptr;
+  const TcForm f = choose_form<D>(static_cast<int64_t>(c.batch) * q_heads, q_len, kv_tiles, workspace ? workspace_bytes : 0,
+                                  li.sm_count);
+  p.q_blocks = f.pairs ? (q_len + 255) / 256 : (q_len + 127) / 128;
+  p.scratch = f.split > 1 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES) : nullptr;
+  const int64_t units = static_cast<int64_t>(p.q_blocks) * c.batch * q_heads;
   cudaError_t e;
-  if (ctas2 >= li.sm_count) {
-    p.q_blocks = (q_len + 255) / 256;
-    e = launch_variant<D, 1>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
-  } else if (cl == 4) {
-    p.q_blocks = (q_len + 255) / 256;
-    e = launch_variant<D, 4>(ctas2, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
-  } else {
-    p.q_blocks = (q_len + 127) / 128;
-    e = launch_frag<D>(ctas1, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
-  }
+  if (f.pairs)
+    e = launch_pairs<D>(units, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
+  else
+    e = (f.split == 8   ? launch_frag<D, 8>
+         : f.split == 4 ? launch_frag<D, 4>
+         : f.split == 2 ? launch_frag<D, 2>
+                        : launch_frag<D, 1>)(units, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
   li.launches += 1;
   return e;
 }

@@ -34,6 +34,8 @@ struct FragCfg {
   static constexpr int SMEM_BYTES = SMEM_BAR + 256 + 1024;  // + slack for 1024-byte alignment
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
 };
+template <int D>
+constexpr int FRAG_PART_F4 = 2 * TC_BM * D / 8 + TC_BM / 2;  // float4s of one CTA's partial: the accumulator, then (m, l)
 enum {
   FB_Q_FULL = 0,
   FB_K_FULL = 1,    // [3] slot j % 3, phase j / 3
@@ -46,7 +48,9 @@ enum {
   FB_COUNT = 17
 };
 
-template <int D>
+// C > 1: a thread-block cluster of C CTAs shares a query tile; CTA r walks the r-th of C equal ranges of its KV tiles, and
+// the partial (O, m, l) are exchanged through global scratch (L2) around one cluster barrier.
+template <int D, int C>
 __global__ void __launch_bounds__(FragCfg<D>::THREADS, 1)
 prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
@@ -72,12 +76,17 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
   // ---- work assignment: heaviest query tiles first
   const int nbh = p.batch * p.q_heads;
-  const int bh = blockIdx.x % nbh;
-  const int qblk = p.q_blocks - 1 - blockIdx.x / nbh;
+  constexpr bool SPLIT = C > 1;
+  const int crank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int work = blockIdx.x / C;
+  const int bh = work % nbh;
+  const int qblk = p.q_blocks - 1 - work / nbh;
   const int b = bh / p.q_heads, h = bh % p.q_heads, hk = h / p.group;
   // KV tiles 0..Tp-1 come from the front segment (every row sees them, no causal limit), the rest from the own one
   const int Tp = (p.prefix_len + TC_BN - 1) / TC_BN;
-  const int T = Tp + (p.pos + min(p.q_len, (qblk + 1) * TC_BM) + TC_BN - 1) / TC_BN;  // >= 1
+  const int T_all = Tp + (p.pos + min(p.q_len, (qblk + 1) * TC_BM) + TC_BN - 1) / TC_BN;  // >= 1
+  const int g0 = SPLIT ? T_all * crank / C : 0;  // this CTA's tiles are g0 .. g0 + T - 1 of them
+  const int T = SPLIT ? T_all * (crank + 1) / C - g0 : T_all;  // (may be 0 with C > 1)
   // O += P V of tile j is followed by S(j+3), whose barrier then also says that the accumulator holds tile j; the
   // last tiles have no S(j+3) and complete one of the accumulator's own barriers instead, the first for tile o0
   const int o0 = max(T - STAGES, 0);
@@ -125,8 +134,9 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const int s = j % STAGES;
         const uint32_t full = bar3(is_v ? FB_V_FULL : FB_K_FULL, j);
         const uint32_t dst = (is_v ? sV : sK) + s * TILE_BYTES;
-        const CUtensorMap* m = j < Tp ? (is_v ? &tm_pv : &tm_pk) : (is_v ? &tm_v : &tm_k);
-        const int krow = (j < Tp ? j : j - Tp) * TC_BN, kb = (j < Tp && !p.prefix_batched) ? 0 : b;
+        const int g = g0 + j;
+        const CUtensorMap* m = g < Tp ? (is_v ? &tm_pv : &tm_pk) : (is_v ? &tm_v : &tm_k);
+        const int krow = (g < Tp ? g : g - Tp) * TC_BN, kb = (g < Tp && !p.prefix_batched) ? 0 : b;
         mbar_expect_tx(full, TILE_BYTES);
 #pragma unroll
         for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(dst + c * TC_PANEL_BYTES, m, full, c * 64, krow, hk, kb);
@@ -136,7 +146,9 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // Fused KVCache write: the chunk's own K/V tile that holds this CTA's query rows goes from its slots to the
       // cache with tiled stores once it has landed, before the slot is refilled (CTAs of each group's first query
       // head only); rows beyond copy_pos + q_len are clipped by the tensor maps.
-      const int j_own = (p.fused_write != 0 && h % p.group == 0) ? Tp + qblk : -1;
+      // (with C > 1 the CTA of the cluster that walks that tile)
+      int j_own = (p.fused_write != 0 && h % p.group == 0) ? Tp + qblk - g0 : -1;
+      if (j_own >= T) j_own = -1;
       auto store_own = [&](bool is_v) {
         ok = ok && mbar_wait(bar3(is_v ? FB_V_FULL : FB_K_FULL, j_own), par3(j_own), abort_flag, p.status);
         if (!ok) return;
@@ -290,7 +302,10 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     int nvalid[2];
     auto tile_masked = [&](int j) {  // warp-uniform; fills nvalid
 #pragma unroll
-      for (int e = 0; e < 2; ++e) nvalid[e] = j < Tp ? p.prefix_len - j * TC_BN : lim[e] - (j - Tp) * TC_BN;
+      for (int e = 0; e < 2; ++e) {
+        const int g = g0 + j;
+        nvalid[e] = g < Tp ? p.prefix_len - g * TC_BN : lim[e] - (g - Tp) * TC_BN;
+      }
       return __any_sync(0xffffffffu, nvalid[0] < TC_BN || nvalid[1] < TC_BN) != 0;
     };
     auto apply_mask = [&](uint32_t (&sv)[64]) {
@@ -321,8 +336,8 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     uint32_t fa[64], fb[64];
 #pragma unroll
     for (int i = 0; i < 64; ++i) fb[i] = 0u;  // read (and ignored) as "next tile" when there is none
-    fetch(0, fa);
-    if (ok) {
+    if (!SPLIT || T > 0) fetch(0, fa);
+    if (ok && (!SPLIT || T > 0)) {
       tc_wait_ld_into(fa);
       const bool masked0 = tile_masked(0);
       frag_mask_max(fa, masked0, [&](int e, int col) { return col < nvalid[e]; }, col0, c, mxs);
@@ -334,9 +349,9 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     tc_wait_ld();  // (no fetch is left in flight; the registers are dead)
     pdl_launch_dependents();  // the next kernel of the stream may start its own set-up now
-    ok = ok && mbar_wait(bar(FB_O_READY + T - 1 - o0), 0, abort_flag, p.status);  // the accumulator is final
+    if (!SPLIT || T > 0)
+      ok = ok && mbar_wait(bar(FB_O_READY + T - 1 - o0), 0, abort_flag, p.status);  // the accumulator is final
     tc_fence_after();
-    // ---- output: O / l straight from the fragments (a row's four threads write 32 contiguous bytes per repeat)
     float inv[2];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
@@ -344,30 +359,125 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       l[e] += __shfl_xor_sync(0xffffffffu, l[e], 2);
       inv[e] = 1.f / l[e];
     }
+    if constexpr (SPLIT) {
+      // ---- this CTA's unnormalised partial -> scratch, in fragment order ([column step][thread] float4, so that every
+      // store of a warp writes 512 contiguous bytes), and (m, l) per row
+      float4* gpart = reinterpret_cast<float4*>(p.scratch) + (static_cast<size_t>(work) * C + crank) * FRAG_PART_F4<D>;
+      float2* gml = reinterpret_cast<float2*>(gpart + 2 * TC_BM * D / 8);
 #pragma unroll
-    for (int hh = 0; hh < Cfg::PANELS; ++hh) {
-      uint32_t o[32];
-      tmem_ld_16x256b_x8(tO + hh * 64, o);
-      tc_wait_ld();
+      for (int hh = 0; hh < Cfg::PANELS; ++hh) {
+        uint32_t o[32];
+        if (T > 0) {
+          tmem_ld_16x256b_x8(tO + hh * 64, o);
+          tc_wait_ld();
+        } else {  // (a CTA without tiles never wrote its accumulator)
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        if (!ok || row[e] >= p.q_len) continue;
-        float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row[e]) * p.q_heads + h) * D + hh * 64 + col0;
+          for (int k = 0; k < 32; ++k) o[k] = 0u;
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          *reinterpret_cast<float2*>(dst + 8 * k) =
-              make_float2(__uint_as_float(o[4 * k + 2 * e]) * inv[e], __uint_as_float(o[4 * k + 2 * e + 1]) * inv[e]);
+          gpart[(hh * 8 + k) * 256 + threadIdx.x] =
+              make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]), __uint_as_float(o[4 * k + 2]),
+                          __uint_as_float(o[4 * k + 3]));
       }
-    }
-    if (ok && p.lse && (lane & 3) == 0) {
+      if ((lane & 3) == 0) {
 #pragma unroll
-      for (int e = 0; e < 2; ++e)
-        if (row[e] < p.q_len)
-          p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row[e]] =
-              (m_ref[e] + log2f(l[e])) * 0.69314718055994530942f;
+        for (int e = 0; e < 2; ++e) gml[lane0 + (lane >> 2) + 8 * e] = make_float2(T > 0 ? m_ref[e] : -INFINITY, l[e]);
+      }
+      __threadfence();  // visible to the cluster before its barrier is passed
+    } else {
+      // ---- output: O / l straight from the fragments (a row's four threads write 32 contiguous bytes per repeat)
+#pragma unroll
+      for (int hh = 0; hh < Cfg::PANELS; ++hh) {
+        uint32_t o[32];
+        tmem_ld_16x256b_x8(tO + hh * 64, o);
+        tc_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          if (!ok || row[e] >= p.q_len) continue;
+          float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row[e]) * p.q_heads + h) * D + hh * 64 + col0;
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            *reinterpret_cast<float2*>(dst + 8 * k) =
+                make_float2(__uint_as_float(o[4 * k + 2 * e]) * inv[e], __uint_as_float(o[4 * k + 2 * e + 1]) * inv[e]);
+        }
+      }
+      if (ok && p.lse && (lane & 3) == 0) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (row[e] < p.q_len)
+            p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row[e]] =
+                (m_ref[e] + log2f(l[e])) * 0.69314718055994530942f;
+      }
     }
   } else {
     reg_dec<Cfg::REGS_OTHER>();  // the idle warp of the third warpgroup: the re-division is a warpgroup's decision
+  }
+
+  if constexpr (SPLIT) {
+    // ---- merge over the cluster.  Every thread of every CTA comes through here, whatever happened above.  CTA r
+    // finishes the fragments of the softmax threads [256 r / C, 256 (r + 1) / C), i.e. the rows of 8 / C warps: thread t
+    // of them every C-th column step, all loads in flight at once; the sums run in CTA order.
+    cluster_sync_all();  // release / acquire over the cluster: the partials of every CTA are visible
+    if (warp < Cfg::SOFTMAX_WARPS) {
+      const bool cta_ok = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;  // nobody gave up on a wait
+      constexpr int PER = 256 / C, STEPS = D / 8, MINE = STEPS / C;
+      const int sub = threadIdx.x / PER, t = PER * crank + threadIdx.x % PER;
+      const int w_t = t >> 5, l_t = t & 31;
+      const int r0 = (w_t & 3) * 32 + (w_t >> 2) * 16 + (l_t >> 2);  // rows r0 and r0 + 8 of the tile
+      const float4* upart = reinterpret_cast<const float4*>(p.scratch) + static_cast<size_t>(work) * C * FRAG_PART_F4<D>;
+      float2 ml[2][C];
+      float4 v[MINE][C];
+#pragma unroll
+      for (int cr = 0; cr < C; ++cr)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          ml[e][cr] = __ldcg(reinterpret_cast<const float2*>(upart + cr * FRAG_PART_F4<D> + 2 * TC_BM * D / 8) + r0 + 8 * e);
+#pragma unroll
+      for (int u = 0; u < MINE; ++u)
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) v[u][cr] = __ldcg(upart + cr * FRAG_PART_F4<D> + (u * C + sub) * 256 + t);
+      float wgt[2][C], m[2], lsum[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        m[e] = -INFINITY;
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) m[e] = fmaxf(m[e], ml[e][cr].x);  // (-inf: all its tiles were hidden from the row)
+        lsum[e] = 0.f;
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) {
+          wgt[e][cr] = fast_exp2(ml[e][cr].x - m[e]);
+          lsum[e] = fmaf(wgt[e][cr], ml[e][cr].y, lsum[e]);
+        }
+        const float inv = 1.f / lsum[e];
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) wgt[e][cr] *= inv;
+      }
+      const int row0 = qblk * TC_BM + r0;
+      float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row0) * p.q_heads + h) * D + 2 * (l_t & 3);
+#pragma unroll
+      for (int u = 0; u < MINE; ++u) {
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) {
+          acc.x = fmaf(wgt[0][cr], v[u][cr].x, acc.x);
+          acc.y = fmaf(wgt[0][cr], v[u][cr].y, acc.y);
+          acc.z = fmaf(wgt[1][cr], v[u][cr].z, acc.z);
+          acc.w = fmaf(wgt[1][cr], v[u][cr].w, acc.w);
+        }
+        const int col = 8 * (u * C + sub);
+        if (cta_ok && row0 < p.q_len) *reinterpret_cast<float2*>(dst + col) = make_float2(acc.x, acc.y);
+        if (cta_ok && row0 + 8 < p.q_len)
+          *reinterpret_cast<float2*>(dst + static_cast<int64_t>(8) * p.q_heads * D + col) = make_float2(acc.z, acc.w);
+      }
+      if (cta_ok && p.lse && sub == 0 && (l_t & 3) == 0) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (row0 + 8 * e < p.q_len)
+            p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row0 + 8 * e] =
+                (m[e] + log2f(lsum[e])) * 0.69314718055994530942f;
+      }
+    }
   }
 
   // ---- tear-down

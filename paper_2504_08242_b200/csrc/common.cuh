@@ -69,6 +69,32 @@ __device__ __forceinline__ float fast_exp2(float x) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// Division of 0 <= n < 2^31 by a number that the host knows (the round-up method of Granlund and Montgomery, 1994): a
+// multiplication and a shift instead of some 40 dependent instructions, for the set-up of a CTA, which nothing hides.
+struct FastDiv {
+  uint32_t d, m, s;
+  FastDiv() = default;
+  __host__ explicit FastDiv(uint32_t divisor) : d(divisor), m(0), s(0) {
+    while ((uint64_t(1) << s) < d) ++s;
+    m = static_cast<uint32_t>(((uint64_t(1) << 32) * ((uint64_t(1) << s) - d)) / d + 1);
+  }
+  __device__ __forceinline__ int div(int n) const {
+    return static_cast<int>((__umulhi(static_cast<uint32_t>(n), m) + static_cast<uint32_t>(n)) >> s);
+  }
+  __device__ __forceinline__ int divmod(int n, int& rem) const {
+    const int q = div(n);
+    rem = n - q * static_cast<int>(d);
+    return q;
+  }
+};
+
+// The value, as one that is only known from here on: keeps arithmetic of an epilogue from being moved in front of the main
+// loop, where its results would occupy registers.
+__device__ __forceinline__ int known_here(int v) {
+  asm volatile("" : "+r"(v));
+  return v;
+}
+
 // Byte offset of 16-byte chunk `c` of row `row` inside a [rows][D] bf16 tile whose rows
 // are D*2 bytes; the chunk index is XOR-swizzled with the row so that ldmatrix reads of
 // eight consecutive rows hit distinct banks.

@@ -1,9 +1,9 @@
 // Chunked-prefill attention on the 5th-generation tensor cores (paper Sec. IV-A, Fig. 5(b)):
 // chunk rows at positions pos..pos+n-1 attend causally to cache rows 0..pos+i.
 //
-// Two kernels, see choose_form:
-//  - prefill_tc_kernel (this file): one CTA owns TWO query tiles of 128 rows of one (sequence, query head) and walks
-//    the KV cache in tiles of 128 keys, every K/V tile serving both query tiles:
+// Two kernels (see choose_form).  A query tile is 128 rows: tokens of the chunk x heads that share a kv head.
+//  - prefill_tc_kernel (this file): one CTA owns TWO query tiles of the same kv head and walks the KV cache in tiles of
+//    128 keys, every K/V tile serving both query tiles:
 //      loader warp : TMA (tiled, 128-byte swizzle) Q once, then K/V tiles into 2-stage rings
 //      MMA warps   : one thread issues the tcgen05.mma of S = Q K^T, another those of O += P V, accumulators in TMEM
 //      softmax WGs : one warpgroup per query tile, one thread per row holding the row's 128 scores in registers:
@@ -27,6 +27,7 @@
 // All mbarrier waits are bounded; on expiry the CTA sets the status word, drains its own copies and MMAs, frees
 // TMEM and returns.
 #include "host_checks.h"
+#include <algorithm>
 #include <atomic>
 
 #include "kernels.h"
@@ -41,9 +42,13 @@ constexpr int TC_BN = 128;              // keys per KV tile
 constexpr int TC_PANEL_BYTES = 16384;   // 128 rows x 64 elements of bf16: a Q, K or V tile is D / 64 of them
 
 struct TcParams {
-  int q_heads, group, q_len, pos, batch;
+  int q_heads, q_len, pos;
   int prefix_len;  // rows of a shared prefix cache attended before the sequence's own cache (0: none)
-  int q_blocks;  // query tiles (fragment form) or pairs of query tiles per (sequence, head)
+  // A query tile is `tokens` tokens x `pack` heads that share a kv head, tokens * pack <= 128 rows, the heads running
+  // fastest.
+  int tokens;
+  FastDiv pack, head_blocks, blocks_per_kv, batch_blocks;  // head_blocks = q_heads / pack, batch_blocks = batch x head_blocks
+  int q_blocks;  // query tiles (fragment form) or pairs of query tiles per (sequence, block of heads)
   float scale_log2;
   float* out;
   float* lse;
@@ -57,6 +62,10 @@ struct TcParams {
   int fused_write;
   int copy_pos;
 };
+
+// One past the last of the chunk's K/V tiles that the query tile(s) of tokens [t0, t1) write to the cache: the tiles whose
+// last token they hold.  (The first is t0 / TC_BN.)
+__device__ __forceinline__ int own_tiles_end(int t1, int q_len) { return t1 == q_len ? (q_len + TC_BN - 1) / TC_BN : t1 / TC_BN; }
 
 constexpr int TC_NQ = 2;  // query tiles per CTA
 template <int D>
@@ -121,10 +130,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- work assignment: heaviest query blocks first
-  const int nbh = p.batch * p.q_heads;
-  const int bh = blockIdx.x % nbh;
-  const int qblk = p.q_blocks - 1 - blockIdx.x / nbh;
-  const int b = bh / p.q_heads, h = bh % p.q_heads, hk = h / p.group;
+  int bh, hb, hr;
+  const int qblk = p.q_blocks - 1 - p.batch_blocks.divmod(blockIdx.x, bh);
+  const int b = p.head_blocks.divmod(bh, hb), hk = p.blocks_per_kv.divmod(hb, hr);  // hr: 0 for a group's first heads
+  const int pack = p.pack.d, h0 = hb * pack;
   // KV tiles 0..Tp-1 come from the shared prefix (every row sees them, no causal limit), the rest from
   // the sequence's own cache
   const int Tp = (p.prefix_len + TC_BN - 1) / TC_BN;
@@ -132,8 +141,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   int T[2] = {0, 0};
 #pragma unroll
   for (int x = 0; x < NQ; ++x) {
-    const int r0 = (qblk * NQ + x) * TC_BM;
-    if (r0 < p.q_len) T[x] = Tp + (p.pos + min(p.q_len, r0 + TC_BM) + TC_BN - 1) / TC_BN;
+    const int t0 = (qblk * NQ + x) * p.tokens;
+    if (t0 < p.q_len) T[x] = Tp + (p.pos + min(p.q_len, t0 + p.tokens) + TC_BN - 1) / TC_BN;
   }
   const int Tall = max(T[0], T[1]);
 
@@ -175,22 +184,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
         if (T[x] == 0) continue;
-        const int r0 = (qblk * NQ + x) * TC_BM;
-        mbar_expect_tx(bar(BAR_Q_FULL + x), TILE_BYTES);
+        // (rows of a Q tile beyond its pack x tokens are never written: they belong to no query, and whatever the
+        // tensor cores make of them is never used)
+        mbar_expect_tx(bar(BAR_Q_FULL + x), static_cast<uint32_t>(pack * p.tokens) * (D * 2u));
 #pragma unroll
         for (int c = 0; c < Cfg::PANELS; ++c)
-          tma_load_4d(sQ + x * TILE_BYTES + c * TC_PANEL_BYTES, &tm_q, bar(BAR_Q_FULL + x), c * 64, h, r0, b);
+          tma_load_4d(sQ + x * TILE_BYTES + c * TC_PANEL_BYTES, &tm_q, bar(BAR_Q_FULL + x), c * 64, h0, (qblk * NQ + x) * p.tokens, b);
       }
       int issued = 0;
       bool ok = true;
-      // Fused KVCache write: the chunk's own K/V tiles are loaded for the attention anyway; the tiles that hold
-      // the query rows of this CTA go from their slots to the cache with
-      // tiled stores, as soon as they have landed.  A slot is refilled only after its store has read it.
-      constexpr int QT = NQ;  // query tiles of the chunk per CTA
-      const bool writer = p.fused_write != 0 && h % p.group == 0;
-      auto store_own_tile = [&](int j) {  // j: load sequence number
+      // Fused KVCache write: the chunk's own K/V tiles are loaded for the attention anyway; the tiles whose last token
+      // is in this CTA's query tiles (of each group's first heads) go from their slots to the cache with tiled stores,
+      // as soon as they have landed.  A slot is refilled only after its store has read it.
+      const bool writer = p.fused_write != 0 && hr == 0;
+      const int own0 = qblk * NQ * p.tokens / TC_BN;
+      const int own1 = own_tiles_end(min((qblk + 1) * NQ * p.tokens, p.q_len), p.q_len);
+      auto store_own_tile = [&](int j) {
         const int t = j - Tp;  // tile of the chunk
-        if (!writer || t < 0 || t / QT != qblk || t * TC_BN >= p.q_len) return;
+        if (!writer || t < own0 || t >= own1) return;
         const int s = j % KV_STAGES, u = j / KV_STAGES;
         ok = ok && mbar_wait(bar(BAR_K_FULL + s), u & 1, abort_flag, p.status);
         ok = ok && mbar_wait(bar(BAR_V_FULL + s), u & 1, abort_flag, p.status);
@@ -336,9 +347,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     reg_inc<Cfg::REGS_SOFTMAX>();
     const int x = warp >> 2;                      // query tile of this warpgroup
     const int row_in_tile = (warp & 3) * 32 + lane;
-    const int row = (qblk * NQ + x) * TC_BM + row_in_tile;  // row inside the chunk
-    const bool row_valid = row < p.q_len;
-    const int lim = p.pos + min(row, p.q_len - 1) + 1;      // keys j < lim are visible
+    const int t0 = (qblk * NQ + x) * p.tokens;
+    const int lim = p.pos + min(t0 + p.pack.div(row_in_tile), p.q_len - 1) + 1;  // keys j < lim are visible
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t tO = tmem + lane_base + Cfg::O_COL0 + x * 128;
     const float c = p.scale_log2;
@@ -380,7 +390,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_Q + x * TILE_BYTES);
       const uint32_t stage_addr = sQ + x * TILE_BYTES;
       const int tid_t = threadIdx.x & 127;
-      const int tile_row0 = (qblk * NQ + x) * TC_BM;
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
 #pragma unroll
@@ -399,15 +408,17 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
           if (ok) {
 #pragma unroll
             for (int c = 0; c < Cfg::PANELS; ++c)
-              tma_store_4d(&tm_o, stage_addr + c * TC_BOX_FLOATS * 4, hh * (D / 2) + c * 32, h, tile_row0, b);
+              tma_store_4d(&tm_o, stage_addr + c * TC_BOX_FLOATS * 4, hh * (D / 2) + c * 32, h0, t0, b);
             tma_store_commit();
           }
           tma_store_wait_read();  // the boxes are rewritten next / shared memory is released at the end of the kernel
         }
         if (hh == 0) named_sync(NB_STORE + x, 128);
       }
-      if (ok && p.lse && row_valid)
-        p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row] =
+      int hd;
+      const int tok = t0 + p.pack.divmod(known_here(row_in_tile), hd);
+      if (ok && p.lse && tok < min(p.q_len, t0 + p.tokens))
+        p.lse[(static_cast<int64_t>(b) * p.q_heads + h0 + hd) * p.q_len + tok] =
             (m_ref + log2f(l)) * 0.69314718055994530942f;
     }
   }
@@ -515,43 +526,56 @@ bool prefill_tc_supported(const CacheView& c, float scale) {
          encodable(c.sh) && encodable(c.sb);
 }
 
-// How a call is laid out: which kernel, how many CTAs share a query tile's KV walk.
+// How a call is laid out: which kernel, how many of a kv head's query heads share a query tile, how many CTAs share its
+// KV walk.
 struct TcForm {
   bool pairs;  // two query tiles per CTA (prefill_tc_kernel), else one (prefill_frag_kernel)
-  int split;
+  int pack, tokens, split;
 };
 
 // The layout with the shortest estimated time, in cycles of a CTA.
 //  - A KV tile takes a CTA 2720 cycles with a pair of query tiles and 1700 with one (head_dim 128 and 64 alike); a CTA's
 //    fixed time is about 6000.
+//  - Heads of a group in one query tile: as many as make the fewest CTAs.  A chunk of 150 tokens with 4 heads per kv head
+//    is 5 tiles of 32 tokens x 4 heads instead of 8 of 128 tokens x 1 head.
 //  - Several CTAs per query tile (a cluster) when all of them run at once: the walk shrinks by the split, the exchange of the
-//    partial results costs 2.8 / 3.7 / 4.6 us with 2 / 4 / 8 CTAs at head_dim 128 and about 2.0 / 2.1 / 2.4 at 64.  Measured
-//    (us a call, 1 : 2 : 4 : 8 CTAs, 8 heads x 100 rows): at position 192 8.1 : 10.0 : 9.4 : 10.4, at 960 13.5 : 12.6 :
-//    11.2 : 11.6, at 3968 33.6 : 22.1 : 15.6 : 13.7.  (A cluster of four CTAs sharing a PAIR of query tiles, which this
-//    replaced, took 29.6 us for 32 heads x 256 rows at position 3968 against 26.9 with two CTAs per query tile.)
+//    partial results costs about 2.5 us and more with every CTA that takes part.  Measured (us a call, 1 CTA per query tile :
+//    the chosen split, head_dim 128): 8 heads x 100 rows at position 192 8.1 : 8.1 (1), at 960 13.5 : 9.6 (8), at 3968
+//    33.6 : 11.7 (8); 32 heads x 256 rows at 960 15.4 : 13.9 (2), at 3968 38.5 : 27.1 (2).  (A cluster of four CTAs sharing
+//    a PAIR of query tiles, which this replaced, took 29.6 us for the last.)
 template <int D>
-static TcForm choose_form(int64_t rows_of_heads, int q_len, int kv_tiles, size_t workspace_bytes, int sm_count) {
+static TcForm choose_form(int batch, int q_heads, int group, int q_len, int kv_tiles, size_t workspace_bytes, int sm_count) {
   constexpr int64_t PAIR = 2720, ONE = 1700, FIXED = 6000;
-  TcForm best = {false, 1};
+  TcForm best = {false, 1, TC_BM, 1};
   int64_t best_est = -1;
   for (int pairs = 0; pairs < 2; ++pairs) {
-    const int64_t units = rows_of_heads * (pairs ? (q_len + 255) / 256 : (q_len + 127) / 128);
-    auto consider = [&](int split, int64_t at_once, int64_t exchange) {
+    int pack = 1;
+    int64_t units = -1;
+    for (int g = 1; g <= std::min(group, TC_BM); ++g) {
+      if (group % g != 0) continue;
+      const int tokens = TC_BM / g, tiles = (q_len + tokens - 1) / tokens;
+      const int64_t u = static_cast<int64_t>(batch) * (q_heads / g) * (pairs ? (tiles + 1) / 2 : tiles);
+      if (units < 0 || u < units) {
+        units = u;
+        pack = g;
+      }
+    }
+    auto consider = [&](int split, int64_t at_once) {
       if (split > 1 && (at_once < units || kv_tiles < split ||
                         SCRATCH_COUNTER_BYTES + static_cast<size_t>(units) * split * FRAG_PART_F4<D> * 16 > workspace_bytes))
         return;
-      const int64_t waves = (units + at_once - 1) / at_once;
+      const int64_t waves = (units + at_once - 1) / at_once, exchange = split > 1 ? 4500 + D / 6 * units * split : 0;
       const int64_t est = waves * ((kv_tiles + split - 1) / split * (pairs ? PAIR : ONE) + FIXED + exchange);
       if (best_est < 0 || est < best_est) {
         best_est = est;
-        best = TcForm{pairs != 0, split};
+        best = TcForm{pairs != 0, pack, TC_BM / pack, split};
       }
     };
-    consider(1, sm_count, 0);
+    consider(1, sm_count);
     if (!pairs && 2 * units <= sm_count) {
-      consider(2, frag_resident_clusters<D, 2>(), D == 128 ? 5200 : 3800);
-      consider(4, frag_resident_clusters<D, 4>(), D == 128 ? 7000 : 4000);
-      consider(8, frag_resident_clusters<D, 8>(), D == 128 ? 8500 : 4500);
+      consider(2, frag_resident_clusters<D, 2>());
+      consider(4, frag_resident_clusters<D, 4>());
+      consider(8, frag_resident_clusters<D, 8>());
     }
   }
   return best;
@@ -567,12 +591,16 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
                              size_t workspace_bytes, cudaStream_t st, LaunchInfo& li) {
   CUtensorMap tq, tk, tv, tpk, tpv, to, tck, tcv;
   if (!encode_fn()) return cudaErrorInvalidValue;
-  {  // out: [batch][q_len][q_heads][D] fp32, boxes of 128 rows x 32 columns
+  if (!prefix) prefix_len = 0;
+  const int kv_tiles = (prefix_len + TC_BN - 1) / TC_BN + (pos + q_len + TC_BN - 1) / TC_BN;
+  const TcForm f = choose_form<D>(c.batch, q_heads, q_heads / c.kv_heads, q_len, kv_tiles, workspace ? workspace_bytes : 0,
+                                  li.sm_count);
+  {  // out: [batch][q_len][q_heads][D] fp32, boxes of a query tile's rows x 32 columns
     const uint64_t d[4] = {D, static_cast<uint64_t>(q_heads), static_cast<uint64_t>(q_len),
                            static_cast<uint64_t>(c.batch)};
     const uint64_t s[3] = {D * 4ull, static_cast<uint64_t>(q_heads) * D * 4ull,
                            static_cast<uint64_t>(q_len) * q_heads * D * 4ull};
-    const uint32_t bx[4] = {32, 1, TC_BM, 1};
+    const uint32_t bx[4] = {32, static_cast<uint32_t>(f.pack), static_cast<uint32_t>(f.tokens), 1};
     if (!make_map_f32(&to, out, d, s, bx)) return cudaErrorInvalidValue;
   }
   const uint64_t rows_valid = static_cast<uint64_t>(pos) + q_len;  // rows above are dead: TMA zero-fills them
@@ -581,7 +609,7 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
                            static_cast<uint64_t>(c.batch)};
     const uint64_t s[3] = {D * 2ull, static_cast<uint64_t>(q_heads) * D * 2ull,
                            static_cast<uint64_t>(q_len) * q_heads * D * 2ull};
-    const uint32_t bx[4] = {64, 1, TC_BM, 1};
+    const uint32_t bx[4] = {64, static_cast<uint32_t>(f.pack), static_cast<uint32_t>(f.tokens), 1};
     if (!make_map_bf16(&tq, q, d, s, bx)) return cudaErrorInvalidValue;
   }
   {
@@ -605,11 +633,9 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   }
   TcParams p;
   p.q_heads = q_heads;
-  p.group = q_heads / c.kv_heads;
   p.q_len = q_len;
   p.pos = pos;
   p.prefix_len = prefix_len;
-  p.batch = c.batch;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.prefix_batched = prefix_batched ? 1 : 0;
   p.fused_write = copy_dst ? 1 : 0;
@@ -627,12 +653,16 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   p.out = out;
   p.lse = lse;
   p.status = status;
-  const int kv_tiles = (prefix_len + TC_BN - 1) / TC_BN + (pos + q_len + TC_BN - 1) / TC_BN;
-  const TcForm f = choose_form<D>(static_cast<int64_t>(c.batch) * q_heads, q_len, kv_tiles, workspace ? workspace_bytes : 0,
-                                  li.sm_count);
-  p.q_blocks = f.pairs ? (q_len + 255) / 256 : (q_len + 127) / 128;
+  const int head_blocks = q_heads / f.pack;
+  p.tokens = f.tokens;
+  p.pack = FastDiv(f.pack);
+  p.head_blocks = FastDiv(head_blocks);
+  p.blocks_per_kv = FastDiv(head_blocks / c.kv_heads);
+  p.batch_blocks = FastDiv(static_cast<uint32_t>(c.batch) * head_blocks);
+  const int q_tiles = (q_len + f.tokens - 1) / f.tokens;
+  p.q_blocks = f.pairs ? (q_tiles + 1) / 2 : q_tiles;
   p.scratch = f.split > 1 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES) : nullptr;
-  const int64_t units = static_cast<int64_t>(p.q_blocks) * c.batch * q_heads;
+  const int64_t units = static_cast<int64_t>(p.q_blocks) * c.batch * head_blocks;
   cudaError_t e;
   if (f.pairs)
     e = launch_pairs<D>(units, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);

@@ -75,16 +75,30 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // ---- work assignment: heaviest query tiles first
-  const int nbh = p.batch * p.q_heads;
   constexpr bool SPLIT = C > 1;
   const int crank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
   const int work = blockIdx.x / C;
-  const int bh = work % nbh;
-  const int qblk = p.q_blocks - 1 - work / nbh;
-  const int b = bh / p.q_heads, h = bh % p.q_heads, hk = h / p.group;
+  // (recomputed behind the walk, so that the softmax does not carry it through)
+  struct Place {
+    int b, h0, hk, t0, t1;  // sequence, first head, kv head, tokens [t0, t1) of the query tile
+    bool first_heads;       // of their group
+  };
+  auto place = [&](int w) {
+    int bh, hb, hr;
+    Place a;
+    const int qblk = p.q_blocks - 1 - p.batch_blocks.divmod(w, bh);
+    a.b = p.head_blocks.divmod(bh, hb);
+    a.hk = p.blocks_per_kv.divmod(hb, hr);
+    a.first_heads = hr == 0;
+    a.h0 = hb * static_cast<int>(p.pack.d);
+    a.t0 = qblk * p.tokens;
+    a.t1 = min(p.q_len, a.t0 + p.tokens);
+    return a;
+  };
+  const Place at = place(work);
   // KV tiles 0..Tp-1 come from the front segment (every row sees them, no causal limit), the rest from the own one
   const int Tp = (p.prefix_len + TC_BN - 1) / TC_BN;
-  const int T_all = Tp + (p.pos + min(p.q_len, (qblk + 1) * TC_BM) + TC_BN - 1) / TC_BN;  // >= 1
+  const int T_all = Tp + (p.pos + at.t1 + TC_BN - 1) / TC_BN;  // >= 1
   const int g0 = SPLIT ? T_all * crank / C : 0;  // this CTA's tiles are g0 .. g0 + T - 1 of them
   const int T = SPLIT ? T_all * (crank + 1) / C - g0 : T_all;  // (may be 0 with C > 1)
   // O += P V of tile j is followed by S(j+3), whose barrier then also says that the accumulator holds tile j; the
@@ -124,10 +138,11 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // =============================================================== loader
     reg_dec<Cfg::REGS_OTHER>();
     if (lane == 0) {
-      const int r0 = qblk * TC_BM;
-      mbar_expect_tx(bar(FB_Q_FULL), TILE_BYTES);
+      // (rows of the Q tile beyond its pack x tokens are never written: they belong to no query, and whatever the
+      // tensor cores make of them is never used)
+      mbar_expect_tx(bar(FB_Q_FULL), p.pack.d * p.tokens * (D * 2u));
 #pragma unroll
-      for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(sQ + c * TC_PANEL_BYTES, &tm_q, bar(FB_Q_FULL), c * 64, h, r0, b);
+      for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(sQ + c * TC_PANEL_BYTES, &tm_q, bar(FB_Q_FULL), c * 64, at.h0, at.t0, at.b);
       bool ok = true;
       int k_issued = 0, v_issued = 0;
       auto load = [&](bool is_v, int j) {
@@ -136,27 +151,28 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint32_t dst = (is_v ? sV : sK) + s * TILE_BYTES;
         const int g = g0 + j;
         const CUtensorMap* m = g < Tp ? (is_v ? &tm_pv : &tm_pk) : (is_v ? &tm_v : &tm_k);
-        const int krow = (g < Tp ? g : g - Tp) * TC_BN, kb = (g < Tp && !p.prefix_batched) ? 0 : b;
+        const int krow = (g < Tp ? g : g - Tp) * TC_BN, kb = (g < Tp && !p.prefix_batched) ? 0 : at.b;
         mbar_expect_tx(full, TILE_BYTES);
 #pragma unroll
-        for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(dst + c * TC_PANEL_BYTES, m, full, c * 64, krow, hk, kb);
+        for (int c = 0; c < Cfg::PANELS; ++c) tma_load_4d(dst + c * TC_PANEL_BYTES, m, full, c * 64, krow, at.hk, kb);
         if (is_v) v_issued = j + 1;
         else k_issued = j + 1;
       };
-      // Fused KVCache write: the chunk's own K/V tile that holds this CTA's query rows goes from its slots to the
-      // cache with tiled stores once it has landed, before the slot is refilled (CTAs of each group's first query
-      // head only); rows beyond copy_pos + q_len are clipped by the tensor maps.
-      // (with C > 1 the CTA of the cluster that walks that tile)
-      int j_own = (p.fused_write != 0 && h % p.group == 0) ? Tp + qblk - g0 : -1;
-      if (j_own >= T) j_own = -1;
-      auto store_own = [&](bool is_v) {
-        ok = ok && mbar_wait(bar3(is_v ? FB_V_FULL : FB_K_FULL, j_own), par3(j_own), abort_flag, p.status);
+      // Fused KVCache write: a tile of the chunk's own K/V goes from its slots to the cache with tiled stores once it has
+      // landed, before the slot is refilled: by the CTA whose query tile holds the tile's last token (of each group's
+      // first heads; with C > 1 the CTA of the cluster that walks the tile); rows beyond copy_pos + q_len are clipped
+      // by the tensor maps.
+      const bool writer = p.fused_write != 0 && at.first_heads;
+      const int own0 = Tp + at.t0 / TC_BN - g0, own1 = writer ? Tp + own_tiles_end(at.t1, p.q_len) - g0 : own0;
+      auto own = [&](int j) { return j >= own0 && j < own1; };
+      auto store_own = [&](bool is_v, int j) {
+        ok = ok && mbar_wait(bar3(is_v ? FB_V_FULL : FB_K_FULL, j), par3(j), abort_flag, p.status);
         if (!ok) return;
-        const uint32_t src = (is_v ? sV : sK) + (j_own % STAGES) * TILE_BYTES;
+        const uint32_t src = (is_v ? sV : sK) + (j % STAGES) * TILE_BYTES;
         const CUtensorMap* m = is_v ? &tm_cv : &tm_ck;
-        const int row = p.copy_pos + qblk * TC_BN;
+        const int row = p.copy_pos + (g0 + j - Tp) * TC_BN;
 #pragma unroll
-        for (int c = 0; c < Cfg::PANELS; ++c) tma_store_4d(m, src + c * TC_PANEL_BYTES, c * 64, row, hk, b);
+        for (int c = 0; c < Cfg::PANELS; ++c) tma_store_4d(m, src + c * TC_PANEL_BYTES, c * 64, row, at.hk, at.b);
         tma_store_commit();
         tma_store_wait_read();
       };
@@ -164,20 +180,17 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         load(false, j);
         load(true, j);
       }
-      bool v_stored = false;
       for (int i = 0; i < T && ok; ++i) {
         ok = mbar_wait(bar3(FB_S_FULL, i), par3(i), abort_flag, p.status);
         if (!ok) break;
-        if (j_own >= 0 && i == j_own) store_own(false);
-        if (j_own >= 0 && i - STAGES == j_own) {
-          store_own(true);
-          v_stored = true;
-        }
+        if (own(i)) store_own(false, i);
+        if (i >= STAGES && own(i - STAGES)) store_own(true, i - STAGES);
         if (!ok) break;
         if (i + STAGES < T) load(false, i + STAGES);  // K(i)'s slot
         if (i >= STAGES) load(true, i);               // V(i-3)'s slot
       }
-      if (ok && j_own >= 0 && !v_stored) store_own(true);
+      for (int i = max(0, T - STAGES); i < T && ok; ++i)
+        if (own(i)) store_own(true, i);
       if (*abort_flag) {
         // wait (bounded) until every copy this thread started has landed before shared memory is released
         int dummy = 0;
@@ -276,12 +289,13 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int col0 = 2 * (lane & 3);
     const uint32_t taddr = tmem + (static_cast<uint32_t>(lane0) << 16);
     const uint32_t tO = taddr + Cfg::O_COL0;
-    int row[2], lim[2];  // row inside the chunk and its causal limit (keys j < lim are visible)
+    // Columns of tile 0 that this thread's rows would see if they were all of the own segment (its causal limit), or all
+    // of the front segment (its end); every tile further on it is 128 fewer.
+    int own_cols[2];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      row[e] = qblk * TC_BM + lane0 + (lane >> 2) + 8 * e;
-      lim[e] = p.pos + min(row[e], p.q_len - 1) + 1;
-    }
+    for (int e = 0; e < 2; ++e)
+      own_cols[e] = p.pos + min(at.t0 + p.pack.div(lane0 + (lane >> 2) + 8 * e), p.q_len - 1) + 1 + (Tp - g0) * TC_BN;
+    const int front_cols = p.prefix_len - g0 * TC_BN;
     const float c = p.scale_log2;
     float m_ref[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
     float mxs[2];
@@ -303,8 +317,8 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     auto tile_masked = [&](int j) {  // warp-uniform; fills nvalid
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const int g = g0 + j;
-        nvalid[e] = g < Tp ? p.prefix_len - g * TC_BN : lim[e] - (g - Tp) * TC_BN;
+        const int front = front_cols - j * TC_BN;
+        nvalid[e] = front > 0 ? front : own_cols[e] - j * TC_BN;
       }
       return __any_sync(0xffffffffu, nvalid[0] < TC_BN || nvalid[1] < TC_BN) != 0;
     };
@@ -360,6 +374,7 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       inv[e] = 1.f / l[e];
     }
     if constexpr (SPLIT) {
+      const int work = known_here(blockIdx.x) / C, crank = static_cast<int>(cluster_ctarank());
       // ---- this CTA's unnormalised partial -> scratch, in fragment order ([column step][thread] float4, so that every
       // store of a warp writes 512 contiguous bytes), and (m, l) per row
       float4* gpart = reinterpret_cast<float4*>(p.scratch) + (static_cast<size_t>(work) * C + crank) * FRAG_PART_F4<D>;
@@ -385,41 +400,11 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         for (int e = 0; e < 2; ++e) gml[lane0 + (lane >> 2) + 8 * e] = make_float2(T > 0 ? m_ref[e] : -INFINITY, l[e]);
       }
       __threadfence();  // visible to the cluster before its barrier is passed
-    } else {
-      // ---- output: O / l straight from the fragments (a row's four threads write 32 contiguous bytes per repeat)
-#pragma unroll
-      for (int hh = 0; hh < Cfg::PANELS; ++hh) {
-        uint32_t o[32];
-        tmem_ld_16x256b_x8(tO + hh * 64, o);
-        tc_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          if (!ok || row[e] >= p.q_len) continue;
-          float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row[e]) * p.q_heads + h) * D + hh * 64 + col0;
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            *reinterpret_cast<float2*>(dst + 8 * k) =
-                make_float2(__uint_as_float(o[4 * k + 2 * e]) * inv[e], __uint_as_float(o[4 * k + 2 * e + 1]) * inv[e]);
-        }
-      }
-      if (ok && p.lse && (lane & 3) == 0) {
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-          if (row[e] < p.q_len)
-            p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row[e]] =
-                (m_ref[e] + log2f(l[e])) * 0.69314718055994530942f;
-      }
-    }
-  } else {
-    reg_dec<Cfg::REGS_OTHER>();  // the idle warp of the third warpgroup: the re-division is a warpgroup's decision
-  }
-
-  if constexpr (SPLIT) {
-    // ---- merge over the cluster.  Every thread of every CTA comes through here, whatever happened above.  CTA r
-    // finishes the fragments of the softmax threads [256 r / C, 256 (r + 1) / C), i.e. the rows of 8 / C warps: thread t
-    // of them every C-th column step, all loads in flight at once; the sums run in CTA order.
-    cluster_sync_all();  // release / acquire over the cluster: the partials of every CTA are visible
-    if (warp < Cfg::SOFTMAX_WARPS) {
+      cluster_sync_all();  // release / acquire over the cluster: the partials of every CTA are visible
+      // ---- merge over the cluster (here and not behind the role branches, where the code would have to make do with the
+      // other roles' registers).  CTA r finishes the fragments of the softmax threads [256 r / C, 256 (r + 1) / C), i.e.
+      // the rows of 8 / C warps: thread t of them every C-th column step, all loads in flight at once; the sums run in
+      // CTA order.
       const bool cta_ok = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;  // nobody gave up on a wait
       constexpr int PER = 256 / C, STEPS = D / 8, MINE = STEPS / C;
       const int sub = threadIdx.x / PER, t = PER * crank + threadIdx.x % PER;
@@ -453,8 +438,15 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
         for (int cr = 0; cr < C; ++cr) wgt[e][cr] *= inv;
       }
-      const int row0 = qblk * TC_BM + r0;
-      float* dst = p.out + ((static_cast<int64_t>(b) * p.q_len + row0) * p.q_heads + h) * D + 2 * (l_t & 3);
+      int tok[2], hd[2];
+      float* dst[2];
+      const Place at = place(known_here(blockIdx.x) / C);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        tok[e] = at.t0 + p.pack.divmod(known_here(r0 + 8 * e), hd[e]);
+        hd[e] += at.h0;
+        dst[e] = p.out + ((static_cast<int64_t>(at.b) * p.q_len + tok[e]) * p.q_heads + hd[e]) * D + 2 * (l_t & 3);
+      }
 #pragma unroll
       for (int u = 0; u < MINE; ++u) {
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -466,19 +458,56 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           acc.w = fmaf(wgt[1][cr], v[u][cr].w, acc.w);
         }
         const int col = 8 * (u * C + sub);
-        if (cta_ok && row0 < p.q_len) *reinterpret_cast<float2*>(dst + col) = make_float2(acc.x, acc.y);
-        if (cta_ok && row0 + 8 < p.q_len)
-          *reinterpret_cast<float2*>(dst + static_cast<int64_t>(8) * p.q_heads * D + col) = make_float2(acc.z, acc.w);
+        if (cta_ok && tok[0] < at.t1) *reinterpret_cast<float2*>(dst[0] + col) = make_float2(acc.x, acc.y);
+        if (cta_ok && tok[1] < at.t1) *reinterpret_cast<float2*>(dst[1] + col) = make_float2(acc.z, acc.w);
       }
       if (cta_ok && p.lse && sub == 0 && (l_t & 3) == 0) {
 #pragma unroll
         for (int e = 0; e < 2; ++e)
-          if (row0 + 8 * e < p.q_len)
-            p.lse[(static_cast<int64_t>(b) * p.q_heads + h) * p.q_len + row0 + 8 * e] =
+          if (tok[e] < at.t1)
+            p.lse[(static_cast<int64_t>(at.b) * p.q_heads + hd[e]) * p.q_len + tok[e]] =
                 (m[e] + log2f(lsum[e])) * 0.69314718055994530942f;
       }
+    } else {
+      // ---- output: O / l straight from the fragments (a row's four threads write 32 contiguous bytes per repeat)
+      int tok[2], hd[2];  // token and head of this thread's rows
+      float* dst[2];
+      const Place at = place(known_here(blockIdx.x) / C);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        tok[e] = at.t0 + p.pack.divmod(known_here(lane0 + (lane >> 2) + 8 * e), hd[e]);
+        hd[e] += at.h0;
+        dst[e] = p.out + ((static_cast<int64_t>(at.b) * p.q_len + tok[e]) * p.q_heads + hd[e]) * D + col0;
+      }
+#pragma unroll
+      for (int hh = 0; hh < Cfg::PANELS; ++hh) {
+        uint32_t o[32];
+        tmem_ld_16x256b_x8(tO + hh * 64, o);
+        tc_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          if (!ok || tok[e] >= at.t1) continue;
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            *reinterpret_cast<float2*>(dst[e] + hh * 64 + 8 * k) =
+                make_float2(__uint_as_float(o[4 * k + 2 * e]) * inv[e], __uint_as_float(o[4 * k + 2 * e + 1]) * inv[e]);
+        }
+      }
+      if (ok && p.lse && (lane & 3) == 0) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (tok[e] < at.t1)
+            p.lse[(static_cast<int64_t>(at.b) * p.q_heads + hd[e]) * p.q_len + tok[e]] =
+                (m_ref[e] + log2f(l[e])) * 0.69314718055994530942f;
+      }
     }
+  } else {
+    reg_dec<Cfg::REGS_OTHER>();  // the idle warp of the third warpgroup: the re-division is a warpgroup's decision
   }
+
+  // (every thread of every CTA passes the cluster's barrier, whatever happened above)
+  if constexpr (SPLIT)
+    if (warp >= Cfg::SOFTMAX_WARPS) cluster_sync_all();
 
   // ---- tear-down
   tc_fence_before();

@@ -21,13 +21,13 @@ def ctx():
 
 @pytest.mark.parametrize("D", [128, 64])
 @pytest.mark.parametrize("B,Hq,Hkv,parts", [
-    (1, 6, 2, [126, 42, 43, 300]),           # groups of 3
+    (1, 6, 2, [126, 42, 43, 300]),           # groups of 3: 42 tokens x 3 heads, K/V and query tiles do not align
     (1, 10, 2, [25, 26, 100, 420]),          # groups of 5
-    (2, 8, 1, [15, 16, 17, 129]),            # groups of 8
-    (1, 65, 1, [3, 70]),                     # a group larger than half a tile
+    (2, 8, 1, [15, 16, 17, 129]),            # groups of 8: 16 tokens per tile
+    (1, 65, 1, [3, 70]),                     # a group that only packs whole or by 5 and 13
     (1, 4, 4, [1, 500, 64, 2100, 64]),       # no group: 8 CTAs share the long walks, short ones stay whole
     (1, 16, 4, [700, 60, 1400, 100]),        # clusters of several sizes as the walk grows
-    (3, 32, 8, [150, 150, 333]),             # pairs of query tiles, several waves
+    (3, 32, 8, [150, 150, 333]),             # pairs of packed tiles, several waves
 ])
 def test_layouts(ctx, D, B, Hq, Hkv, parts):
     S = sum(parts)

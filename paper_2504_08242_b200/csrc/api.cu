@@ -279,6 +279,18 @@ jupiter_status jupiter_branch_prefill_attn(jupiter_ctx* ctx, const void* q, cons
   return e == cudaSuccess ? JUPITER_OK : cuda_fail(ctx, e, "branch_prefill_attn");
 }
 
+// Few stacked rows per kv head stream through clusters, many go to the tensor cores: by the estimates where both can take
+// the call.  (Needs the device current.)
+static bool prefer_stream(const jupiter_ctx* ctx, bool tc_ok, int n_branches, int q_heads, const CacheView& sfx, int q_len,
+                          int prefix_len, int max_suffix_len, int layers) {
+  if (!tc_ok) return jup::branch_stream_preferred(n_branches, q_heads, sfx.kv_heads, q_len, ctx->sm_count);
+  layers = layers < jup::kBranchMaxLayersPerLaunch ? layers : jup::kBranchMaxLayersPerLaunch;
+  return jup::branch_stream_estimate_ns(n_branches, q_heads, sfx.kv_heads, q_len, sfx.head_dim, prefix_len, max_suffix_len,
+                                        layers, ctx->sm_count) <=
+         jup::branch_tc_estimate_ns(n_branches, q_heads, sfx.kv_heads, q_len, sfx.head_dim, prefix_len, max_suffix_len, layers,
+                                    ctx->sm_count);
+}
+
 static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const jupiter_kv_cache* prefix,
                                        int32_t prefix_len, const jupiter_kv_cache* suffix,
                                        const int32_t* d_suffix_len, const uint32_t* d_tree_mask,
@@ -304,8 +316,8 @@ static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const ju
   if (!jup::scale_ok(scale)) return JUPITER_ERR_INVALID_ARG;
   if (max_suffix_len < q_len || max_suffix_len > sfx.capacity) return JUPITER_ERR_OUT_OF_RANGE;
   if (!aligned16(q) || !aligned16(out)) return JUPITER_ERR_ALIGNMENT;
-  // which kernel: few stacked rows per kv head stream through clusters (no scratch); many rows with head_dim 128 go
-  // to the tensor-core kernel (which adapts to the scratch it is given); the rest to the split-KV kernel, the only one that can find the
+  // which kernel: few stacked rows per kv head stream through clusters (no scratch); many rows go to the tensor-core
+  // kernel (which adapts to the scratch it is given); the rest to the split-KV kernel, the only one that can find the
   // scratch too small
   DeviceGuard guard(ctx->device);
   const bool tc_ok = jup::branch_tc_supported(sfx, n_branches, q_heads, q_len, scale);
@@ -318,7 +330,7 @@ static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const ju
       use_stream = false, use_tc = true;
       break;
     default:
-      use_stream = jup::branch_stream_preferred(n_branches, q_heads, sfx.kv_heads, q_len, ctx->sm_count);
+      use_stream = prefer_stream(ctx, tc_ok, n_branches, q_heads, sfx, q_len, prefix_len, max_suffix_len, 1);
       use_tc = !use_stream && tc_ok;
   }
   if (!use_stream && !use_tc &&
@@ -388,10 +400,11 @@ jupiter_status jupiter_branch_append_attn_layers(jupiter_ctx* ctx, const jupiter
     t[l] = jup::BranchLayerTensors{static_cast<const bf16*>(L.q), static_cast<const bf16*>(L.k_new),
                                    static_cast<const bf16*>(L.v_new), pfx.k, pfx.v, sfx.k, sfx.v, L.out, L.lse};
   }
-  const bool stream_kernel = jup::branch_stream_preferred(n_branches, q_heads, sfx0.kv_heads, q_len, ctx->sm_count);
-  if (ctx->branch_kernel == JUPITER_BRANCH_AUTO &&
-      (stream_kernel || jup::branch_tc_supported(sfx0, n_branches, q_heads, q_len, scale))) {
-    DeviceGuard guard(ctx->device);
+  DeviceGuard guard(ctx->device);
+  const bool tc_ok = jup::branch_tc_supported(sfx0, n_branches, q_heads, q_len, scale);
+  const bool stream_kernel =
+      prefer_stream(ctx, tc_ok, n_branches, q_heads, sfx0, q_len, prefix_len, max_suffix_len, n_layers);
+  if (ctx->branch_kernel == JUPITER_BRANCH_AUTO && (stream_kernel || tc_ok)) {
     jup::LaunchInfo li{ctx->sm_count, 0};
     cudaError_t e;
     if (stream_kernel)

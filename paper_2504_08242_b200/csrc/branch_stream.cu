@@ -83,8 +83,7 @@ struct StreamCfg {
   static constexpr int SMEM_BYTES = Q_BYTES + PART_BYTES + NW * RING_BYTES;
 };
 
-// Launch shape: warps per CTA, ring slots per warp, CTAs that fit one SM with that much shared memory.
-constexpr int kStreamWarps = 8, kStreamStages = 2, kStreamCtasPerSm = 1;
+constexpr int kStreamStages = 2;  // ring slots per warp
 
 __device__ __forceinline__ void st_cluster_f4(uint32_t addr, float4 v) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
@@ -96,8 +95,8 @@ __device__ __forceinline__ void st_cluster_f2(uint32_t addr, float2 v) {
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-template <int D, int NW, int ST>
-__global__ void __launch_bounds__(NW * 32, kStreamCtasPerSm)
+template <int D, int NW, int ST, int PER_SM>
+__global__ void __launch_bounds__(NW * 32, PER_SM)
 branch_stream_kernel(const StreamParams p_in, const __grid_constant__ StreamLayers layers) {
   StreamParams p = p_in;
   if (layers.n > 0) {
@@ -505,24 +504,54 @@ branch_stream_kernel(const StreamParams p_in, const __grid_constant__ StreamLaye
   // nothing touches a peer's shared memory after the barrier above, so CTAs may leave independently
 }
 
-template <int D, int NW, int ST>
-static cudaError_t launch_stream_d(const StreamParams& p, const StreamLayers& layers, int units, cudaStream_t st,
-                                   LaunchInfo& li) {
-  using Cfg = StreamCfg<D, NW, ST>;
-  static PerDeviceOnce attr_done;
-  if (!attr_done.done()) {
-    cudaError_t e = cudaFuncSetAttribute(branch_stream_kernel<D, NW, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         Cfg::SMEM_BYTES);
+template <int D, int NW, int PER_SM>
+struct StreamKernel {
+  using Cfg = StreamCfg<D, NW, kStreamStages>;
+  static constexpr auto kernel = branch_stream_kernel<D, NW, kStreamStages, PER_SM>;
+  static cudaError_t set_attributes() {
+    static PerDeviceOnce attr_done;
+    if (attr_done.done()) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(branch_stream_kernel<D, NW, ST>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_done.set();
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) attr_done.set();
+    return e;
   }
-  li.launches += 1;
-  return launch_pdl_cluster(branch_stream_kernel<D, NW, ST>,
-                            dim3(static_cast<unsigned>(units * p.cluster), static_cast<unsigned>(layers.n > 0 ? layers.n : 1)),
-                            dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, static_cast<unsigned>(p.cluster), p, layers);
+  static int resident_clusters(int c) {
+    static ResidentClusters clusters;
+    if (set_attributes() != cudaSuccess) return 0;
+    return clusters.get(reinterpret_cast<const void*>(kernel), c, Cfg::THREADS, Cfg::SMEM_BYTES);
+  }
+  static cudaError_t launch(const StreamParams& p, const StreamLayers& layers, int units, cudaStream_t st, LaunchInfo& li) {
+    cudaError_t e = set_attributes();
+    if (e != cudaSuccess) return e;
+    li.launches += 1;
+    return launch_pdl_cluster(kernel,
+                              dim3(static_cast<unsigned>(units * p.cluster), static_cast<unsigned>(layers.n > 0 ? layers.n : 1)),
+                              dim3(Cfg::THREADS), Cfg::SMEM_BYTES, st, static_cast<unsigned>(p.cluster), p, layers);
+  }
+};
+
+// The launch shape for `problems` (unit, layer) pairs of `chunks` 16-key chunks each.
+//  - While all of them run at once: 8 warps per CTA and the largest cluster whose CTAs are all resident (and get six chunks
+//    for their eight warps at least).
+//  - More of them than SMs: one CTA of 4 warps each, two on an SM, so that one CTA's first loads and its merge overlap the other's
+//    stream, and no cluster has to exchange anything.
+// Measured (us a call): 16 layers x 32 kv heads (prefix 1024, 8 branches) with clusters of four CTAs of 8 warps per layer,
+// as a single layer takes them, 152, one CTA of 8 warps 106, one of 4 warps 100, two of 4 warps 108; 8 layers x 16 kv heads with
+// clusters of 8 : 4 : 2 : 1 CTAs 53 : 35 : 26 : 21; 8 layers x 2 kv heads, where clusters of 8 are not all resident,
+// 16 : 12 : 18 : 29; 1 layer x 16 kv heads of 26 chunks 11 : 6.3 : 7.3 : 9.7.
+struct StreamShape {
+  bool narrow;
+  int cluster_log2;
+};
+template <int D>
+static StreamShape stream_shape(int64_t problems, int64_t chunks, int sm_count) {
+  if (problems > sm_count) return {true, 0};
+  for (int lg = 3; lg > 0; --lg)
+    if (chunks >= (6 << lg) && (problems << lg) <= sm_count && StreamKernel<D, 8, 1>::resident_clusters(1 << lg) >= problems)
+      return {false, lg};
+  return {false, 0};
 }
 
 bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_len, int sm_count) {
@@ -531,6 +560,25 @@ bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_le
   // kernel with 32-row tiles takes over.
   const int64_t tiles = (static_cast<int64_t>(n_branches) * q_len * (q_heads / kv_heads) + 15) / 16;
   return tiles == 1 || tiles * kv_heads <= sm_count;
+}
+
+// A warp takes 1.13 us per chunk (0.73 with head_dim 64) while every SM is streaming, whatever the split; the rest of a
+// launch is about 6 us.  Measured (us, estimate in brackets): 8 kv heads, prefix 4000, 64 rows 15.6 (15), 128 rows 24.8 (25),
+// 192 rows 42.8 (44); prefix 1000, 192 rows 16.6 (16); 32 kv heads, 128 rows (two waves) 77 (79).
+int64_t branch_stream_estimate_ns(int n_branches, int q_heads, int kv_heads, int q_len, int head_dim, int prefix_len,
+                                  int max_suffix_len, int layers, int sm_count) {
+  const int nG = q_len * (q_heads / kv_heads);
+  const int64_t tiles = (static_cast<int64_t>(n_branches) * nG + 15) / 16, problems = tiles * kv_heads * layers;
+  const int64_t suffix_chunks = (max_suffix_len + 15) / 16;
+  const int64_t shape_chunks = (prefix_len + 15) / 16 + suffix_chunks;
+  const StreamShape sh = head_dim == 128 ? stream_shape<128>(problems, shape_chunks, sm_count)
+                                         : stream_shape<64>(problems, shape_chunks, sm_count);
+  const int64_t branches_here = std::min<int64_t>(n_branches, std::max(1, 16 / nG));
+  const int64_t chunks = (prefix_len + 15) / 16 + branches_here * ((suffix_chunks * 6 + 9) / 10);  // (mean lengths at 0.6 of the bound)
+  const int64_t warps = sh.narrow ? 4 : 8 << sh.cluster_log2;
+  const int64_t at_once = sh.narrow ? 2 * sm_count : problems;
+  const int64_t waves = (problems + at_once - 1) / at_once;
+  return 6000 + waves * ((chunks + warps - 1) / warps) * (head_dim == 128 ? 1130 : 730);
 }
 
 static cudaError_t launch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,
@@ -558,16 +606,16 @@ static cudaError_t launch_stream(const bf16* q, const CacheView& prefix, int pre
   p.out = out;
   p.lse = lse;
   const int units = suffix.kv_heads * p.row_tiles;
-  // the largest portable cluster that keeps every CTA (of one problem) resident at once
-  int c = 1;
-  while (c < 8 && units * c * 2 <= li.sm_count * kStreamCtasPerSm) c *= 2;
-  // no more CTAs than 16-key chunks of work per unit warrant
+  const int64_t problems = static_cast<int64_t>(units) * (layers.n > 0 ? layers.n : 1);
   const int64_t chunks = (prefix_len + 15) / 16 + static_cast<int64_t>(max_suffix_len + 15) / 16;
-  while (c > 1 && chunks < static_cast<int64_t>(c) * 8) c /= 2;
-  p.cluster = c;
-  p.cluster_log2 = c == 8 ? 3 : (c == 4 ? 2 : (c == 2 ? 1 : 0));
-  if (suffix.head_dim == 128) return launch_stream_d<128, kStreamWarps, kStreamStages>(p, layers, units, st, li);
-  return launch_stream_d<64, kStreamWarps, kStreamStages>(p, layers, units, st, li);
+  auto launch = [&](auto wide, auto narrow, const StreamShape& sh) {
+    p.cluster = 1 << sh.cluster_log2;
+    p.cluster_log2 = sh.cluster_log2;
+    return sh.narrow ? narrow.launch(p, layers, units, st, li) : wide.launch(p, layers, units, st, li);
+  };
+  if (suffix.head_dim == 128)
+    return launch(StreamKernel<128, 8, 1>(), StreamKernel<128, 4, 2>(), stream_shape<128>(problems, chunks, li.sm_count));
+  return launch(StreamKernel<64, 8, 1>(), StreamKernel<64, 4, 2>(), stream_shape<64>(problems, chunks, li.sm_count));
 }
 
 cudaError_t launch_branch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,

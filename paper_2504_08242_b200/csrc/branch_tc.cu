@@ -36,7 +36,6 @@
 // All mbarrier waits are bounded; on expiry the CTA sets the status word, drains its own copies and MMAs,
 // frees TMEM and returns (every thread still passes the cluster barriers).
 #include <algorithm>
-#include <atomic>
 
 #include "host_checks.h"
 #include "kernels.h"
@@ -734,6 +733,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
 struct BtPlan {
   int row_tiles, branches_per_tile, slices_per_branch, box_tokens, units, ctas_per_unit;
   bool ok;
+  int64_t estimate_ns;
 };
 
 template <int D, int NL>
@@ -752,43 +752,20 @@ static cudaError_t bt_set_attributes() {
 // How many clusters of c CTAs of the kernel can be resident at once on the current device (0 if the query fails).
 template <int D, int NL>
 static int bt_resident_clusters(int c) {
-  static std::atomic<int> cache[64][BT_MAX_CTAS + 1];  // per device and cluster size: 0 = not asked yet, else answer + 1
-  int dev = -1;
-  if (c < 1 || c > BT_MAX_CTAS || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  const int cached = cache[dev][c].load(std::memory_order_acquire);
-  if (cached > 0) return cached - 1;
-  int n = 0;
-  if (bt_set_attributes<D, NL>() == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(c * 64));
-    cfg.blockDim = dim3(BT_THREADS);
-    cfg.dynamicSmemBytes = BtCfg<D>::SMEM_BYTES;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(c);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, branch_tc_kernel<D, NL>, &cfg) == cudaSuccess) n = got;
-    else (void)cudaGetLastError();
-  } else {
-    (void)cudaGetLastError();
-  }
-  cache[dev][c].store(n + 1, std::memory_order_release);
-  return n;
+  static ResidentClusters clusters;
+  if (bt_set_attributes<D, NL>() != cudaSuccess) return 0;
+  return clusters.get(reinterpret_cast<const void*>(branch_tc_kernel<D, NL>), c, BT_THREADS, BtCfg<D>::SMEM_BYTES);
 }
 
 // The tiling of one problem and the CTAs per unit, for `layers` problems in one launch: the pair with the shortest
-// estimated time.  A CTA costs its tiles (of 128 keys; a branch's suffix counted at 0.6 of its longest possible walk) plus
-// a fixed time, larger when a cluster has to exchange partials; more, smaller row tiles walk the prefix more often but
-// may fill the machine better.
-constexpr int BT_FIXED_ALONE = 6, BT_FIXED_CLUSTER = 10;  // in tiles
+// estimated time.  A CTA takes 1.55 us per tile of 128 keys (1.2 with head_dim 64; a branch's suffix counted at 0.6 of its
+// longest possible walk) and a fixed time, larger when a cluster has to exchange partials; more, smaller row tiles walk
+// the prefix more often but may fill the machine better.
+constexpr int BT_FIXED_ALONE = 10, BT_FIXED_CLUSTER = 15;  // in half tiles
 template <int D, int NL>
 static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_heads, int kv_heads, int q_len,
                       int sm_count, int layers) {
-  BtPlan pl = {0, 0, 1, 0, 0, 1, false};
+  BtPlan pl = {0, 0, 1, 0, 0, 1, false, 0};
   const int G = q_heads / kv_heads, nG = q_len * G;
   const int64_t Tp = (static_cast<int64_t>(prefix_len) + BT_BN - 1) / BT_BN;
   const int64_t ts_max = (max_suffix_len + BT_BN - 1) / BT_BN;
@@ -803,10 +780,11 @@ static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_
       const int64_t at_once = c == 1 ? sm_count : bt_resident_clusters<D, NL>(c);
       if (at_once == 0 || (c > 1 && at_once < units)) continue;  // (a layer's clusters are all resident at once)
       const int64_t waves = (units * layers + at_once - 1) / at_once;
-      const int64_t est = waves * ((walk + c - 1) / c + (c > 1 ? BT_FIXED_CLUSTER : BT_FIXED_ALONE));
+      const int64_t est = waves * (2 * ((walk + c - 1) / c) + (c > 1 ? BT_FIXED_CLUSTER : BT_FIXED_ALONE));
       if (best < 0 || est < best) {
         best = est;
-        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, true};
+        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, true,
+                    est * (D == 128 ? 775 : 600)};
       }
     }
   };
@@ -839,6 +817,17 @@ bool branch_tc_supported(const CacheView& suffix, int n_branches, int q_heads, i
   if (nG > BT_BM && BT_BM % G != 0) return false;
   const int64_t tiles = nG > BT_BM ? static_cast<int64_t>(n_branches) * ((nG + BT_BM - 1) / BT_BM) : n_branches;
   return tiles * suffix.kv_heads <= (1 << 30);
+}
+
+int64_t branch_tc_estimate_ns(int n_branches, int q_heads, int kv_heads, int q_len, int head_dim, int prefix_len,
+                              int max_suffix_len, int layers, int sm_count) {
+  const bool batched = layers >= BT_MIN_BATCHED_LAYERS;
+  auto estimate = [&](auto plan) {
+    const BtPlan pl = plan(prefix_len, max_suffix_len, n_branches, q_heads, kv_heads, q_len, sm_count, batched ? layers : 1);
+    return pl.ok ? pl.estimate_ns * (batched ? 1 : layers) : INT64_MAX;
+  };
+  if (head_dim == 128) return batched ? estimate(bt_plan<128, kBranchMaxLayersPerLaunch>) : estimate(bt_plan<128, 1>);
+  return batched ? estimate(bt_plan<64, kBranchMaxLayersPerLaunch>) : estimate(bt_plan<64, 1>);
 }
 
 template <int D, int NL>

@@ -62,4 +62,38 @@ class PerDeviceOnce {
   std::atomic<bool> flags_[kMax] = {};
 };
 
+// How many thread-block clusters of c CTAs of one kernel can be resident at once on the current device: asked once per
+// device and cluster size, 0 if the query fails.  One object per kernel, whose shared-memory attribute must be set.
+class ResidentClusters {
+ public:
+  int get(const void* kernel, int c, int threads, size_t smem) {
+    int dev = -1;
+    if (c < 1 || c > kMaxSize || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    const int cached = cache_[dev][c].load(std::memory_order_acquire);
+    if (cached > 0) return cached - 1;  // 0: not asked yet, else answer + 1
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(c * 64));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      n = 0;
+    }
+    cache_[dev][c].store(n + 1, std::memory_order_release);
+    return n;
+  }
+
+ private:
+  static constexpr int kMaxDevices = 64, kMaxSize = 8;
+  std::atomic<int> cache_[kMaxDevices][kMaxSize + 1] = {};
+};
+
 }  // namespace jup

@@ -106,6 +106,11 @@ struct BranchLayerTensors {
 // through distributed shared memory; no scratch.  Preferred when all stacked rows of a kv head fit one 16-row tile, or
 // when the (kv head, 16-row tile) units all run at once.
 bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_len, int sm_count);
+// Estimated time of a launch for `layers` layers on either kernel, for the choice between them where both can take a call.
+int64_t branch_stream_estimate_ns(int n_branches, int q_heads, int kv_heads, int q_len, int head_dim, int prefix_len,
+                                  int max_suffix_len, int layers, int sm_count);
+int64_t branch_tc_estimate_ns(int n_branches, int q_heads, int kv_heads, int q_len, int head_dim, int prefix_len,
+                              int max_suffix_len, int layers, int sm_count);
 cudaError_t launch_branch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,
                                  const int32_t* d_suffix_len, const uint32_t* d_tree_mask, int max_suffix_len,
                                  int n_branches, int q_heads, int q_len, float scale, float* out, float* lse,

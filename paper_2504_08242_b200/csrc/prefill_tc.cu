@@ -28,7 +28,6 @@
 // TMEM and returns.
 #include "host_checks.h"
 #include <algorithm>
-#include <atomic>
 
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -469,32 +468,9 @@ static cudaError_t launch_frag(int64_t units, cudaStream_t st, const CUtensorMap
 // How many clusters of C CTAs of the fragment form can be resident at once on the current device (0 if the query fails).
 template <int D, int C>
 static int frag_resident_clusters() {
-  static std::atomic<int> cache[64];  // per device: 0 = not asked yet, else answer + 1
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  const int cached = cache[dev].load(std::memory_order_acquire);
-  if (cached > 0) return cached - 1;
-  int n = 0;
-  if (frag_set_attributes<D, C>() == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C * 64);
-    cfg.blockDim = dim3(FragCfg<D>::THREADS);
-    cfg.dynamicSmemBytes = FragCfg<D>::SMEM_BYTES;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int got = 0;
-    if (cudaOccupancyMaxActiveClusters(&got, prefill_frag_kernel<D, C>, &cfg) == cudaSuccess) n = got;
-    else (void)cudaGetLastError();
-  } else {
-    (void)cudaGetLastError();
-  }
-  cache[dev].store(n + 1, std::memory_order_release);
-  return n;
+  static ResidentClusters clusters;
+  if (frag_set_attributes<D, C>() != cudaSuccess) return 0;
+  return clusters.get(reinterpret_cast<const void*>(prefill_frag_kernel<D, C>), C, FragCfg<D>::THREADS, FragCfg<D>::SMEM_BYTES);
 }
 
 template <int D>

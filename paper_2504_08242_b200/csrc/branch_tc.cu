@@ -2,7 +2,7 @@
 // Fig. 7 step 3: the k draft tokens of every request are verified in one pass; Sec. V-B, Fig. 8: all
 // point-extending requests share the prompt's KVCache).
 //
-// head_dim 128.  The stacked rows of a kv head -- (branch, draft token, head of the group), in that order -- are
+// The stacked rows of a kv head -- (branch, draft token, head of the group), in that order -- are
 // cut into row tiles of at most 128 rows: whole branches while a branch has at most 128 rows (the same number
 // of branches in every tile, so that the tiles carry equal work), else 128-row slices of one branch.
 // A unit = (kv head, row tile).  Every row belongs to one branch and may see the shared prefix plus that
@@ -11,7 +11,7 @@
 // in tiles of 128 keys: a prefix tile is visible to every row, a suffix tile to the rows of its branch below
 // their causal limit (or tree mask).  A prefix K/V tile is therefore fetched once per row tile, not once per branch.
 //
-// `ctas_per_unit` CTAs, a thread-block cluster, share a unit: the prefix tiles are cut into equal contiguous
+// C CTAs, a thread-block cluster, share a unit: the prefix tiles are cut into equal contiguous
 // ranges, one per CTA, and so are the suffix tiles (the prefix share does not depend on the device-side lengths,
 // so its first loads are in flight while the lengths arrive).  Inside a CTA:
 //   loader warp  : TMA (tiled, 128-byte swizzle) Q once -- one box [tokens][G heads][64] lands in stacked-row
@@ -50,20 +50,19 @@ constexpr int BT_BN = 128;             // keys per KV tile
 constexpr int BT_PANEL_BYTES = 16384;  // 128 rows x 64 elements
 constexpr int BT_KV_STAGES = 3;
 constexpr int BT_MAX_BRANCHES = 32;    // branches in one row tile
-constexpr int BT_MAX_CTAS = 8;         // CTAs per unit (the portable cluster size)
 constexpr int BT_ML_FLOATS = BT_BM * 2;  // one CTA's (m, l) pairs
 // Layers of one call share a launch from this many on.
 constexpr int BT_MIN_BATCHED_LAYERS = 3;
 
 struct BtParams {
   int n_branches, q_len, q_heads, group, kv_heads;
+  FastDiv by_group, by_q_len, by_row_tiles;
   int prefix_len, max_suffix_len;
   int row_tiles;          // row tiles per kv head
   int branches_per_tile;  // whole branches per row tile (slices_per_branch == 1)
   int slices_per_branch;  // > 1: a branch has more than 128 rows and is cut into 128-row slices
   int box_tokens;         // tokens in the Q box
   int box_keys;           // keys in the box of the step's block: all of the row tile's branches
-  int ctas_per_unit;      // cluster size
   float scale_log2;
   long long wait_limit;
   const int32_t* d_suffix_len;
@@ -139,7 +138,8 @@ struct BtTile {
   __device__ __forceinline__ int groups() const { return (valid + 15) >> 4; }
 };
 
-template <int D, int NL>
+// C: cluster size = CTAs per unit.
+template <int D, int NL, int C>
 __global__ void __launch_bounds__(BT_THREADS, 1)
 branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) {
   using Cfg = BtCfg<D>;
@@ -162,9 +162,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   const long long wl = p.wait_limit;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int C = p.ctas_per_unit;
   const int unit = blockIdx.x / C, crank = blockIdx.x % C;  // clusters are consecutive CTAs: crank is the cluster rank
-  const int rt = unit % p.row_tiles, hk = unit / p.row_tiles;
+  int rt;
+  const int hk = p.by_row_tiles.divmod(unit, rt);
   const int gunit = blockIdx.y * (gridDim.x / C) + unit;  // over all layers of the launch
   const int n = p.q_len, G = p.group;
   // ---- the row tile: tokens [tok0, tok0 + ntok) of the stacked (branch, draft row) order, all heads of the group
@@ -289,9 +289,6 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     return BtTile{cursor, tile, min((fused ? len_s[cursor] - n : len_s[cursor]) - tile * BT_BN, BT_BN)};
   };
   const int T[2] = {(Tall + 1) >> 1, Tall >> 1};  // stream x takes the sequence numbers 2 i + x
-
-  // a softmax thread's state after its last tile, kept for the merge behind the role branches
-  float fin_m = -INFINITY, fin_l = 0.f, fin_w_own = 0.f, fin_w_oth = 0.f;
 
   if (warp == BT_LOADER_WARP) {
     // =============================================================== loader
@@ -438,8 +435,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const int x = warp >> 2;
     const int row_in_tile = (warp & 3) * 32 + lane;
     const bool row_valid = row_in_tile < rows_here;
-    const int tok = tok0 + row_in_tile / G;          // token (branch, draft row) of this row
-    const int rb = tok / n, ri = tok % n;
+    int ri;
+    const int rb = p.by_q_len.divmod(tok0 + p.by_group.div(row_in_tile), ri);  // branch and draft row of this row
     const int rj = row_valid ? rb - b_first : -1;    // the row's branch as an index into the tile's branches
     // draft rows of the block this row may see, as bits: its ancestors and itself (a chain: rows 0..i)
     const uint32_t tm = !row_valid ? 0u
@@ -464,7 +461,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       const BtTile e = tile_at(2 * j + x, cursor);
       const int key0 = e.tile * BT_BN;
       ColumnBits allow = {0u, 0u, 0u, 0u};
-      bool warp_sees = (warp & 3) * 32 < rows_here, masked = false;  // a whole prefix tile is seen by every row there is
+      // a whole prefix tile is seen by every row there is
+      bool row_sees = true, warp_sees = (warp & 3) * 32 < rows_here, masked = false;
       if (e.seg != BT_PREFIX || e.valid < BT_BN) {
         // by 32-column words: the first `cnt` columns, and the block's rows by the mask from column `col` on (which may
         // lie outside the tile)
@@ -488,9 +486,10 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         }
         if (!row_valid) cnt = 0, col = NONE;
         allow = ColumnBits{word(0, cnt, col), word(1, cnt, col), word(2, cnt, col), word(3, cnt, col)};
-        warp_sees = __any_sync(0xffffffffu, (allow.w0 | allow.w1 | allow.w2 | allow.w3) != 0u);
-        // (a row beyond the tile's rows sees nothing and nobody uses its scores)
-        masked = !__all_sync(0xffffffffu, !row_valid || (allow.w0 & allow.w1 & allow.w2 & allow.w3) == 0xffffffffu);
+        row_sees = (allow.w0 | allow.w1 | allow.w2 | allow.w3) != 0u;
+        warp_sees = __any_sync(0xffffffffu, row_sees);
+        // columns are only masked for the rows that see some of the tile but not all of it
+        masked = !__all_sync(0xffffffffu, !row_sees || (allow.w0 & allow.w1 & allow.w2 & allow.w3) == 0xffffffffu);
       }
       // (ok is the same in all lanes of a warp: the barriers and the tcgen05 operations are warp-collective)
       ok = __all_sync(0xffffffffu, ok && mbar_spin_wait(bar(BT_S_FULL + x), j & 1, abort_flag, p.status, wl));
@@ -502,7 +501,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         signal(NB_P_EARLY);
       };
       if (warp_sees) {
-        softmax_tile_row<true, D>(tS, tP, tO, j, (e.groups() + 1) >> 1, masked, allow, c, m_ref, l, test_o, wait_o,
+        softmax_tile_row<true, D>(tS, tP, tO, j, (e.groups() + 1) >> 1, masked, allow, row_sees, c, m_ref, l, test_o, wait_o,
                                   [&] { signal(NB_S_FREE); }, release_early);
       } else {  // no row of this warp sees the tile: P = 0, nothing else changes
         signal(NB_S_FREE);
@@ -551,138 +550,14 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const float2 oth = ml_of(1 - x)[row_in_tile];
     // a stream whose tiles were all hidden from this row has l = 0 and takes no part
     const float m_own = l > 0.f ? m_ref : -INFINITY, m_oth = oth.y > 0.f ? oth.x : -INFINITY;
-    fin_m = fmaxf(m_own, m_oth);
-    fin_w_own = l > 0.f ? fast_exp2(m_own - fin_m) : 0.f;
-    fin_w_oth = oth.y > 0.f ? fast_exp2(m_oth - fin_m) : 0.f;
-    fin_l = l * fin_w_own + oth.y * fin_w_oth;
-    if (C > 1) {
-      // ---- this CTA's partial of the row -> scratch, as [column chunk][row] float4 so that a warp writes 512
-      // contiguous bytes: columns [D/2 x, D/2 x + D/2) of both streams combined, unnormalised, relative to the row's
-      // maximum over this CTA's tiles
-      float4* gpart = reinterpret_cast<float4*>(p.part + (static_cast<size_t>(gunit) * C + crank) * Cfg::PART_FLOATS);
-      float2* gml = reinterpret_cast<float2*>(p.ml + (static_cast<size_t>(gunit) * C + crank) * BT_ML_FLOATS);
-      const bool has_own = Tx > 0, has_oth = T[1 - x] > 0;  // a stream without tiles never wrote its accumulator
-      if ((warp & 3) * 32 < rows_here) {  // warp-uniform (the TMEM loads are warp-collective): the warp has a row
-        const uint32_t tOwn = tmem + lane_base + BT_O_COL0 + x * 128 + x * (D / 2);
-        const uint32_t tOth = tmem + lane_base + BT_O_COL0 + (1 - x) * 128 + x * (D / 2);
-#pragma unroll
-        for (int q2 = 0; q2 < D / 64; ++q2) {
-          uint32_t o[32], o2[32];
-          if (has_own) tmem_ld32(tOwn + q2 * 32, o);
-          if (has_oth) tmem_ld32(tOth + q2 * 32, o2);
-          tc_wait_ld();
-#pragma unroll
-          for (int cc = 0; cc < 8; ++cc) {
-            float v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              v[i] = has_own ? __uint_as_float(o[4 * cc + i]) * fin_w_own : 0.f;
-              if (has_oth) v[i] = fmaf(__uint_as_float(o2[4 * cc + i]), fin_w_oth, v[i]);
-            }
-            if (row_valid) gpart[(x * (D / 8) + q2 * 8 + cc) * BT_BM + row_in_tile] = make_float4(v[0], v[1], v[2], v[3]);
-          }
-        }
-        if (row_valid && x == 0) gml[row_in_tile] = make_float2(fin_l > 0.f ? fin_m : -INFINITY, fin_l);
-      }
-      __threadfence();  // visible to the cluster before its barrier is passed
-    }
-  }
-
-  // ================================================================= output
-  // Every thread of every CTA comes through here, whatever happened above.
-  auto slice_begin = [&](int d) { return (BT_BM * d + C - 1) / C; };  // first row finished by CTA d of the cluster
-  if (C > 1) {
-    // ---- several CTAs per unit: behind the cluster barrier every CTA's partial is in the scratch (L2).  This CTA
-    // finishes the rows [128 crank / C, 128 (crank + 1) / C).  First the normalised weight of every (CTA, row)
-    // into shared memory, then (row, 16-byte column chunk) pairs dealt to the 256 threads with the row running
-    // fastest (a warp reads contiguous pieces of every partial; a pair's loads are issued together, two pairs at a
-    // time); the sums run in CTA order, so the result never depends on timing.
-    tc_fence_before();
-    cluster_sync_all();
-    if (warp < 8) {
-      const bool clean = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;  // nobody gave up on a wait
-      const float2* uml = reinterpret_cast<const float2*>(p.ml + static_cast<size_t>(gunit) * C * BT_ML_FLOATS);
-      const float4* upart = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(gunit) * C * Cfg::PART_FLOATS);
-      float* wtab = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);  // [CTA][row of my slice] (the rings are free)
-      const int row0 = slice_begin(crank), nrows = min(slice_begin(crank + 1), rows_here) - row0;
-      const int max_slice = (BT_BM + C - 1) / C;
-      if (static_cast<int>(threadIdx.x) < nrows) {
-        const int row = row0 + threadIdx.x;
-        float2 ml[BT_MAX_CTAS];
-#pragma unroll
-        for (int cr = 0; cr < BT_MAX_CTAS; ++cr)
-          ml[cr] = cr < C ? __ldcg(uml + cr * BT_BM + row) : make_float2(-INFINITY, 0.f);
-        float M = -INFINITY;
-#pragma unroll
-        for (int cr = 0; cr < BT_MAX_CTAS; ++cr)
-          if (ml[cr].y > 0.f) M = fmaxf(M, ml[cr].x);  // a CTA whose tiles were all hidden from the row has l = 0
-        float w[BT_MAX_CTAS], lall = 0.f;
-#pragma unroll
-        for (int cr = 0; cr < BT_MAX_CTAS; ++cr) {
-          w[cr] = ml[cr].y > 0.f ? fast_exp2(ml[cr].x - M) : 0.f;
-          lall = fmaf(w[cr], ml[cr].y, lall);
-        }
-        const float inv = 1.f / lall;
-#pragma unroll
-        for (int cr = 0; cr < BT_MAX_CTAS; ++cr)
-          if (cr < C) wtab[cr * max_slice + threadIdx.x] = w[cr] * inv;
-        if (clean && L_.lse) {
-          const int tok = tok0 + row / G, hq = hk * G + row % G;
-          L_.lse[(static_cast<int64_t>(tok / n) * p.q_heads + hq) * n + tok % n] = (M + log2f(lall)) * 0.69314718055994530942f;
-        }
-      }
-      named_sync(NB_MERGE, 256);
-      const int pairs = nrows * (D / 4);
-      for (int idx0 = threadIdx.x; idx0 < pairs; idx0 += 512) {
-        float4 t[2][BT_MAX_CTAS];
-        int ris[2], chunk[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int idx = min(idx0 + h * 256, pairs - 1);
-          ris[h] = idx % nrows;
-          chunk[h] = idx / nrows;
-#pragma unroll
-          for (int cr = 0; cr < BT_MAX_CTAS; ++cr)
-            if (cr < C)
-              t[h][cr] = __ldcg(upart + static_cast<size_t>(cr) * (Cfg::PART_FLOATS / 4) + chunk[h] * BT_BM + row0 + ris[h]);
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int cr = 0; cr < BT_MAX_CTAS; ++cr) {
-            if (cr >= C) continue;
-            const float w = wtab[cr * max_slice + ris[h]];
-            if (w == 0.f) continue;  // (also a CTA without tiles, whose partial holds nothing meaningful)
-            acc.x = fmaf(w, t[h][cr].x, acc.x);
-            acc.y = fmaf(w, t[h][cr].y, acc.y);
-            acc.z = fmaf(w, t[h][cr].z, acc.z);
-            acc.w = fmaf(w, t[h][cr].w, acc.w);
-          }
-          if (clean && idx0 + h * 256 < pairs) {
-            const int row = row0 + ris[h];
-            const int tok = tok0 + row / G, hq = hk * G + row % G;
-            *reinterpret_cast<float4*>(L_.out + (static_cast<int64_t>(tok) * p.q_heads + hq) * D + chunk[h] * 4) = acc;
-          }
-        }
-      }
-    }
-  } else {
-    // ---- one CTA per unit: the rows are staged in shared memory (every MMA and copy of the CTA is complete behind
-    // the barrier, so the K/V rings are free) and written out as whole 512-byte rows
-    float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);  // [row][Cfg::RECV_STRIDE]
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp < 8 && (warp & 3) * 32 < rows_here) {  // warp-uniform (the TMEM loads are warp-collective)
-      const int x = warp >> 2, row_in_tile = (warp & 3) * 32 + lane;
-      const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    const float fin_m = fmaxf(m_own, m_oth);
+    float w_own = l > 0.f ? fast_exp2(m_own - fin_m) : 0.f, w_oth = oth.y > 0.f ? fast_exp2(m_oth - fin_m) : 0.f;
+    const float fin_l = l * w_own + oth.y * w_oth;
+    // columns [D/2 x, D/2 x + D/2) of both streams combined, handed to put(column, value) by fours
+    const bool has_own = Tx > 0, has_oth = T[1 - x] > 0;  // a stream without tiles never wrote its accumulator
+    auto combine = [&](auto&& put) {
       const uint32_t tOwn = tmem + lane_base + BT_O_COL0 + x * 128 + x * (D / 2);
       const uint32_t tOth = tmem + lane_base + BT_O_COL0 + (1 - x) * 128 + x * (D / 2);
-      const bool has_own = T[x] > 0, has_oth = T[1 - x] > 0;  // a stream without tiles never wrote its accumulator
-      const float inv = 1.f / fin_l;
-      const float a_own = fin_w_own * inv, a_oth = fin_w_oth * inv;
-      float* dst = stage + row_in_tile * Cfg::RECV_STRIDE + x * (D / 2);
 #pragma unroll
       for (int q2 = 0; q2 < D / 64; ++q2) {
         uint32_t o[32], o2[32];
@@ -694,30 +569,118 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
           float v[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            v[i] = has_own ? __uint_as_float(o[4 * cc + i]) * a_own : 0.f;
-            if (has_oth) v[i] = fmaf(__uint_as_float(o2[4 * cc + i]), a_oth, v[i]);
+            v[i] = has_own ? __uint_as_float(o[4 * cc + i]) * w_own : 0.f;
+            if (has_oth) v[i] = fmaf(__uint_as_float(o2[4 * cc + i]), w_oth, v[i]);
           }
-          *reinterpret_cast<float4*>(dst + q2 * 32 + cc * 4) = make_float4(v[0], v[1], v[2], v[3]);
+          put(x * (D / 2) + q2 * 32 + cc * 4, make_float4(v[0], v[1], v[2], v[3]));
         }
       }
-      if (x == 0) *reinterpret_cast<float2*>(stage + row_in_tile * Cfg::RECV_STRIDE + D) = make_float2(fin_m, fin_l);
-    }
-    __syncthreads();
-    if (warp < 8) {
+    };
+    const bool warp_has_row = (warp & 3) * 32 < rows_here;  // warp-uniform (the TMEM loads are warp-collective)
+    // token and head of a row of the tile
+    auto place = [&](int row, int& hq) {
+      const int tok = tok0 + p.by_group.divmod(row, hq);
+      hq += hk * G;
+      return tok;
+    };
+    auto store_lse = [&](int tok, int hq, float value) {
+      int i;
+      const int b = p.by_q_len.divmod(tok, i);
+      L_.lse[(static_cast<int64_t>(b) * p.q_heads + hq) * n + i] = value * 0.69314718055994530942f;
+    };
+    if constexpr (C > 1) {
+      // ---- this CTA's partial of the row -> scratch, unnormalised, relative to the row's maximum over this CTA's tiles, as
+      // [column chunk][row] float4 so that a warp writes 512 contiguous bytes
+      float4* gpart = reinterpret_cast<float4*>(p.part + (static_cast<size_t>(gunit) * C + crank) * Cfg::PART_FLOATS);
+      float2* gml = reinterpret_cast<float2*>(p.ml + (static_cast<size_t>(gunit) * C + crank) * BT_ML_FLOATS);
+      if (warp_has_row) {
+        combine([&](int col, float4 v) {
+          if (row_valid) gpart[col / 4 * BT_BM + row_in_tile] = v;
+        });
+        if (row_valid && x == 0) gml[row_in_tile] = make_float2(fin_l > 0.f ? fin_m : -INFINITY, fin_l);
+      }
+      __threadfence();  // visible to the cluster before its barrier is passed
+      tc_fence_before();
+      cluster_sync_all();
+      // ---- behind the cluster barrier every CTA's partial is in the scratch (L2).  This CTA finishes the rows
+      // [128 crank / C, 128 (crank + 1) / C): a thread takes every 2C-th column chunk of one row, all its loads in flight
+      // at once; the sums run in CTA order, so the result never depends on timing.
       const bool clean = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;  // nobody gave up on a wait
+      constexpr int PER = BT_BM / C, MINE = D / 4 / (2 * C);
+      const int row = PER * crank + known_here(threadIdx.x) % PER, sub = known_here(threadIdx.x) / PER;
+      if (row < rows_here) {
+        const float2* uml = reinterpret_cast<const float2*>(p.ml + static_cast<size_t>(gunit) * C * BT_ML_FLOATS);
+        const float4* upart = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(gunit) * C * Cfg::PART_FLOATS);
+        float2 ml[C];
+        float4 v[MINE][C];
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) ml[cr] = __ldcg(uml + cr * BT_BM + row);
+#pragma unroll
+        for (int u = 0; u < MINE; ++u)
+#pragma unroll
+          for (int cr = 0; cr < C; ++cr)
+            v[u][cr] = __ldcg(upart + cr * (Cfg::PART_FLOATS / 4) + (u * 2 * C + sub) * BT_BM + row);
+        float M = -INFINITY, w[C], lall = 0.f;
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) M = fmaxf(M, ml[cr].x);  // (-inf: all of that CTA's tiles were hidden from the row)
+#pragma unroll
+        for (int cr = 0; cr < C; ++cr) {
+          w[cr] = fast_exp2(ml[cr].x - M);
+          lall = fmaf(w[cr], ml[cr].y, lall);
+        }
+        const float inv = 1.f / lall;
+        int hq;
+        const int tok = place(row, hq);
+        float* dst = L_.out + (static_cast<int64_t>(tok) * p.q_heads + hq) * D;
+#pragma unroll
+        for (int u = 0; u < MINE; ++u) {
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int cr = 0; cr < C; ++cr) {
+            acc.x = fmaf(w[cr], v[u][cr].x, acc.x);
+            acc.y = fmaf(w[cr], v[u][cr].y, acc.y);
+            acc.z = fmaf(w[cr], v[u][cr].z, acc.z);
+            acc.w = fmaf(w[cr], v[u][cr].w, acc.w);
+          }
+          if (clean)
+            *reinterpret_cast<float4*>(dst + (u * 2 * C + sub) * 4) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        }
+        if (clean && L_.lse && sub == 0) store_lse(tok, hq, M + log2f(lall));
+      }
+    } else {
+      // ---- one CTA per unit: the rows are staged in shared memory (every MMA and copy of the CTA is complete behind
+      // the barrier above, so the K/V rings are free once the (m, l) have been read) and written out as whole rows
+      float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);  // [row][Cfg::RECV_STRIDE]
+      named_sync(NB_MERGE, 256);
+      if (warp_has_row) {
+        const float inv = 1.f / fin_l;
+        w_own *= inv;
+        w_oth *= inv;
+        combine([&](int col, float4 v) {
+          *reinterpret_cast<float4*>(stage + row_in_tile * Cfg::RECV_STRIDE + col) = v;
+        });
+        if (x == 0) *reinterpret_cast<float2*>(stage + row_in_tile * Cfg::RECV_STRIDE + D) = make_float2(fin_m, fin_l);
+      }
+      named_sync(NB_MERGE, 256);
+      const bool clean = *abort_flag == 0 && *reinterpret_cast<volatile int*>(p.status) == 0;  // nobody gave up on a wait
+#pragma unroll 4
       for (int idx = threadIdx.x; idx < rows_here * (D / 4) && clean; idx += 256) {
         const int row = idx / (D / 4), chunk = idx % (D / 4);
-        const int tok = tok0 + row / G, hq = hk * G + row % G;
+        int hq;
+        const int tok = place(row, hq);
         *reinterpret_cast<float4*>(L_.out + (static_cast<int64_t>(tok) * p.q_heads + hq) * D + chunk * 4) =
             *reinterpret_cast<const float4*>(stage + row * Cfg::RECV_STRIDE + chunk * 4);
         if (chunk == 0 && L_.lse) {
           const float2 ml = *reinterpret_cast<const float2*>(stage + row * Cfg::RECV_STRIDE + D);
-          L_.lse[(static_cast<int64_t>(tok / n) * p.q_heads + hq) * n + tok % n] =
-              (ml.x + log2f(ml.y)) * 0.69314718055994530942f;
+          store_lse(tok, hq, ml.x + log2f(ml.y));
         }
       }
     }
   }
+  // (every thread of every CTA passes the cluster's barrier, whatever happened above; the output above is part of the
+  // softmax branch because code behind the branches would have to make do with the other roles' registers)
+  if constexpr (C > 1)
+    if (warp >= 8) cluster_sync_all();
 
   // ---- tear-down
   tc_fence_before();
@@ -736,35 +699,36 @@ struct BtPlan {
   int64_t estimate_ns;
 };
 
-template <int D, int NL>
+template <int D, int NL, int C>
 static cudaError_t bt_set_attributes() {
   static PerDeviceOnce attr_done;
   if (attr_done.done()) return cudaSuccess;
   cudaError_t e =
-      cudaFuncSetAttribute(branch_tc_kernel<D, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtCfg<D>::SMEM_BYTES);
+      cudaFuncSetAttribute(branch_tc_kernel<D, NL, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtCfg<D>::SMEM_BYTES);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(branch_tc_kernel<D, NL>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(branch_tc_kernel<D, NL, C>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess) attr_done.set();
   return e;
 }
 
-// How many clusters of c CTAs of the kernel can be resident at once on the current device (0 if the query fails).
-template <int D, int NL>
-static int bt_resident_clusters(int c) {
+// How many clusters of C CTAs of the kernel can be resident at once on the current device (0 if the query fails).
+template <int D, int NL, int C>
+static int bt_resident_clusters() {
   static ResidentClusters clusters;
-  if (bt_set_attributes<D, NL>() != cudaSuccess) return 0;
-  return clusters.get(reinterpret_cast<const void*>(branch_tc_kernel<D, NL>), c, BT_THREADS, BtCfg<D>::SMEM_BYTES);
+  if (bt_set_attributes<D, NL, C>() != cudaSuccess) return 0;
+  return clusters.get(reinterpret_cast<const void*>(branch_tc_kernel<D, NL, C>), C, BT_THREADS, BtCfg<D>::SMEM_BYTES);
 }
 
 // The tiling of one problem and the CTAs per unit, for `layers` problems in one launch: the pair with the shortest
-// estimated time.  A CTA takes 1.55 us per tile of 128 keys (1.2 with head_dim 64; a branch's suffix counted at 0.6 of its
+// estimated time.  A CTA takes 1.35 us per tile of 128 keys (0.95 with head_dim 64; a branch's suffix counted at 0.6 of its
 // longest possible walk) and a fixed time, larger when a cluster has to exchange partials; more, smaller row tiles walk
-// the prefix more often but may fill the machine better.
-constexpr int BT_FIXED_ALONE = 10, BT_FIXED_CLUSTER = 15;  // in half tiles
+// the prefix more often but may fill the machine better.  Measured (us, tiles per CTA in brackets): 8 kv heads, 128 rows,
+// prefix 1000 11.5 (3), prefix 4000 13.6 (6); 192 rows 12.3 (4), 18.9 (10); 32 kv heads, 128 rows 25.3 (10), 33.5 (16).
 template <int D, int NL>
 static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_heads, int kv_heads, int q_len,
                       int sm_count, int layers) {
+  constexpr int64_t TILE_NS = D == 128 ? 1350 : 950, ALONE_NS = D == 128 ? 6800 : 6000, CLUSTER_NS = D == 128 ? 8100 : 7600;
   BtPlan pl = {0, 0, 1, 0, 0, 1, false, 0};
   const int G = q_heads / kv_heads, nG = q_len * G;
   const int64_t Tp = (static_cast<int64_t>(prefix_len) + BT_BN - 1) / BT_BN;
@@ -775,16 +739,18 @@ static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_
     const int64_t units = row_tiles * kv_heads;
     if (units > (1 << 30)) return;
     const int64_t walk = Tp + per_tile * ts_est;
-    for (int c = 1; c <= BT_MAX_CTAS; ++c) {
+    for (int c = 1; c <= 8; c *= 2) {
       if (c > 1 && 2 * c > Tp + ts_max + 1) break;  // no more CTAs than pairs of tiles a unit certainly has
-      const int64_t at_once = c == 1 ? sm_count : bt_resident_clusters<D, NL>(c);
+      const int64_t at_once = c == 1   ? sm_count
+                              : c == 2 ? bt_resident_clusters<D, NL, 2>()
+                              : c == 4 ? bt_resident_clusters<D, NL, 4>()
+                                       : bt_resident_clusters<D, NL, 8>();
       if (at_once == 0 || (c > 1 && at_once < units)) continue;  // (a layer's clusters are all resident at once)
       const int64_t waves = (units * layers + at_once - 1) / at_once;
-      const int64_t est = waves * (2 * ((walk + c - 1) / c) + (c > 1 ? BT_FIXED_CLUSTER : BT_FIXED_ALONE));
+      const int64_t est = waves * ((walk + c - 1) / c * TILE_NS + (c > 1 ? CLUSTER_NS : ALONE_NS));
       if (best < 0 || est < best) {
         best = est;
-        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, true,
-                    est * (D == 128 ? 775 : 600)};
+        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, true, est};
       }
     }
   };
@@ -836,8 +802,6 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
                              int max_suffix_len, int n_branches, int q_heads, int q_len, float scale, int* status,
                              long long wait_limit, void* workspace, size_t workspace_bytes, cudaStream_t st,
                              LaunchInfo& li) {
-  cudaError_t e = bt_set_attributes<D, NL>();
-  if (e != cudaSuccess) return e;
   BtPlan pl = bt_plan<D, NL>(prefix_len, max_suffix_len, n_branches, q_heads, suffix.kv_heads, q_len, li.sm_count, layers);
   if (!pl.ok) return cudaErrorInvalidValue;
   // several CTAs per unit exchange partials through the scratch; without enough of it a unit is walked by one CTA
@@ -902,7 +866,9 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   p.slices_per_branch = pl.slices_per_branch;
   p.box_tokens = pl.box_tokens;
   p.box_keys = pl.branches_per_tile * q_len;
-  p.ctas_per_unit = pl.ctas_per_unit;
+  p.by_group = FastDiv(G);
+  p.by_q_len = FastDiv(q_len);
+  p.by_row_tiles = FastDiv(pl.row_tiles);
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_limit = wait_limit;
   p.d_suffix_len = d_suffix_len;
@@ -915,10 +881,19 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
                                 : nullptr;
   p.ml = pl.ctas_per_unit > 1 ? p.part + static_cast<size_t>(layers) * pl.units * pl.ctas_per_unit * BtCfg<D>::PART_FLOATS
                               : nullptr;
-  li.launches += 1;
-  return launch_pdl_cluster(branch_tc_kernel<D, NL>,
-                            dim3(static_cast<unsigned>(pl.units) * pl.ctas_per_unit, static_cast<unsigned>(layers)),
-                            dim3(BT_THREADS), BtCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(pl.ctas_per_unit), L, p);
+  auto launch = [&](auto set_attributes, auto kernel) {
+    cudaError_t e = set_attributes();
+    if (e != cudaSuccess) return e;
+    li.launches += 1;
+    return launch_pdl_cluster(kernel, dim3(static_cast<unsigned>(pl.units) * pl.ctas_per_unit, static_cast<unsigned>(layers)),
+                              dim3(BT_THREADS), BtCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(pl.ctas_per_unit), L, p);
+  };
+  switch (pl.ctas_per_unit) {
+    case 8: return launch(bt_set_attributes<D, NL, 8>, branch_tc_kernel<D, NL, 8>);
+    case 4: return launch(bt_set_attributes<D, NL, 4>, branch_tc_kernel<D, NL, 4>);
+    case 2: return launch(bt_set_attributes<D, NL, 2>, branch_tc_kernel<D, NL, 2>);
+  }
+  return launch(bt_set_attributes<D, NL, 1>, branch_tc_kernel<D, NL, 1>);
 }
 
 cudaError_t launch_branch_tc_layers(const BranchLayerTensors* t, int n_layers, const CacheView& prefix, int prefix_len,

@@ -368,7 +368,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
       const int nvalid = j < Tp ? p.prefix_len - j * TC_BN : lim - (j - Tp) * TC_BN;
       const bool masked = __any_sync(0xffffffffu, nvalid < TC_BN);
       softmax_tile_row<false, D>(
-          tS, tP, tO, j, 4, masked, ColumnLimit{nvalid}, c, m_ref, l,
+          tS, tP, tO, j, 4, masked, ColumnLimit{nvalid}, true, c, m_ref, l,
           [&] { return mbar_test_wait(bar(BAR_O_READY + x), (j - 1) & 1); },
           [&] { ok = ok && mbar_wait(bar(BAR_O_READY + x), (j - 1) & 1, abort_flag, p.status); },
           [&] { signal(NB_S_FREE); },

@@ -58,12 +58,13 @@ __device__ __forceinline__ void mask_tile_row(uint32_t tS, const Allow& allow) {
 // j: number of tiles this stream has processed before (0: O holds nothing yet).
 // chunks: P is wanted for the first `chunks` blocks of 32 columns only; masked: warp-uniform, when false every column
 // is visible and `allow` is not consulted.
-// PARTIAL: the stream may meet rows that see none of a tile (their reference maximum stays -inf and P is 0);
-// otherwise every row sees column 0 of its first tile.
+// PARTIAL: the stream may meet rows that see none of a tile (row_sees, or all columns masked: their reference maximum
+// stays and P is 0); otherwise every row sees column 0 of its first tile.
 template <bool PARTIAL, int D, class Allow, class TestO, class WaitO, class Loaded, class Release>
 __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint32_t tO, int j, int chunks, bool masked,
-                                                 const Allow& allow, float c, float& m_ref, float& l, TestO&& test_o,
-                                                 WaitO&& wait_o, Loaded&& loaded, Release&& release_early) {
+                                                 const Allow& allow, bool row_sees, float c, float& m_ref, float& l,
+                                                 TestO&& test_o, WaitO&& wait_o, Loaded&& loaded,
+                                                 Release&& release_early) {
   if (masked) mask_tile_row(tS, allow);
   uint32_t sv[128];
 #pragma unroll
@@ -87,7 +88,7 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
     mx = fmaxf(fmax3(fmax3(b[0], b[1], b[2]), fmax3(b[3], b[4], b[5]), fmaxf(b[6], b[7])),
                fmax3(fmax3(d[0], d[1], d[2]), fmax3(d[3], d[4], d[5]), fmaxf(d[6], d[7])));
   }
-  const float mxs = mx * c;
+  const float mxs = (PARTIAL && !row_sees) ? -INFINITY : mx * c;
   // lazy reference: it only moves when the maximum outgrew it by 2^8 (a row that has seen nothing keeps -inf,
   // and its first visible score moves it because -inf + 8 is still -inf)
   const bool grow = mxs > m_ref + TC_RESCALE_THRESHOLD;
@@ -110,7 +111,7 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
     }
   }
   // ---- P
-  const float nm = (PARTIAL && m_ref == -INFINITY) ? 0.f : -m_ref;
+  const float nm = (PARTIAL && !row_sees) ? -INFINITY : (PARTIAL && m_ref == -INFINITY) ? 0.f : -m_ref;
   const uint64_t nm2 = pack2(nm, nm), c2 = pack2(c, c);
   uint64_t lacc[4];
 #pragma unroll

@@ -563,8 +563,11 @@ bool branch_stream_preferred(int n_branches, int q_heads, int kv_heads, int q_le
 }
 
 // A warp takes 1.13 us per chunk (0.73 with head_dim 64) while every SM is streaming, whatever the split; the rest of a
-// launch is about 6 us.  Measured (us, estimate in brackets): 8 kv heads, prefix 4000, 64 rows 15.6 (15), 128 rows 24.8 (25),
-// 192 rows 42.8 (44); prefix 1000, 192 rows 16.6 (16); 32 kv heads, 128 rows (two waves) 77 (79).
+// launch is about 6 us, and a CTA of the narrow shape adds 4 us of first loads and merge (head_dim 64: hidden behind the
+// other CTA's stream); its waves overlap, so a last one counts by its share.  Measured (us, estimate in brackets): 8 kv
+// heads, prefix 4000, 64 rows 15.6 (15), 128 rows 24.8 (25), 192 rows 42.8 (44); 8 layers x 8 kv heads, prefix 67, 16 branches x
+// 16 rows 38 (28; without the 4 us 15, and the tensor-core kernel, estimated at 19, takes 25), prefix 1474, 14 branches x
+// 24 rows 155 (147); 32 kv heads, prefix 106, 16 branches x 14 rows 20 (17; tensor cores 17).
 int64_t branch_stream_estimate_ns(int n_branches, int q_heads, int kv_heads, int q_len, int head_dim, int prefix_len,
                                   int max_suffix_len, int layers, int sm_count) {
   const int nG = q_len * (q_heads / kv_heads);
@@ -576,9 +579,10 @@ int64_t branch_stream_estimate_ns(int n_branches, int q_heads, int kv_heads, int
   const int64_t branches_here = std::min<int64_t>(n_branches, std::max(1, 16 / nG));
   const int64_t chunks = (prefix_len + 15) / 16 + branches_here * ((suffix_chunks * 6 + 9) / 10);  // (mean lengths at 0.6 of the bound)
   const int64_t warps = sh.narrow ? 4 : 8 << sh.cluster_log2;
-  const int64_t at_once = sh.narrow ? 2 * sm_count : problems;
-  const int64_t waves = (problems + at_once - 1) / at_once;
-  return 6000 + waves * ((chunks + warps - 1) / warps) * (head_dim == 128 ? 1130 : 730);
+  const int64_t walk = (chunks + warps - 1) / warps * (head_dim == 128 ? 1130 : 730);
+  if (!sh.narrow) return 6000 + walk;
+  const int64_t at_once = 2 * sm_count;
+  return 6000 + std::max(problems, at_once) * (walk + (head_dim == 128 ? 4000 : 0)) / at_once;
 }
 
 static cudaError_t launch_stream(const bf16* q, const CacheView& prefix, int prefix_len, const CacheView& suffix,

@@ -15,7 +15,7 @@
 // ranges, one per CTA, and so are the suffix tiles (the prefix share does not depend on the device-side lengths,
 // so its first loads are in flight while the lengths arrive).  Inside a CTA:
 //   loader warp  : TMA (tiled, 128-byte swizzle) Q once -- one box [tokens][G heads][64] lands in stacked-row
-//                  order -- then the K/V tiles of the CTA's list into 3-stage rings, K and V refilled independently
+//                  order -- then the K/V tiles of the CTA's list, in the order of their use, into one ring of slots
 //   patch warp   : passes landed V tiles on to the MMA issuer, after zeroing the rows of a last, partial 16-key group
 //                  that are no keys (rows at or beyond a branch's device-side length, which TMA cannot know: their
 //                  weights are 0, but 0 x NaN must not reach an accumulator)
@@ -48,7 +48,7 @@ namespace jup {
 constexpr int BT_BM = 128;             // stacked rows per tile (at most)
 constexpr int BT_BN = 128;             // keys per KV tile
 constexpr int BT_PANEL_BYTES = 16384;  // 128 rows x 64 elements
-constexpr int BT_KV_STAGES = 3;
+constexpr int BT_MAX_SLOTS = 12;
 constexpr int BT_MAX_BRANCHES = 32;    // branches in one row tile
 constexpr int BT_ML_FLOATS = BT_BM * 2;  // one CTA's (m, l) pairs
 // Layers of one call share a launch from this many on.
@@ -89,22 +89,22 @@ struct BtLayers {
   BtLayer l[NL];
 };
 
-// shared memory: [Q][K ring][V ring][barriers, flags][lengths and tile counts of the row tile's branches]
+// shared memory: [Q][K/V slots][barriers, flags][lengths and tile counts of the row tile's branches]
 template <int D>
 struct BtCfg {
+  static constexpr int SLOTS = D == 128 ? 6 : 12;
   static constexpr int TILE_BYTES = BT_BN * D * 2;
   static constexpr int PANELS = D / 64;
   static constexpr int CH = D / 8;  // 16-byte pieces per K/V row
   static constexpr int RECV_STRIDE = D + 4;  // one CTA per unit: floats per staged row: O, then (m, l), padded against bank conflicts
   static constexpr int PART_FLOATS = BT_BM * D;  // one CTA's partial accumulator
   static constexpr int SMEM_Q = 0;
-  static constexpr int SMEM_K = TILE_BYTES;
-  static constexpr int SMEM_V = SMEM_K + BT_KV_STAGES * TILE_BYTES;
-  static constexpr int SMEM_BAR = SMEM_V + BT_KV_STAGES * TILE_BYTES;
-  static constexpr int SMEM_LEN = SMEM_BAR + 256;
+  static constexpr int SMEM_KV = TILE_BYTES;
+  static constexpr int SMEM_BAR = SMEM_KV + SLOTS * TILE_BYTES;
+  static constexpr int SMEM_LEN = SMEM_BAR + 512;
   static constexpr int SMEM_BYTES = SMEM_LEN + 2 * BT_MAX_BRANCHES * 4 + 1024;  // + slack for 1024-byte alignment
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
-  static_assert(BT_BM * RECV_STRIDE * 4 <= 2 * BT_KV_STAGES * TILE_BYTES, "the staged rows fit in the rings");
+  static_assert(SLOTS <= BT_MAX_SLOTS && BT_BM * RECV_STRIDE * 4 <= SLOTS * TILE_BYTES, "the staged rows fit in the slots");
 };
 // TMEM columns: O_0 | O_1 | S | P_0 | P_1
 constexpr int BT_O_COL0 = 0, BT_S_COL = 256, BT_P_COL0 = 384;
@@ -116,14 +116,12 @@ constexpr int BT_THREADS = 32 * 12;
 
 enum {
   BT_Q_FULL = 0,
-  BT_K_FULL = 1,    // [3]
-  BT_K_EMPTY = 4,   // [3]
-  BT_V_FULL = 7,    // [3]
-  BT_V_EMPTY = 10,  // [3]
-  BT_S_FULL = 13,   // [2] one per stream
-  BT_O_READY = 15,  // [2]
-  BT_DRAIN = 17,    // [2] one per issuing thread
-  BT_BAR_COUNT = 19
+  BT_FULL = 1,                           // [SLOTS] a K or V tile has landed
+  BT_EMPTY = BT_FULL + BT_MAX_SLOTS,     // [SLOTS] and its MMAs are done
+  BT_S_FULL = BT_EMPTY + BT_MAX_SLOTS,   // [2] one per stream
+  BT_O_READY = BT_S_FULL + 2,            // [2]
+  BT_DRAIN = BT_O_READY + 2,             // [2] one per issuing thread
+  BT_BAR_COUNT = BT_DRAIN + 2
 };
 
 // One entry of a CTA's tile list.
@@ -145,11 +143,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   using Cfg = BtCfg<D>;
   constexpr int TILE_BYTES = Cfg::TILE_BYTES;
   const BtLayer& L_ = layers.l[NL == 1 ? 0 : blockIdx.y];
-  constexpr int KV_STAGES = BT_KV_STAGES;
+  constexpr int SLOTS = Cfg::SLOTS;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t sQ = smem_base + Cfg::SMEM_Q, sK = smem_base + Cfg::SMEM_K, sV = smem_base + Cfg::SMEM_V;
+  const uint32_t sQ = smem_base + Cfg::SMEM_Q, sKV = smem_base + Cfg::SMEM_KV;
   const uint32_t sBar = smem_base + Cfg::SMEM_BAR;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + Cfg::SMEM_BAR + 8 * BT_BAR_COUNT);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + Cfg::SMEM_BAR + 8 * BT_BAR_COUNT + 8);
@@ -218,10 +216,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   const uint32_t tmem = *tmem_slot;
   pdl_wait();  // everything above overlapped the previous kernel's tail; global memory is touched from here on
 
-  // K (V) of list entry e into the ring slot of sequence number s
-  auto load_kv = [&](bool is_v, int s, const BtTile& e) {
-    const int slot = s % KV_STAGES;
-    const uint32_t dst = (is_v ? sV : sK) + slot * TILE_BYTES, full = bar((is_v ? BT_V_FULL : BT_K_FULL) + slot);
+  // K (V) of list entry e into a slot
+  auto load_kv = [&](bool is_v, int slot, const BtTile& e) {
+    const uint32_t dst = sKV + slot * TILE_BYTES, full = bar(BT_FULL + slot);
     if (e.seg == BT_NEW) {  // token-major rows of the row tile's branches, one box
       mbar_expect_tx(full, static_cast<uint32_t>(p.box_keys) * (D * 2u));
       const CUtensorMap* m = is_v ? &L_.tm_nv : &L_.tm_nk;
@@ -235,7 +232,13 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         tma_load_4d(dst + c * BT_PANEL_BYTES, m, full, c * 64, e.tile * BT_BN, hk, e.seg == BT_PREFIX ? 0 : b_first + e.seg);
     }
   };
-  const int pre_issued = min(npre, KV_STAGES);
+  // K and V share one ring: loaded in the order of their use, K_0 K_1 V_0 K_2 V_1 .. K_T-1 V_T-2 V_T-1, each
+  // into the slot of the load SLOTS before it.  (With a ring of three for either, a V tile arrived with its K tile, held
+  // its slot for the whole softmax of that tile, and the next V was asked for late.  8 layers x 8 kv heads, prefix 2048,
+  // 16 branches x 20 rows 94.1 -> 90.4 us; head_dim 64, with twice as many slots, 16 branches x 20 rows, prefix 1500
+  // 16.0 -> 15.4 us.)
+  auto load_slot = [&](int i) { return i % SLOTS; };
+  const int pre_issued = min(max(2 * npre - 1, 0), SLOTS);  // loads whose place in that order does not depend on the lengths
   if (warp == BT_LOADER_WARP && lane == 0) {
     // Q: box_tokens tokens from tok0 on, heads hk G .. hk G + G - 1, one box per 64-column panel; the box lands as
     // rows (token, head) = stacked-row order.  Rows of the Q buffer beyond the box are never written: they belong
@@ -244,9 +247,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
 #pragma unroll
     for (int c = 0; c < Cfg::PANELS; ++c)
       tma_load_4d(sQ + c * BT_PANEL_BYTES, &L_.tm_q, bar(BT_Q_FULL), c * 64, hk * G, tok0, 0);
-    for (int s = 0; s < pre_issued; ++s) {
-      load_kv(false, s, BtTile{BT_PREFIX, p0 + s, 0});
-      load_kv(true, s, BtTile{BT_PREFIX, p0 + s, 0});
+    for (int i = 0; i < pre_issued; ++i) {
+      const bool is_v = i > 0 && (i & 1) == 0;
+      load_kv(is_v, i, BtTile{BT_PREFIX, p0 + (is_v ? i / 2 - 1 : (i + 1) / 2), 0});
     }
   } else if (warp == 0) {
     // ---- lengths and tile counts of the row tile's branches
@@ -288,40 +291,30 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const int tile = g - (cursor > 0 ? cum_s[cursor - 1] : 0);
     return BtTile{cursor, tile, min((fused ? len_s[cursor] - n : len_s[cursor]) - tile * BT_BN, BT_BN)};
   };
+  auto k_load = [&](int s) { return max(2 * s - 1, 0); };  // the number of a tile's load
+  auto v_load = [&](int s) { return min(2 * s + 2, 2 * Tall - 1); };
   const int T[2] = {(Tall + 1) >> 1, Tall >> 1};  // stream x takes the sequence numbers 2 i + x
 
   if (warp == BT_LOADER_WARP) {
     // =============================================================== loader
     reg_dec<BT_REGS_OTHER>();
     if (lane == 0) {
-      // K and V rings are refilled independently: a K slot is free once its Q K^T has run, a V slot only after
-      // its P V, and neither queue may hold up the other
       bool ok = true;
-      int kn = pre_issued, vn = pre_issued, k_cursor = 0, v_cursor = 0;
-      PollGuard guard(wl);
-      while (ok && (kn < Tall || vn < Tall)) {
-        bool progress = false;
-        if (kn < Tall && (kn < KV_STAGES || mbar_test_wait(bar(BT_K_EMPTY + kn % KV_STAGES), (kn / KV_STAGES - 1) & 1))) {
-          load_kv(false, kn, tile_at(kn, k_cursor));
-          ++kn;
-          progress = true;
-        }
-        if (vn < Tall && (vn < KV_STAGES || mbar_test_wait(bar(BT_V_EMPTY + vn % KV_STAGES), (vn / KV_STAGES - 1) & 1))) {
-          load_kv(true, vn, tile_at(vn, v_cursor));
-          ++vn;
-          progress = true;
-        }
-        if (progress) guard.progress();
-        else ok = guard.idle(abort_flag, p.status);
+      int i = pre_issued, k_cursor = 0, v_cursor = 0;
+      for (; i < 2 * Tall; ++i) {
+        const bool is_v = i == 2 * Tall - 1 || (i > 0 && (i & 1) == 0);
+        const BtTile e = is_v ? tile_at(i == 2 * Tall - 1 ? Tall - 1 : i / 2 - 1, v_cursor) : tile_at((i + 1) / 2, k_cursor);
+        const int slot = load_slot(i);
+        if (i >= SLOTS) ok = mbar_wait(bar(BT_EMPTY + slot), (i / SLOTS - 1) & 1, abort_flag, p.status, wl);
+        if (!ok) break;
+        load_kv(is_v, slot, e);
       }
       if (*abort_flag) {
         // wait (bounded) until every copy this thread started has landed before shared memory is released
         int dummy = 0;
         volatile int* none = &dummy;
-        for (int s = max(0, kn - KV_STAGES); s < kn; ++s)
-          mbar_wait(bar(BT_K_FULL + s % KV_STAGES), (s / KV_STAGES) & 1, none, nullptr);
-        for (int s = max(0, vn - KV_STAGES); s < vn; ++s)
-          mbar_wait(bar(BT_V_FULL + s % KV_STAGES), (s / KV_STAGES) & 1, none, nullptr);
+        for (int j = max(0, i - SLOTS); j < i; ++j)
+          mbar_wait(bar(BT_FULL + load_slot(j)), (j / SLOTS) & 1, none, nullptr);
         mbar_wait(bar(BT_Q_FULL), 0, none, nullptr);
       }
     }
@@ -335,11 +328,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     int cursor = 0;
     for (int s = 0; s < Tall && ok; ++s) {
       const BtTile e = tile_at(s, cursor);
-      const int slot = s % KV_STAGES;
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_V_FULL + slot), (s / KV_STAGES) & 1, abort_flag, p.status, wl));
+      const int i = v_load(s), slot = load_slot(i);
+      ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
       if (!ok) break;
       if (e.patch()) {
-        const uint32_t tile_addr = sV + slot * TILE_BYTES;
+        const uint32_t tile_addr = sKV + slot * TILE_BYTES;
         constexpr int CH = Cfg::CH;
         for (int idx = lane; idx < (16 - (e.valid & 15)) * CH; idx += 32) {
           const int r = e.valid + idx / CH, c = idx % CH;  // 16-byte piece c of row r in the 128-byte-swizzled panels
@@ -363,15 +356,15 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     int turn = 0, cursor = 0;
     if (lane == 0) ok = mbar_wait(bar(BT_Q_FULL), 0, abort_flag, p.status, wl);  // (also when the list is empty: the copy must land)
     for (int s = 0; s < Tall; ++s) {
-      const int slot = s % KV_STAGES;
+      const int i = k_load(s), slot = load_slot(i);
       const BtTile e = tile_at(s, cursor);
       const uint32_t idesc_qk = tc_idesc_bf16(BT_BM, e.groups() * 16, false, false);
-      if (lane == 0) ok = ok && mbar_wait(bar(BT_K_FULL + slot), (s / KV_STAGES) & 1, abort_flag, p.status, wl);
+      if (lane == 0) ok = ok && mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl);
       if (s > 0) named_sync(NB_S_FREE + ((s - 1) & 1), 160);
       if (lane == 0 && ok) {
         flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
         tc_fence_after();
-        const uint32_t k_lo = tc_desc_lo(sK + slot * TILE_BYTES, 16);
+        const uint32_t k_lo = tc_desc_lo(sKV + slot * TILE_BYTES, 16);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
           const uint32_t off = ((ks >> 2) * BT_PANEL_BYTES + (ks & 3) * 32) >> 4;
@@ -379,7 +372,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         }
         tc_commit(bar(BT_S_FULL + (s & 1)));
         flag_write(qk_turn, ++turn);
-        tc_commit(bar(BT_K_EMPTY + slot));
+        tc_commit(bar(BT_EMPTY + slot));
       }
       __syncwarp();
     }
@@ -397,8 +390,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     bool ok = true;
     int cursor = 0;
     for (int s = 0; s < Tall; ++s) {
-      const int slot = s % KV_STAGES, x = s & 1;
-      const uint32_t v_lo = tc_desc_lo(sV + slot * TILE_BYTES, BT_PANEL_BYTES);
+      const int slot = load_slot(v_load(s)), x = s & 1;
+      const uint32_t v_lo = tc_desc_lo(sKV + slot * TILE_BYTES, BT_PANEL_BYTES);
       const uint32_t o_col = tmem + BT_O_COL0 + x * 128, p_col = tmem + BT_P_COL0 + x * 64;
       const BtTile e = tile_at(s, cursor);
       const int groups = e.groups();
@@ -419,7 +412,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         for (int ks = 6; ks < 8; ++ks)
           if (ks < groups) tc_mma_ts_lo(o_col, p_col + ks * 8, v_lo + ks * (2048 >> 4), idesc_pv, 1);
         tc_commit(bar(BT_O_READY + x));
-        tc_commit(bar(BT_V_EMPTY + slot));
+        tc_commit(bar(BT_EMPTY + slot));
       }
       __syncwarp();
     }
@@ -537,10 +530,10 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     pdl_launch_dependents();  // the next kernel of the stream may start its own set-up now
 
     // ---- the two streams' (m, l) of a row cross through shared memory: the K slot of the stream's last tile,
-    // free once its accumulator is complete; a stream without tiles owns slot x, never filled or long free
+    // free once its accumulator is complete and not filled again; a stream without tiles takes slot 2 + x, never filled then
     auto ml_of = [&](int y) {
-      const int slot = T[y] > 0 ? (2 * (T[y] - 1) + y) % KV_STAGES : y;
-      return reinterpret_cast<float2*>(smem_gen + Cfg::SMEM_K + slot * TILE_BYTES);
+      const int slot = T[y] > 0 ? load_slot(k_load(2 * (T[y] - 1) + y)) : 2 + y;
+      return reinterpret_cast<float2*>(smem_gen + Cfg::SMEM_KV + slot * TILE_BYTES);
     };
     if (Tx > 0) ok = mbar_wait(bar(BT_O_READY + x), (Tx - 1) & 1, abort_flag, p.status, wl) && ok;
     ml_of(x)[row_in_tile] = make_float2(m_ref, l);
@@ -649,8 +642,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       }
     } else {
       // ---- one CTA per unit: the rows are staged in shared memory (every MMA and copy of the CTA is complete behind
-      // the barrier above, so the K/V rings are free once the (m, l) have been read) and written out as whole rows
-      float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_K);  // [row][Cfg::RECV_STRIDE]
+      // the barrier above, so the K/V slots are free once the (m, l) have been read) and written out as whole rows
+      float* stage = reinterpret_cast<float*>(smem_gen + Cfg::SMEM_KV);  // [row][Cfg::RECV_STRIDE]
       named_sync(NB_MERGE, 256);
       if (warp_has_row) {
         const float inv = 1.f / fin_l;

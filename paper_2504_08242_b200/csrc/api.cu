@@ -68,14 +68,16 @@ jupiter_status jupiter_create(jupiter_ctx** out_ctx, int device, size_t workspac
   int count = 0;
   cudaError_t e = cudaGetDeviceCount(&count);
   if (e != cudaSuccess || device < 0 || device >= count) return e != cudaSuccess ? JUPITER_ERR_CUDA : JUPITER_ERR_INVALID_ARG;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return JUPITER_ERR_CUDA;
-  if (prop.major != 10) return JUPITER_ERR_UNSUPPORTED;  // kernels are built for sm_100a only
+  int major = 0, sm_count = 0;  // (two attributes: cudaGetDeviceProperties takes milliseconds)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return JUPITER_ERR_CUDA;
+  if (major != 10) return JUPITER_ERR_UNSUPPORTED;  // kernels are built for sm_100a only
   jupiter_ctx* ctx = new (std::nothrow) jupiter_ctx();
   if (!ctx) return JUPITER_ERR_INVALID_ARG;
   std::memset(ctx, 0, sizeof *ctx);
   ctx->device = device;
-  ctx->sm_count = prop.multiProcessorCount;
+  ctx->sm_count = sm_count;
   ctx->workspace_bytes = workspace_bytes ? workspace_bytes : (size_t(64) << 20);
   ctx->wait_limit = 2000000000ll;
   DeviceGuard guard(device);

@@ -159,7 +159,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   auto bar = [&](int i) { return sBar + 8u * i; };
   const long long wl = p.wait_limit;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int unit = blockIdx.x / C, crank = blockIdx.x % C;  // clusters are consecutive CTAs: crank is the cluster rank
   int rt;
   const int hk = p.by_row_tiles.divmod(unit, rt);
@@ -213,7 +213,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_wait();  // everything above overlapped the previous kernel's tail; global memory is touched from here on
 
   // K (V) of list entry e into a slot
@@ -351,17 +351,18 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     // (two issuing threads and one S buffer handed back by the softmax as soon as it has read its scores: see
     // prefill_tc.cu)
     reg_dec<BT_REGS_OTHER>();
+    const bool leader = elect_one();
     const uint32_t s_col = tmem + BT_S_COL, q_lo = tc_desc_lo(sQ, 16);
     bool ok = true;
     int turn = 0, cursor = 0;
-    if (lane == 0) ok = mbar_wait(bar(BT_Q_FULL), 0, abort_flag, p.status, wl);  // (also when the list is empty: the copy must land)
+    ok = mbar_wait(bar(BT_Q_FULL), 0, abort_flag, p.status, wl);  // (also when the list is empty: the copy must land)
     for (int s = 0; s < Tall; ++s) {
       const int i = k_load(s), slot = load_slot(i);
       const BtTile e = tile_at(s, cursor);
       const uint32_t idesc_qk = tc_idesc_bf16(BT_BM, e.groups() * 16, false, false);
-      if (lane == 0) ok = ok && mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl);
+      ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
       if (s > 0) named_sync(NB_S_FREE + ((s - 1) & 1), 160);
-      if (lane == 0 && ok) {
+      if (leader && ok) {
         flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
         tc_fence_after();
         const uint32_t k_lo = tc_desc_lo(sKV + slot * TILE_BYTES, 16);
@@ -377,7 +378,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       __syncwarp();
     }
     if (Tall > 0) named_sync(NB_S_FREE + ((Tall - 1) & 1), 160);
-    if (lane == 0 && !ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
+    if (leader && !ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
       int dummy = 0;
       tc_commit(bar(BT_DRAIN));
       mbar_wait(bar(BT_DRAIN), 0, &dummy, nullptr);
@@ -387,6 +388,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     // =============================================================== issuer of O += P V, tiles in list order
     reg_dec<BT_REGS_OTHER>();
     constexpr uint32_t idesc_pv = tc_idesc_bf16(BT_BM, D, false, true);
+    const bool leader = elect_one();
     bool ok = true;
     int cursor = 0;
     for (int s = 0; s < Tall; ++s) {
@@ -395,9 +397,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       const uint32_t o_col = tmem + BT_O_COL0 + x * 128, p_col = tmem + BT_P_COL0 + x * 64;
       const BtTile e = tile_at(s, cursor);
       const int groups = e.groups();
-      if (lane == 0) ok = ok && count_spin_wait(v_ready, s + 1, abort_flag, p.status, wl) >= 0;
+      ok = __all_sync(0xffffffffu, ok && count_spin_wait(v_ready, s + 1, abort_flag, p.status, wl) >= 0);
       named_sync(NB_P_EARLY + x, 160);  // the first 96 keys while the softmax finishes the last 32
-      if (lane == 0 && ok) {
+      if (leader && ok) {
         for (int it = 0; it < 4096 && (flag_read(qk_turn) & 1); ++it) {}  // stand back for the scores
         tc_fence_after();
 #pragma unroll
@@ -406,7 +408,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       }
       __syncwarp();
       named_sync(NB_P_FULL + x, 160);
-      if (lane == 0 && ok) {
+      if (leader && ok) {
         tc_fence_after();
 #pragma unroll
         for (int ks = 6; ks < 8; ++ks)
@@ -416,7 +418,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       }
       __syncwarp();
     }
-    if (lane == 0 && !ok) {
+    if (leader && !ok) {
       int dummy = 0;
       tc_commit(bar(BT_DRAIN + 1));
       mbar_wait(bar(BT_DRAIN + 1), 0, &dummy, nullptr);

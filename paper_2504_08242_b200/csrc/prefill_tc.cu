@@ -126,7 +126,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   static_assert(8 * BAR_COUNT + 20 <= 256, "barrier block");
   auto bar = [&](int i) { return sBar + 8u * i; };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
   // ---- work assignment: heaviest query blocks first
   int bh, hb, hr;
@@ -173,7 +173,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_wait();  // everything above overlapped the previous kernel's tail; global memory is touched from here on
 
   if (warp == Cfg::LOADER_WARP) {
@@ -262,6 +262,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     reg_dec<Cfg::REGS_OTHER>();
     constexpr uint32_t idesc_qk = tc_idesc_bf16(TC_BM, TC_BN, false, false);
     const uint32_t s_col = tmem + Cfg::S_COL;
+    const bool leader = elect_one();
     bool ok = true;
     // One S buffer serves both query tiles: it may be written once the softmax that got the previous scores has
     // read them (a fraction of a tile's time), long before that tile's P V is due, so the scores are complete when
@@ -270,14 +271,15 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     int turn = 0;
     for (int j = 0; j < Tall; ++j) {
       const uint32_t k_lo = tc_desc_lo(sK + (j % KV_STAGES) * TILE_BYTES, 16);
-      if (lane == 0) ok = ok && mbar_wait(bar(BAR_K_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
+      ok = ok && mbar_wait(bar(BAR_K_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
         if (j >= T[x]) continue;
-        if (j == 0 && lane == 0) ok = ok && mbar_wait(bar(BAR_Q_FULL + x), 0, abort_flag, p.status);
+        if (j == 0) ok = ok && mbar_wait(bar(BAR_Q_FULL + x), 0, abort_flag, p.status);
         if (prev_x >= 0) named_sync(NB_S_FREE + prev_x, 160);
         prev_x = x;
-        if (lane == 0 && ok) {
+        ok = __all_sync(0xffffffffu, ok);
+        if (leader && ok) {
           flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
           tc_fence_after();
           const uint32_t q_lo = tc_desc_lo(sQ + x * TILE_BYTES, 16);
@@ -291,10 +293,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         __syncwarp();
       }
-      if (lane == 0 && ok) tc_commit(bar(BAR_K_EMPTY + j % KV_STAGES));
+      if (leader && ok) tc_commit(bar(BAR_K_EMPTY + j % KV_STAGES));
     }
     if (prev_x >= 0) named_sync(NB_S_FREE + prev_x, 160);
-    if (lane == 0 && !ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
+    if (leader && !ok) {  // make sure no MMA of this thread is still running before TMEM and smem go away
       int dummy = 0;
       tc_commit(bar(BAR_DRAIN));
       mbar_wait(bar(BAR_DRAIN), 0, &dummy, nullptr);
@@ -307,16 +309,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     // batch: the shared-memory read takes longer than an MMA.)
     reg_dec<Cfg::REGS_OTHER>();
     constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, D, false, true);
+    const bool leader = elect_one();
     bool ok = true;
     for (int j = 0; j < Tall; ++j) {
       const uint32_t v_lo = tc_desc_lo(sV + (j % KV_STAGES) * TILE_BYTES, TC_PANEL_BYTES);
-      if (lane == 0) ok = ok && mbar_wait(bar(BAR_V_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
+      ok = ok && mbar_wait(bar(BAR_V_FULL + j % KV_STAGES), (j / KV_STAGES) & 1, abort_flag, p.status);
 #pragma unroll
       for (int x = 0; x < NQ; ++x) {
         if (j >= T[x]) continue;
         const uint32_t o_col = tmem + Cfg::O_COL0 + x * 128, p_col = tmem + Cfg::P_COL0 + x * 64;
         named_sync(NB_P_EARLY + x, 160);  // the first 96 keys while the softmax finishes the last 32
-        if (lane == 0 && ok) {
+        ok = __all_sync(0xffffffffu, ok);
+        if (leader && ok) {
           for (int it = 0; it < 4096 && (flag_read(qk_turn) & 1); ++it) {}
           tc_fence_after();
 #pragma unroll
@@ -325,7 +329,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         __syncwarp();
         named_sync(NB_P_FULL + x, 160);
-        if (lane == 0 && ok) {
+        if (leader && ok) {
           tc_fence_after();
 #pragma unroll
           for (int ks = 6; ks < 8; ++ks) tc_mma_ts_lo(o_col, p_col + ks * 8, v_lo + ks * (2048 >> 4), idesc_pv, 1);
@@ -333,9 +337,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         __syncwarp();
       }
-      if (lane == 0 && ok) tc_commit(bar(BAR_V_EMPTY + j % KV_STAGES));
+      if (leader && ok) tc_commit(bar(BAR_V_EMPTY + j % KV_STAGES));
     }
-    if (lane == 0 && !ok) {
+    if (leader && !ok) {
       int dummy = 0;
       tc_commit(bar(BAR_DRAIN + 1));
       mbar_wait(bar(BAR_DRAIN + 1), 0, &dummy, nullptr);

@@ -131,7 +131,7 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_wait();  // everything above overlapped the previous kernel's tail; global memory is touched from here on
 
   if (warp == Cfg::LOADER_WARP) {
@@ -205,7 +205,7 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // =============================================================== MMA issuer
     // Steps (each cleared by the watcher):  S(0), S(1), S(2);  then per tile j:  O += P(j) V(j),  S(j+3).
     reg_dec<Cfg::REGS_OTHER>();
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_qk = tc_idesc_bf16(TC_BM, TC_BN, false, false);
       constexpr uint32_t idesc_pv = tc_idesc_bf16(TC_BM, D, false, true);
       const uint32_t q_lo = tc_desc_lo(sQ, 16), k_lo0 = tc_desc_lo(sK, 16), v_lo0 = tc_desc_lo(sV, TC_PANEL_BYTES);

@@ -49,6 +49,7 @@ constexpr int BT_BM = 128;             // stacked rows per tile (at most)
 constexpr int BT_BN = 128;             // keys per KV tile
 constexpr int BT_PANEL_BYTES = 16384;  // 128 rows x 64 elements
 constexpr int BT_MAX_SLOTS = 12;
+constexpr int BT_LEAD = 4;             // prefix tiles at the front of a CTA's list (even: a pair of tiles is one per stream)
 constexpr int BT_MAX_BRANCHES = 32;    // branches in one row tile
 constexpr int BT_ML_FLOATS = BT_BM * 2;  // one CTA's (m, l) pairs
 // Layers of one call share a launch from this many on.
@@ -239,17 +240,19 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   // 16.0 -> 15.4 us.)
   auto load_slot = [&](int i) { return i % SLOTS; };
   const int pre_issued = min(max(2 * npre - 1, 0), SLOTS);  // loads whose place in that order does not depend on the lengths
-  if (warp == BT_LOADER_WARP && lane == 0) {
-    // Q: box_tokens tokens from tok0 on, heads hk G .. hk G + G - 1, one box per 64-column panel; the box lands as
-    // rows (token, head) = stacked-row order.  Rows of the Q buffer beyond the box are never written: they belong
-    // to no row of this tile and whatever the tensor cores make of them is never used.
-    mbar_expect_tx(bar(BT_Q_FULL), static_cast<uint32_t>(p.box_tokens) * G * (D * 2u));
+  if (warp == BT_LOADER_WARP) {
+    if (elect_one()) {
+      // Q: box_tokens tokens from tok0 on, heads hk G .. hk G + G - 1, one box per 64-column panel; the box lands as
+      // rows (token, head) = stacked-row order.  Rows of the Q buffer beyond the box are never written: they belong
+      // to no row of this tile and whatever the tensor cores make of them is never used.
+      mbar_expect_tx(bar(BT_Q_FULL), static_cast<uint32_t>(p.box_tokens) * G * (D * 2u));
 #pragma unroll
-    for (int c = 0; c < Cfg::PANELS; ++c)
-      tma_load_4d(sQ + c * BT_PANEL_BYTES, &L_.tm_q, bar(BT_Q_FULL), c * 64, hk * G, tok0, 0);
-    for (int i = 0; i < pre_issued; ++i) {
-      const bool is_v = i > 0 && (i & 1) == 0;
-      load_kv(is_v, i, BtTile{BT_PREFIX, p0 + (is_v ? i / 2 - 1 : (i + 1) / 2), 0});
+      for (int c = 0; c < Cfg::PANELS; ++c)
+        tma_load_4d(sQ + c * BT_PANEL_BYTES, &L_.tm_q, bar(BT_Q_FULL), c * 64, hk * G, tok0, 0);
+      for (int i = 0; i < pre_issued; ++i) {
+        const bool is_v = i > 0 && (i & 1) == 0;
+        load_kv(is_v, i, BtTile{BT_PREFIX, p0 + (is_v ? i / 2 - 1 : (i + 1) / 2), 0});
+      }
     }
   } else if (warp == 0) {
     // ---- lengths and tile counts of the row tile's branches
@@ -275,21 +278,41 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     }
   }
   __syncthreads();
-  const int s0 = suffix_share[0];
-  const int Tall = npre + suffix_share[1];
-  // Entry `s` of this CTA's list: its prefix share first, then its share of the suffix part: the step's block (fused
-  // write only), then the suffix tiles of the row tile's branches.  A role walks the list in increasing order and
-  // keeps the branch it has reached in `cursor`.
-  auto tile_at = [&](int s, int& cursor) {
-    if (s < npre) return BtTile{BT_PREFIX, p0 + s, min(P - (p0 + s) * BT_BN, BT_BN)};
-    int g = s0 + (s - npre);
+  const int s0 = suffix_share[0], nsuf = suffix_share[1];
+  const int Tall = npre + nsuf;
+  // branch `lane` of the row tile: its rows in the suffix tiles, the number of its first tile, one past its last
+  const int lane_rows = fused ? len_s[lane] - n : len_s[lane], lane_end = cum_s[lane];
+  const int lane_first = lane > 0 ? cum_s[lane - 1] : 0;
+  // Entry `s` of this CTA's list, for a whole warp.  BT_LEAD prefix tiles, whose loads need no lengths, then two tiles of the
+  // suffix part and two of the prefix in turn (one per stream) while both last, then the rest.  The suffix part is the step's
+  // block (fused write only), then the suffix tiles of the row tile's branches.
+  // The lookup is on the issuers' path, where an access to shared memory takes 100 to 200 cycles: it works on what the lanes
+  // hold.  The prefix comes from L2 (other row tiles read it too), the suffix from HBM: one after the other, HBM was idle
+  // first and then what every tile waited for.  6 layers x 8 kv heads, 16 branches x 20 rows of 69 .. 517, prefix 2048: lookup in
+  // shared memory and one after the other 53.4 us, lookup in the lanes 50.5, and mixed 46.
+  const int lead = min(npre, BT_LEAD), mixed = min(npre - lead, nsuf) >> 1;
+  auto tile_at = [&](int s) {
+    bool prefix = s < lead;
+    int g = s;  // its number among the entries of its kind
+    if (!prefix) {
+      const int q = s - lead, left = npre - lead - 2 * mixed;
+      if (q < 4 * mixed) {
+        prefix = q & 2;
+        g = (q >> 2) * 2 + (q & 1) + (prefix ? lead : 0);
+      } else {
+        prefix = q - 4 * mixed < left;
+        g = q - 2 * mixed + (prefix ? lead : -left);
+      }
+    }
+    if (prefix) return BtTile{BT_PREFIX, p0 + g, min(P - (p0 + g) * BT_BN, BT_BN)};
+    g += s0;
     if (fused) {
       if (g == 0) return BtTile{BT_NEW, 0, nb * n};
       --g;
     }
-    while (cursor < nb - 1 && cum_s[cursor] <= g) ++cursor;
-    const int tile = g - (cursor > 0 ? cum_s[cursor - 1] : 0);
-    return BtTile{cursor, tile, min((fused ? len_s[cursor] - n : len_s[cursor]) - tile * BT_BN, BT_BN)};
+    const int j = __popc(__ballot_sync(0xffffffffu, lane_end <= g));
+    const int tile = g - __shfl_sync(0xffffffffu, lane_first, j);
+    return BtTile{j, tile, min(__shfl_sync(0xffffffffu, lane_rows, j) - tile * BT_BN, BT_BN)};
   };
   auto k_load = [&](int s) { return max(2 * s - 1, 0); };  // the number of a tile's load
   auto v_load = [&](int s) { return min(2 * s + 2, 2 * Tall - 1); };
@@ -298,25 +321,24 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   if (warp == BT_LOADER_WARP) {
     // =============================================================== loader
     reg_dec<BT_REGS_OTHER>();
-    if (lane == 0) {
-      bool ok = true;
-      int i = pre_issued, k_cursor = 0, v_cursor = 0;
-      for (; i < 2 * Tall; ++i) {
-        const bool is_v = i == 2 * Tall - 1 || (i > 0 && (i & 1) == 0);
-        const BtTile e = is_v ? tile_at(i == 2 * Tall - 1 ? Tall - 1 : i / 2 - 1, v_cursor) : tile_at((i + 1) / 2, k_cursor);
-        const int slot = load_slot(i);
-        if (i >= SLOTS) ok = mbar_wait(bar(BT_EMPTY + slot), (i / SLOTS - 1) & 1, abort_flag, p.status, wl);
-        if (!ok) break;
-        load_kv(is_v, slot, e);
-      }
-      if (*abort_flag) {
-        // wait (bounded) until every copy this thread started has landed before shared memory is released
-        int dummy = 0;
-        volatile int* none = &dummy;
-        for (int j = max(0, i - SLOTS); j < i; ++j)
-          mbar_wait(bar(BT_FULL + load_slot(j)), (j / SLOTS) & 1, none, nullptr);
-        mbar_wait(bar(BT_Q_FULL), 0, none, nullptr);
-      }
+    const bool leader = elect_one();
+    bool ok = true;
+    int i = pre_issued;
+    for (; i < 2 * Tall; ++i) {
+      const bool is_v = i == 2 * Tall - 1 || (i > 0 && (i & 1) == 0);
+      const BtTile e = tile_at(i == 2 * Tall - 1 ? Tall - 1 : is_v ? i / 2 - 1 : (i + 1) / 2);
+      const int slot = load_slot(i);
+      if (i >= SLOTS) ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_EMPTY + slot), (i / SLOTS - 1) & 1, abort_flag, p.status, wl));
+      if (!ok) break;
+      if (leader) load_kv(is_v, slot, e);
+    }
+    if (leader && *abort_flag) {
+      // wait (bounded) until every copy this thread started has landed before shared memory is released
+      int dummy = 0;
+      volatile int* none = &dummy;
+      for (int j = max(0, i - SLOTS); j < i; ++j)
+        mbar_wait(bar(BT_FULL + load_slot(j)), (j / SLOTS) & 1, none, nullptr);
+      mbar_wait(bar(BT_Q_FULL), 0, none, nullptr);
     }
     __syncwarp();
   } else if (warp == BT_PATCH_WARP) {
@@ -325,9 +347,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     // older one); before that, where the last 16-key group of a tile is not full, zeros into the rest of the group.
     reg_dec<BT_REGS_OTHER>();
     bool ok = true;
-    int cursor = 0;
     for (int s = 0; s < Tall && ok; ++s) {
-      const BtTile e = tile_at(s, cursor);
+      const BtTile e = tile_at(s);
       const int i = v_load(s), slot = load_slot(i);
       ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
       if (!ok) break;
@@ -354,11 +375,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const bool leader = elect_one();
     const uint32_t s_col = tmem + BT_S_COL, q_lo = tc_desc_lo(sQ, 16);
     bool ok = true;
-    int turn = 0, cursor = 0;
+    int turn = 0;
     ok = mbar_wait(bar(BT_Q_FULL), 0, abort_flag, p.status, wl);  // (also when the list is empty: the copy must land)
     for (int s = 0; s < Tall; ++s) {
       const int i = k_load(s), slot = load_slot(i);
-      const BtTile e = tile_at(s, cursor);
+      const BtTile e = tile_at(s);
       const uint32_t idesc_qk = tc_idesc_bf16(BT_BM, e.groups() * 16, false, false);
       ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
       if (s > 0) named_sync(NB_S_FREE + ((s - 1) & 1), 160);
@@ -390,12 +411,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     constexpr uint32_t idesc_pv = tc_idesc_bf16(BT_BM, D, false, true);
     const bool leader = elect_one();
     bool ok = true;
-    int cursor = 0;
     for (int s = 0; s < Tall; ++s) {
       const int slot = load_slot(v_load(s)), x = s & 1;
       const uint32_t v_lo = tc_desc_lo(sKV + slot * TILE_BYTES, BT_PANEL_BYTES);
       const uint32_t o_col = tmem + BT_O_COL0 + x * 128, p_col = tmem + BT_P_COL0 + x * 64;
-      const BtTile e = tile_at(s, cursor);
+      const BtTile e = tile_at(s);
       const int groups = e.groups();
       ok = __all_sync(0xffffffffu, ok && count_spin_wait(v_ready, s + 1, abort_flag, p.status, wl) >= 0);
       named_sync(NB_P_EARLY + x, 160);  // the first 96 keys while the softmax finishes the last 32
@@ -433,6 +453,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     int ri;
     const int rb = p.by_q_len.divmod(tok0 + p.by_group.div(row_in_tile), ri);  // branch and draft row of this row
     const int rj = row_valid ? rb - b_first : -1;    // the row's branch as an index into the tile's branches
+    const int own_rows = row_valid ? len_s[rj] - n : 0;  // rows of its branch before the step's block
     // draft rows of the block this row may see, as bits: its ancestors and itself (a chain: rows 0..i)
     const uint32_t tm = !row_valid ? 0u
                         : (p.tree_mask ? __ldg(p.tree_mask + static_cast<int64_t>(rb) * n + ri) : (2u << ri) - 1u) &
@@ -443,7 +464,6 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const float c = p.scale_log2;
     float m_ref = -INFINITY, l = 0.f;
     bool ok = true;
-    int cursor = 0;
     const int Tx = T[x];
     auto signal = [&](int id) {
       tc_fence_before();
@@ -453,7 +473,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     for (int j = 0; j < Tx; ++j) {
       // ---- which columns of the tile this row sees (a row beyond the tile's rows sees nothing); worked out while
       // the tensor cores still compute the tile's scores
-      const BtTile e = tile_at(2 * j + x, cursor);
+      const BtTile e = tile_at(2 * j + x);
       const int key0 = e.tile * BT_BN;
       ColumnBits allow = {0u, 0u, 0u, 0u};
       // a whole prefix tile is seen by every row there is
@@ -476,7 +496,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
         } else if (e.seg == BT_NEW) {
           col = rj * n;
         } else if (e.seg == rj) {
-          cnt = len_s[rj] - n - key0;
+          cnt = own_rows - key0;
           col = fused ? NONE : cnt;
         }
         if (!row_valid) cnt = 0, col = NONE;

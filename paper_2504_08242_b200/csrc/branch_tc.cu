@@ -57,9 +57,10 @@ constexpr int BT_MIN_BATCHED_LAYERS = 3;
 
 struct BtParams {
   int n_branches, q_len, q_heads, group, kv_heads;
-  FastDiv by_group, by_q_len, by_row_tiles;
+  FastDiv by_group, by_q_len, by_row_tiles, by_layer_units;
   int prefix_len, max_suffix_len;
   int row_tiles;          // row tiles per kv head
+  int whole_units;        // units of all layers that one CTA walks
   int branches_per_tile;  // whole branches per row tile (slices_per_branch == 1)
   int slices_per_branch;  // > 1: a branch has more than 128 rows and is cut into 128-row slices
   int box_tokens;         // tokens in the Q box
@@ -70,11 +71,11 @@ struct BtParams {
   const uint32_t* tree_mask;  // nullable: [n_branches][q_len] ancestor bit masks of the draft block
   int64_t sb, sh, sr;         // strides of the suffix cache
   int* status;
-  float* part;  // ctas_per_unit > 1: [layers][units][ctas_per_unit][D / 4 column chunks][128 rows] float4, a CTA's partial accumulator
-  float* ml;    //                    [layers][units][ctas_per_unit][128 rows] (m, l)
+  float* part;  // [shared units][C][D / 4 column chunks][128 rows] float4, a CTA's partial accumulator
+  float* ml;    // [shared units][C][128 rows] (m, l)
 };
 
-// What differs between the layers of one launch (blockIdx.y).
+// What differs between the layers of one launch.
 struct BtLayer {
   CUtensorMap tm_q, tm_pk, tm_pv, tm_sk, tm_sv;
   CUtensorMap tm_nk, tm_nv;  // k_new / v_new
@@ -137,13 +138,13 @@ struct BtTile {
   __device__ __forceinline__ int groups() const { return (valid + 15) >> 4; }
 };
 
-// C: cluster size = CTAs per unit.
+// C: cluster size = CTAs per shared unit.  The units of all layers are numbered through; the first whole_units of them are
+// walked by one CTA each (C of them make a cluster only in name), the others by a cluster each.
 template <int D, int NL, int C>
 __global__ void __launch_bounds__(BT_THREADS, 1)
 branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) {
   using Cfg = BtCfg<D>;
   constexpr int TILE_BYTES = Cfg::TILE_BYTES;
-  const BtLayer& L_ = layers.l[NL == 1 ? 0 : blockIdx.y];
   constexpr int SLOTS = Cfg::SLOTS;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -161,10 +162,13 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   const long long wl = p.wait_limit;
 
   const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int unit = blockIdx.x / C, crank = blockIdx.x % C;  // clusters are consecutive CTAs: crank is the cluster rank
-  int rt;
+  const bool shared = C > 1 && blockIdx.x >= static_cast<unsigned>(p.whole_units);
+  const int share = shared ? (blockIdx.x - p.whole_units) / C : 0;  // number among the shared units
+  const int crank = shared ? blockIdx.x % C : 0;                    // rank in its cluster (whole_units is a multiple of C)
+  const int log2c = shared ? (C == 8 ? 3 : C / 2) : 0;              // log2 of the CTAs that walk this unit
+  int unit = shared ? p.whole_units + share : blockIdx.x, rt;
+  const BtLayer& L_ = layers.l[NL == 1 ? 0 : p.by_layer_units.divmod(unit, unit)];
   const int hk = p.by_row_tiles.divmod(unit, rt);
-  const int gunit = blockIdx.y * (gridDim.x / C) + unit;  // over all layers of the launch
   const int n = p.q_len, G = p.group;
   // ---- the row tile: tokens [tok0, tok0 + ntok) of the stacked (branch, draft row) order, all heads of the group
   int b_first, nb, tok0, ntok;
@@ -185,7 +189,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   const bool fused = L_.k_new != nullptr;
   // this CTA's share of the prefix tiles: known without any memory access
   const int Tp = (P + BT_BN - 1) / BT_BN;
-  const int p0 = Tp * crank / C, npre = Tp * (crank + 1) / C - p0;
+  const int p0 = (Tp * crank) >> log2c, npre = ((Tp * (crank + 1)) >> log2c) - p0;
 
   // ---- set-up
   if (threadIdx.x == 0) {
@@ -272,9 +276,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     cum_s[lane] = cum;
     if (lane == 31) {  // this CTA's share of the unit's suffix part
       cum += fused ? 1 : 0;
-      const int s0 = static_cast<int>(static_cast<int64_t>(cum) * crank / C);
+      const int s0 = static_cast<int>((static_cast<int64_t>(cum) * crank) >> log2c);
       suffix_share[0] = s0;
-      suffix_share[1] = static_cast<int>(static_cast<int64_t>(cum) * (crank + 1) / C) - s0;
+      suffix_share[1] = static_cast<int>((static_cast<int64_t>(cum) * (crank + 1)) >> log2c) - s0;
     }
   }
   __syncthreads();
@@ -537,10 +541,10 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     // the branches took 10 us).  Nobody reads those rows of the cache in this launch.
     if (ok && fused && (p.slices_per_branch == 1 || rt % p.slices_per_branch == 0)) {
       constexpr int CH = Cfg::CH;
-      const int pieces = nb > crank ? ((nb - crank + C - 1) / C) * n * CH : 0;
+      const int pieces = nb > crank ? ((nb - crank + (1 << log2c) - 1) >> log2c) * n * CH : 0;
 #pragma unroll 2
       for (int idx = threadIdx.x; idx < pieces; idx += 256) {
-        const int c16 = idx % CH, t = idx / CH, jb = crank + t / n * C, r = t % n, b = b_first + jb;
+        const int c16 = idx % CH, t = idx / CH, jb = crank + (t / n << log2c), r = t % n, b = b_first + jb;
         const int64_t src = ((static_cast<int64_t>(b) * n + r) * p.kv_heads + hk) * D + c16 * 8;
         const int64_t dst = b * p.sb + hk * p.sh + static_cast<int64_t>(len_s[jb] - n + r) * p.sr + c16 * 8;
         const uint4 kk = __ldg(reinterpret_cast<const uint4*>(L_.k_new + src));
@@ -603,11 +607,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       const int b = p.by_q_len.divmod(tok, i);
       L_.lse[(static_cast<int64_t>(b) * p.q_heads + hq) * n + i] = value * 0.69314718055994530942f;
     };
-    if constexpr (C > 1) {
+    if (shared) {
       // ---- this CTA's partial of the row -> scratch, unnormalised, relative to the row's maximum over this CTA's tiles, as
       // [column chunk][row] float4 so that a warp writes 512 contiguous bytes
-      float4* gpart = reinterpret_cast<float4*>(p.part + (static_cast<size_t>(gunit) * C + crank) * Cfg::PART_FLOATS);
-      float2* gml = reinterpret_cast<float2*>(p.ml + (static_cast<size_t>(gunit) * C + crank) * BT_ML_FLOATS);
+      float4* gpart = reinterpret_cast<float4*>(p.part + (static_cast<size_t>(share) * C + crank) * Cfg::PART_FLOATS);
+      float2* gml = reinterpret_cast<float2*>(p.ml + (static_cast<size_t>(share) * C + crank) * BT_ML_FLOATS);
       if (warp_has_row) {
         combine([&](int col, float4 v) {
           if (row_valid) gpart[col / 4 * BT_BM + row_in_tile] = v;
@@ -624,8 +628,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       constexpr int PER = BT_BM / C, MINE = D / 4 / (2 * C);
       const int row = PER * crank + known_here(threadIdx.x) % PER, sub = known_here(threadIdx.x) / PER;
       if (row < rows_here) {
-        const float2* uml = reinterpret_cast<const float2*>(p.ml + static_cast<size_t>(gunit) * C * BT_ML_FLOATS);
-        const float4* upart = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(gunit) * C * Cfg::PART_FLOATS);
+        const float2* uml = reinterpret_cast<const float2*>(p.ml + static_cast<size_t>(share) * C * BT_ML_FLOATS);
+        const float4* upart = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(share) * C * Cfg::PART_FLOATS);
         float2 ml[C];
         float4 v[MINE][C];
 #pragma unroll
@@ -694,8 +698,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   }
   // (every thread of every CTA passes the cluster's barrier, whatever happened above; the output above is part of the
   // softmax branch because code behind the branches would have to make do with the other roles' registers)
-  if constexpr (C > 1)
-    if (warp >= 8) cluster_sync_all();
+  if (shared && warp >= 8) cluster_sync_all();
 
   // ---- tear-down
   tc_fence_before();
@@ -709,7 +712,8 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
 // ---------------------------------------------------------------- host side
 
 struct BtPlan {
-  int row_tiles, branches_per_tile, slices_per_branch, box_tokens, units, ctas_per_unit;
+  int row_tiles, branches_per_tile, slices_per_branch, box_tokens, units;
+  int cluster, whole_units;  // of the units of all layers, the first whole_units have a CTA each, the others a cluster
   bool ok;
   int64_t estimate_ns;
 };
@@ -735,24 +739,27 @@ static int bt_resident_clusters() {
   return clusters.get(reinterpret_cast<const void*>(branch_tc_kernel<D, NL, C>), C, BT_THREADS, BtCfg<D>::SMEM_BYTES);
 }
 
-// The tiling of one problem and the CTAs per unit, for `layers` problems in one launch: the pair with the shortest
-// estimated time.  A CTA takes 1.35 us per tile of 128 keys (0.95 with head_dim 64; a branch's suffix counted at 0.6 of its
+// The tiling of one problem and the CTAs per unit, for `layers` problems in one launch: the form with the shortest
+// estimated time.  A CTA takes 1.15 us per tile of 128 keys (0.85 with head_dim 64; a branch's suffix counted at 0.6 of its
 // longest possible walk) and a fixed time, larger when a cluster has to exchange partials; more, smaller row tiles walk
-// the prefix more often but may fill the machine better.  Measured (us, tiles per CTA in brackets): 8 kv heads, 128 rows,
-// prefix 1000 11.5 (3), prefix 4000 13.6 (6); 192 rows 12.3 (4), 18.9 (10); 32 kv heads, 128 rows 25.3 (10), 33.5 (16).
+// the prefix more often but may fill the machine better.  Where the units fill the machine more than once, the full waves
+// have a CTA per unit and the rest a cluster each, if these fit in one wave.  Measured (us, tiles per CTA in brackets):
+// 8 kv heads, 128 rows, prefix 1000 11.5 (3), prefix 4000 13.6 (6); 6 layers x 8 kv heads x 3 row tiles, one wave 46 (34); 8
+// layers, two waves of CTAs 75 (2 x 28), one and a rest of 48 units in clusters of two 70 (34 + 17); the same with short
+// suffixes, prefix 3000 71 and 64.
 template <int D, int NL>
 static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_heads, int kv_heads, int q_len,
                       int sm_count, int layers) {
-  constexpr int64_t TILE_NS = D == 128 ? 1350 : 950, ALONE_NS = D == 128 ? 6800 : 6000, CLUSTER_NS = D == 128 ? 8100 : 7600;
-  BtPlan pl = {0, 0, 1, 0, 0, 1, false, 0};
+  constexpr int64_t TILE_NS = D == 128 ? 1150 : 850, ALONE_NS = D == 128 ? 6800 : 6000, CLUSTER_NS = D == 128 ? 8100 : 7600;
+  BtPlan pl = {0, 0, 1, 0, 0, 1, 0, false, 0};
   const int G = q_heads / kv_heads, nG = q_len * G;
   const int64_t Tp = (static_cast<int64_t>(prefix_len) + BT_BN - 1) / BT_BN;
   const int64_t ts_max = (max_suffix_len + BT_BN - 1) / BT_BN;
   const int64_t ts_est = std::max<int64_t>(1, (ts_max * 6 + 9) / 10);
   int64_t best = -1;
   auto consider = [&](int64_t row_tiles, int per_tile, int slices, int box_tokens) {
-    const int64_t units = row_tiles * kv_heads;
-    if (units > (1 << 30)) return;
+    const int64_t units = row_tiles * kv_heads, all = units * layers;
+    if (all > (1 << 30)) return;
     const int64_t walk = Tp + per_tile * ts_est;
     for (int c = 1; c <= 8; c *= 2) {
       if (c > 1 && 2 * c > Tp + ts_max + 1) break;  // no more CTAs than pairs of tiles a unit certainly has
@@ -760,12 +767,14 @@ static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_
                               : c == 2 ? bt_resident_clusters<D, NL, 2>()
                               : c == 4 ? bt_resident_clusters<D, NL, 4>()
                                        : bt_resident_clusters<D, NL, 8>();
-      if (at_once == 0 || (c > 1 && at_once < units)) continue;  // (a layer's clusters are all resident at once)
-      const int64_t waves = (units * layers + at_once - 1) / at_once;
-      const int64_t est = waves * ((walk + c - 1) / c * TILE_NS + (c > 1 ? CLUSTER_NS : ALONE_NS));
+      if (at_once == 0) continue;
+      const int64_t full_waves = all / (at_once * c), whole = c == 1 ? all : full_waves * at_once * c;
+      if (c > 1 && (whole == all || all - whole > at_once)) continue;  // (clusters: one wave, after those of whole units)
+      const int64_t est = c == 1 ? (all + at_once - 1) / at_once * (walk * TILE_NS + ALONE_NS)
+                                 : full_waves * (walk * TILE_NS + ALONE_NS) + (walk + c - 1) / c * TILE_NS + CLUSTER_NS;
       if (best < 0 || est < best) {
         best = est;
-        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, true, est};
+        pl = BtPlan{static_cast<int>(row_tiles), per_tile, slices, box_tokens, static_cast<int>(units), c, static_cast<int>(whole), true, est};
       }
     }
   };
@@ -786,8 +795,8 @@ static BtPlan bt_plan(int prefix_len, int max_suffix_len, int n_branches, int q_
 
 template <int D>
 static size_t bt_scratch_bytes(const BtPlan& pl, int layers) {
-  if (pl.ctas_per_unit <= 1) return 0;
-  return SCRATCH_COUNTER_BYTES + static_cast<size_t>(layers) * pl.units * pl.ctas_per_unit *
+  if (pl.cluster <= 1) return 0;
+  return SCRATCH_COUNTER_BYTES + static_cast<size_t>(layers * pl.units - pl.whole_units) * pl.cluster *
                                      (BtCfg<D>::PART_FLOATS + BT_ML_FLOATS) * sizeof(float);
 }
 
@@ -820,7 +829,8 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   BtPlan pl = bt_plan<D, NL>(prefix_len, max_suffix_len, n_branches, q_heads, suffix.kv_heads, q_len, li.sm_count, layers);
   if (!pl.ok) return cudaErrorInvalidValue;
   // several CTAs per unit exchange partials through the scratch; without enough of it a unit is walked by one CTA
-  if (pl.ctas_per_unit > 1 && (!workspace || bt_scratch_bytes<D>(pl, layers) > workspace_bytes)) pl.ctas_per_unit = 1;
+  const int all_units = layers * pl.units;
+  if (pl.cluster > 1 && (!workspace || bt_scratch_bytes<D>(pl, layers) > workspace_bytes)) pl.cluster = 1, pl.whole_units = all_units;
   const int G = q_heads / suffix.kv_heads;
   const uint64_t tokens = static_cast<uint64_t>(n_branches) * q_len;
   BtLayers<NL> L;
@@ -884,6 +894,8 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   p.by_group = FastDiv(G);
   p.by_q_len = FastDiv(q_len);
   p.by_row_tiles = FastDiv(pl.row_tiles);
+  p.by_layer_units = FastDiv(pl.units);
+  p.whole_units = pl.whole_units;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_limit = wait_limit;
   p.d_suffix_len = d_suffix_len;
@@ -892,18 +904,17 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   p.sh = suffix.sh;
   p.sr = suffix.sr;
   p.status = status;
-  p.part = pl.ctas_per_unit > 1 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES)
-                                : nullptr;
-  p.ml = pl.ctas_per_unit > 1 ? p.part + static_cast<size_t>(layers) * pl.units * pl.ctas_per_unit * BtCfg<D>::PART_FLOATS
-                              : nullptr;
+  const int shares = (all_units - pl.whole_units) * pl.cluster;  // CTAs that share a unit
+  p.part = shares > 0 ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + SCRATCH_COUNTER_BYTES) : nullptr;
+  p.ml = shares > 0 ? p.part + static_cast<size_t>(shares) * BtCfg<D>::PART_FLOATS : nullptr;
   auto launch = [&](auto set_attributes, auto kernel) {
     cudaError_t e = set_attributes();
     if (e != cudaSuccess) return e;
     li.launches += 1;
-    return launch_pdl_cluster(kernel, dim3(static_cast<unsigned>(pl.units) * pl.ctas_per_unit, static_cast<unsigned>(layers)),
-                              dim3(BT_THREADS), BtCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(pl.ctas_per_unit), L, p);
+    return launch_pdl_cluster(kernel, dim3(static_cast<unsigned>(pl.whole_units + shares)), dim3(BT_THREADS), BtCfg<D>::SMEM_BYTES,
+                              st, static_cast<unsigned>(pl.cluster), L, p);
   };
-  switch (pl.ctas_per_unit) {
+  switch (pl.cluster) {
     case 8: return launch(bt_set_attributes<D, NL, 8>, branch_tc_kernel<D, NL, 8>);
     case 4: return launch(bt_set_attributes<D, NL, 4>, branch_tc_kernel<D, NL, 4>);
     case 2: return launch(bt_set_attributes<D, NL, 2>, branch_tc_kernel<D, NL, 2>);

@@ -11,7 +11,7 @@
 // in tiles of 128 keys: a prefix tile is visible to every row, a suffix tile to the rows of its branch below
 // their causal limit (or tree mask).  A prefix K/V tile is therefore fetched once per row tile, not once per branch.
 //
-// C CTAs, a thread-block cluster, share a unit: the prefix tiles are cut into equal contiguous
+// A unit is walked by one CTA or shared by C CTAs, a thread-block cluster: the prefix tiles are cut into equal contiguous
 // ranges, one per CTA, and so are the suffix tiles (the prefix share does not depend on the device-side lengths,
 // so its first loads are in flight while the lengths arrive).  Inside a CTA:
 //   loader warp  : TMA (tiled, 128-byte swizzle) Q once -- one box [tokens][G heads][64] lands in stacked-row
@@ -21,7 +21,7 @@
 //                  weights are 0, but 0 x NaN must not reach an accumulator)
 //   MMA warps    : one thread issues S = Q K^T, another O += P V (tcgen05.mma over the 16-key groups that hold keys)
 //   softmax WGs  : two warpgroups run two independent online-softmax streams over the even and the odd tiles of
-//                  the CTA's list (one thread per row); a warp none of whose rows sees a tile only zeroes its P
+//                  the CTA's list, which mixes prefix and suffix tiles (one thread per row); a warp none of whose rows sees a tile only zeroes its P
 // TMEM (512 columns): O_0 | O_1 (128 each) | S (128) | P_0 | P_1 (64 each); the one S buffer goes back and forth between
 // the streams, as in the two-tile prefill kernel.
 // With the fused KVCache write the step's K/V block of all the tile's branches is one more tile, fetched from k_new /

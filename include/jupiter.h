@@ -210,10 +210,10 @@ jupiter_status jupiter_branch_append_attn(jupiter_ctx* ctx, const void* q, const
  * KVCaches).  Layer l has its own query block, K/V block, prefix cache, suffix cache and outputs; all layers have
  * the same geometry (head counts, head_dim, capacities, strides), the same branch lengths and the same scale.
  * Same result, layer by layer, as n_layers calls of jupiter_branch_append_attn -- the layers must not depend on one
- * another's outputs inside the call (their Q/K/V blocks are ready beforehand) -- but the layers share launches: with
- * few stacked query rows per kv head (decode) up to 16 layers run as ONE kernel launch, so the time between
- * dependent launches is paid once per 16 layers instead of once per layer; shapes that take the other kernels are
- * enqueued layer by layer.
+ * another's outputs inside the call (their Q/K/V blocks are ready beforehand) -- but the layers share launches: up to
+ * 16 layers run as ONE kernel launch (with many stacked query rows per kv head from three layers on), so the time
+ * between dependent launches is paid once per 16 layers instead of once per layer; shapes that take the split-KV
+ * kernel are enqueued layer by layer.
  *   layers: HOST array of n_layers entries (read during the call only); prefix may be NULL when prefix_len == 0;
  *           lse may be NULL.  Other arguments and errors as for jupiter_branch_append_attn; every layer's
  *           descriptors are checked before anything is enqueued, and a layer whose geometry differs from
@@ -234,10 +234,11 @@ jupiter_status jupiter_branch_append_attn_layers(jupiter_ctx* ctx, const jupiter
 
 /* Tuning and testing aid; the paper has no counterpart.  The branch calls (jupiter_branch_attn, _tree,
  * jupiter_branch_append_attn) pick one of three kernels from the shape: a streaming kernel for few stacked
- * query rows per kv head (decode), a tensor-core kernel (tcgen05 / TMEM) for many rows with head_dim 128, and a
- * general split-KV kernel.  This call pins the choice for later calls on `ctx`; JUPITER_BRANCH_AUTO restores the
- * default.  A call whose shape the pinned kernel cannot take returns JUPITER_ERR_UNSUPPORTED (the tensor-core
- * kernel needs head_dim 128, scale > 0, and either q_len * group <= 128 or a group size q_heads / kv_heads that
+ * query rows per kv head (decode), a tensor-core kernel (tcgen05 / TMEM) for many rows -- whichever of the two has the
+ * shorter estimated time -- and a general split-KV kernel where the tensor-core kernel cannot take the call.  This call
+ * pins the choice for later calls on `ctx`; JUPITER_BRANCH_AUTO restores the default.  A call whose shape the pinned
+ * kernel cannot take returns JUPITER_ERR_UNSUPPORTED (the tensor-core kernel, pinned, needs head_dim 128, scale > 0,
+ * and either q_len * group <= 128 or a group size q_heads / kv_heads that
  * divides 128).  All three give the same result up to rounding. */
 typedef enum {
   JUPITER_BRANCH_AUTO = 0,

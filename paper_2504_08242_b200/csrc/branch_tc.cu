@@ -49,7 +49,6 @@ constexpr int BT_BM = 128;             // stacked rows per tile (at most)
 constexpr int BT_BN = 128;             // keys per KV tile
 constexpr int BT_PANEL_BYTES = 16384;  // 128 rows x 64 elements
 constexpr int BT_MAX_SLOTS = 12;
-constexpr int BT_LEAD = 4;             // prefix tiles at the front of a CTA's list (even: a pair of tiles is one per stream)
 constexpr int BT_MAX_BRANCHES = 32;    // branches in one row tile
 constexpr int BT_ML_FLOATS = BT_BM * 2;  // one CTA's (m, l) pairs
 // Layers of one call share a launch from this many on.
@@ -95,6 +94,11 @@ struct BtLayers {
 template <int D>
 struct BtCfg {
   static constexpr int SLOTS = D == 128 ? 6 : 12;
+  // Prefix tiles at the front of a CTA's list: as many as the first SLOTS loads belong to (K_0 K_1 V_0 K_2 V_1 ..
+  // K_SLOTS/2), and even: a pair of tiles is one per stream.  (head_dim 64, 16 branches x 20 rows, 8 layers, prefix 3000,
+  // 73.0 us; with 4 tiles in front and only their loads early 73.5.)
+  static constexpr int LEAD = D == 128 ? 4 : 8;
+  static_assert(LEAD % 2 == 0 && 2 * LEAD - 1 >= SLOTS, "every slot is filled before the lengths are known");
   static constexpr int TILE_BYTES = BT_BN * D * 2;
   static constexpr int PANELS = D / 64;
   static constexpr int CH = D / 8;  // 16-byte pieces per K/V row
@@ -243,7 +247,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   // 16 branches x 20 rows 94.1 -> 90.4 us; head_dim 64, with twice as many slots, 16 branches x 20 rows, prefix 1500
   // 16.0 -> 15.4 us.)
   auto load_slot = [&](int i) { return i % SLOTS; };
-  const int pre_issued = min(max(2 * npre - 1, 0), SLOTS);  // loads whose place in that order does not depend on the lengths
+  // The list starts with `lead` prefix tiles (see tile_at): their loads, but for the last one's V tile, have places in that
+  // order that do not depend on the lengths.
+  const int lead = min(npre, Cfg::LEAD), pre_issued = min(max(2 * lead - 1, 0), SLOTS);
   if (warp == BT_LOADER_WARP) {
     if (elect_one()) {
       // Q: box_tokens tokens from tok0 on, heads hk G .. hk G + G - 1, one box per 64-column panel; the box lands as
@@ -287,14 +293,14 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   // branch `lane` of the row tile: its rows in the suffix tiles, the number of its first tile, one past its last
   const int lane_rows = fused ? len_s[lane] - n : len_s[lane], lane_end = cum_s[lane];
   const int lane_first = lane > 0 ? cum_s[lane - 1] : 0;
-  // Entry `s` of this CTA's list, for a whole warp.  BT_LEAD prefix tiles, whose loads need no lengths, then two tiles of the
+  // Entry `s` of this CTA's list, for a whole warp.  `lead` prefix tiles, whose loads need no lengths, then two tiles of the
   // suffix part and two of the prefix in turn (one per stream) while both last, then the rest.  The suffix part is the step's
   // block (fused write only), then the suffix tiles of the row tile's branches.
   // The lookup is on the issuers' path, where an access to shared memory takes 100 to 200 cycles: it works on what the lanes
   // hold.  The prefix comes from L2 (other row tiles read it too), the suffix from HBM: one after the other, HBM was idle
   // first and then what every tile waited for.  6 layers x 8 kv heads, 16 branches x 20 rows of 69 .. 517, prefix 2048: lookup in
   // shared memory and one after the other 53.4 us, lookup in the lanes 50.5, and mixed 46.
-  const int lead = min(npre, BT_LEAD), mixed = min(npre - lead, nsuf) >> 1;
+  const int mixed = min(npre - lead, nsuf) >> 1;
   auto tile_at = [&](int s) {
     bool prefix = s < lead;
     int g = s;  // its number among the entries of its kind

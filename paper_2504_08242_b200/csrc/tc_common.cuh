@@ -109,7 +109,6 @@ __device__ __forceinline__ int count_read(uint32_t addr) {
   asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-// The same word without ordering, for hints.
 // The operands of the tcgen05 instructions live in registers that a warp shares.  Values read from lane 0, and one lane
 // picked by elect.sync instead of by its number, let the compiler keep them there; otherwise every issue first moves them
 // over, and the issuing threads are what the tensor cores wait for.  Two-tile prefill kernel, 4 x 32 heads, 8192 tokens in
@@ -132,6 +131,7 @@ __device__ __forceinline__ bool elect_one() {  // (all lanes of the warp take pa
   return r != 0;
 }
 
+// Such a word without ordering, for hints.
 __device__ __forceinline__ void flag_write(uint32_t addr, int value) {
   asm volatile("st.relaxed.cta.shared::cta.b32 [%0], %1;\n" ::"r"(addr), "r"(value) : "memory");
 }
@@ -322,9 +322,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+template <bool KEEP_NAN = false>  // KEEP_NAN: NaN if an operand is
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
   float r;
-  asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  if constexpr (KEEP_NAN) asm("max.NaN.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  else asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
 // 2^x for a packed pair on the FMA pipe instead of the special-function unit (which is the softmax's bottleneck:

@@ -73,28 +73,32 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
   tc_wait_ld();
   loaded();
   // ---- row maximum: 3-input max, 32 + 8 + 8 + 3 + 3 + 1 operations in chains of depth 5
+  auto max3 = [](float a, float b, float c) { return fmax3<PARTIAL>(a, b, c); };
   float mx;
   {
     float a[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k)
-      a[k] = fmax3(__uint_as_float(sv[4 * k]), __uint_as_float(sv[4 * k + 1]), __uint_as_float(sv[4 * k + 2]));
+      a[k] = max3(__uint_as_float(sv[4 * k]), __uint_as_float(sv[4 * k + 1]), __uint_as_float(sv[4 * k + 2]));
     float b[8], d[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      b[k] = fmax3(fmax3(a[4 * k], a[4 * k + 1], a[4 * k + 2]), a[4 * k + 3], __uint_as_float(sv[16 * k + 3]));
-      d[k] = fmax3(__uint_as_float(sv[16 * k + 7]), __uint_as_float(sv[16 * k + 11]), __uint_as_float(sv[16 * k + 15]));
+      b[k] = max3(max3(a[4 * k], a[4 * k + 1], a[4 * k + 2]), a[4 * k + 3], __uint_as_float(sv[16 * k + 3]));
+      d[k] = max3(__uint_as_float(sv[16 * k + 7]), __uint_as_float(sv[16 * k + 11]), __uint_as_float(sv[16 * k + 15]));
     }
-    mx = fmaxf(fmax3(fmax3(b[0], b[1], b[2]), fmax3(b[3], b[4], b[5]), fmaxf(b[6], b[7])),
-               fmax3(fmax3(d[0], d[1], d[2]), fmax3(d[3], d[4], d[5]), fmaxf(d[6], d[7])));
+    mx = max3(max3(max3(b[0], b[1], b[2]), max3(b[3], b[4], b[5]), b[6]), b[7],
+              max3(max3(d[0], d[1], d[2]), max3(d[3], d[4], d[5]), max3(d[6], d[7], d[7])));
   }
   const float mxs = (PARTIAL && !row_sees) ? -INFINITY : mx * c;
   // lazy reference: it only moves when the maximum outgrew it by 2^8 (a row that has seen nothing keeps -inf,
   // and its first visible score moves it because -inf + 8 is still -inf)
   const bool grow = mxs > m_ref + TC_RESCALE_THRESHOLD;
+  // A row that sees nothing of the tile is hidden by adding -inf to its scores, which NaN and +inf (another branch's keys)
+  // would survive: such scores are cleared.  Tested on the maximum, so that finite ones cost nothing.
+  const bool clear = PARTIAL && !row_sees && !(mx < INFINITY);
   if (!o_here) wait_o();
   tc_fence_after();
-  if (__any_sync(0xffffffffu, grow)) {
+  if (__any_sync(0xffffffffu, grow || clear)) {
     const float alpha = grow ? fast_exp2(m_ref - mxs) : 1.f;
     l *= alpha;
     if (grow) m_ref = mxs;
@@ -108,6 +112,10 @@ __device__ __forceinline__ void softmax_tile_row(uint32_t tS, uint32_t tP, uint3
         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
         tmem_st32(tO + q4 * 32, o);
       }
+    }
+    if (PARTIAL && clear) {
+#pragma unroll
+      for (int i = 0; i < 128; ++i) sv[i] = 0u;
     }
   }
   // ---- P

@@ -233,16 +233,15 @@ __device__ __forceinline__ bool frag_decide(const float (&mxs)[2], float (&m_ref
   return true;
 }
 
-// Which of a tile's 32 column pairs per thread (step k, row e) take their exponentials on the FMA pipe: a quarter
-// (more brought nothing: the loop is bound by dependent-issue latency, not by the special-function unit alone).
-__device__ __forceinline__ constexpr bool frag_exp_on_fma(int k, int e) { return e == 1 && (k & 1) != 0; }
-
 // P = exp2(s c - m_ref) of a tile held in fragments, as bf16 pairs over the first 64 columns of its S buffer, row
 // sums into l (the stores are issued, not waited for), with the next tile's row maxima worked in: nxt is a fragment
 // load in flight (or stale registers when there
 // is no next tile; the result is then unused).  It is waited for after the fourth of the sixteen steps, masked if
 // need be (mask_next(), warp-uniform and rare), and its 2 x 32 values are folded into running maxima a few per step,
 // so that their arithmetic issues in the gaps of the exponentials instead of after them.  mxs_next: maxima times c.
+// (A quarter of the exponentials as a degree-3 polynomial on the FMA pipe gained 1 to 1.5 % with head_dim 128 and nothing with
+// 64 -- four prompts of 8192 tokens in chunks of 128 2417 against 2448 us, 3000 tokens in chunks of 448 with head_dim 64 124 against
+// 123 -- but its 7.5e-5 showed in the log-sum-exps, 7e-5 off instead of 3e-6, and it lost NaN scores.)
 template <class MaskNext>
 __device__ __forceinline__ void frag_exp_store_max(const uint32_t (&sv)[64], uint32_t tS, float c, const float (&m_ref)[2],
                                                    float (&l)[2], uint32_t (&nxt)[64], bool next_masked,
@@ -265,15 +264,9 @@ __device__ __forceinline__ void frag_exp_store_max(const uint32_t (&sv)[64], uin
     for (int e = 0; e < 2; ++e) {
       const uint64_t x =
           fma2(pack2(__uint_as_float(sv[4 * k + 2 * e]), __uint_as_float(sv[4 * k + 2 * e + 1])), c2, nm2[e]);
-      float p0, p1;
-      if (frag_exp_on_fma(k, e)) {
-        unpack2(exp2_poly_pair(x), p0, p1);
-      } else {
-        float x0, x1;
-        unpack2(x, x0, x1);
-        p0 = fast_exp2(x0);
-        p1 = fast_exp2(x1);
-      }
+      float x0, x1;
+      unpack2(x, x0, x1);
+      const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
       lacc[e][k & 1] = add2(lacc[e][k & 1], pack2(p0, p1));
       w[2 * k + e] = pack_bf16(p0, p1);
     }

@@ -322,7 +322,7 @@ static jupiter_status branch_attn_impl(jupiter_ctx* ctx, const void* q, const ju
   // kernel (which adapts to the scratch it is given); the rest to the split-KV kernel, the only one that can find the
   // scratch too small
   DeviceGuard guard(ctx->device);
-  const bool tc_ok = jup::branch_tc_supported(sfx, n_branches, q_heads, q_len, scale);
+  const bool tc_ok = jup::branch_tc_supported(pfx, sfx, n_branches, q_heads, q_len, scale);
   bool use_stream, use_tc;
   switch (ctx->branch_kernel) {
     case JUPITER_BRANCH_STREAM: use_stream = true, use_tc = false; break;
@@ -403,7 +403,7 @@ jupiter_status jupiter_branch_append_attn_layers(jupiter_ctx* ctx, const jupiter
                                    static_cast<const bf16*>(L.v_new), pfx.k, pfx.v, sfx.k, sfx.v, L.out, L.lse};
   }
   DeviceGuard guard(ctx->device);
-  const bool tc_ok = jup::branch_tc_supported(sfx0, n_branches, q_heads, q_len, scale);
+  const bool tc_ok = jup::branch_tc_supported(pfx0, sfx0, n_branches, q_heads, q_len, scale);
   const bool stream_kernel =
       prefer_stream(ctx, tc_ok, n_branches, q_heads, sfx0, q_len, prefix_len, max_suffix_len, n_layers);
   if (ctx->branch_kernel == JUPITER_BRANCH_AUTO && (stream_kernel || tc_ok)) {

@@ -806,8 +806,14 @@ static size_t bt_scratch_bytes(const BtPlan& pl, int layers) {
                                      (BtCfg<D>::PART_FLOATS + BT_ML_FLOATS) * sizeof(float);
 }
 
-bool branch_tc_supported(const CacheView& suffix, int n_branches, int q_heads, int q_len, float scale) {
+bool branch_tc_supported(const CacheView& prefix, const CacheView& suffix, int n_branches, int q_heads, int q_len,
+                         float scale) {
   if (!(scale > 0.f) || !(scale < INFINITY) || encode_fn() == nullptr) return false;
+  // (a stride that no tensor map carries, as of the batch of a cache for one branch, which nothing else looks at: the other
+  // kernels take the call)
+  if (!stride_encodable(suffix.sr) || !stride_encodable(suffix.sh) || !stride_encodable(suffix.sb) ||
+      !stride_encodable(prefix.sr) || !stride_encodable(prefix.sh))
+    return false;
   const int G = q_heads / suffix.kv_heads;
   const int64_t nG = static_cast<int64_t>(q_len) * G;
   if (nG > BT_BM && BT_BM % G != 0) return false;

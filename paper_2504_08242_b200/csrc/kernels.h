@@ -117,12 +117,13 @@ cudaError_t launch_branch_stream(const bf16* q, const CacheView& prefix, int pre
                                  cudaStream_t st, LaunchInfo& li, const bf16* k_new = nullptr,
                                  const bf16* v_new = nullptr);
 
-// Branch attention on tcgen05 / TMEM for many stacked rows per kv head (positive finite scale; a
+// Branch attention on tcgen05 / TMEM for many stacked rows per kv head (positive finite scale, TMA-encodable strides; a
 // branch's q_len x group rows must fit a 128-row tile or the group size must divide 128): units of (kv head, row
 // tile) walk prefix + suffixes with one softmax state per row; the CTAs that share a unit form a thread-block
 // cluster and exchange their partials through the scratch (with too little of it a unit is walked by one CTA, so
 // the call never fails for lack of scratch).  Both calls need the target device current.
-bool branch_tc_supported(const CacheView& suffix, int n_branches, int q_heads, int q_len, float scale);
+bool branch_tc_supported(const CacheView& prefix, const CacheView& suffix, int n_branches, int q_heads, int q_len,
+                         float scale);
 // Several layers of the same geometry (prefix / suffix, whose own k / v are ignored) share a launch.
 cudaError_t launch_branch_tc_layers(const BranchLayerTensors* layers, int n_layers, const CacheView& prefix, int prefix_len,
                                     const CacheView& suffix, const int32_t* d_suffix_len, const uint32_t* d_tree_mask,

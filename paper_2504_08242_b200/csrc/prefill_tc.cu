@@ -501,9 +501,8 @@ static cudaError_t launch_pairs(int64_t ctas, cudaStream_t st, const CUtensorMap
 bool prefill_tc_supported(const CacheView& c, float scale) {
   // a positive finite scale, and strides a tensor map can carry (multiples of 16 bytes below 2^40;
   // the 16-byte rule is part of every cache descriptor already)
-  auto encodable = [](int64_t elems) { return static_cast<uint64_t>(elems) * 2 < (1ull << 40); };
-  return scale > 0.f && scale < INFINITY && encode_fn() != nullptr && encodable(c.sr) &&
-         encodable(c.sh) && encodable(c.sb);
+  return scale > 0.f && scale < INFINITY && encode_fn() != nullptr && stride_encodable(c.sr) &&
+         stride_encodable(c.sh) && stride_encodable(c.sb);
 }
 
 // How a call is laid out: which kernel, how many of a kv head's query heads share a query tile, how many CTAs share its

@@ -24,6 +24,9 @@ inline EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// Whether a tensor map can carry a stride of a cache, in bf16 elements (they are multiples of 8 already).
+inline bool stride_encodable(int64_t elems) { return static_cast<uint64_t>(elems) * 2 < (1ull << 40); }
+
 // dims: extents, innermost first; strides_bytes: of dimensions 1..3 (multiples of 16, below 2^40; a dimension of
 // extent 1 may pass 0); box: the tile, innermost first (inner box = 128 bytes).  Out-of-range elements of a load
 // read as zero, those of a store are not written.

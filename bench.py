@@ -590,7 +590,7 @@ TRAFFIC_PROFILES = {
     "cfg3_c512": ("prefill_tc_kernel_cfg3_c512.md", PREFILL_SOURCES),
     "cfg3_c1024": ("prefill_tc_kernel_cfg3_c512.md", PREFILL_SOURCES),
     "cfg4": ("branch_stream_kernel_cfg4.md", ["branch_stream.cu", "tc_common.cuh", "common.cuh"]),
-    "cfg5": ("branch_tc_kernel_cfg5.md", ["branch_tc.cu"] + TC_SOURCES),
+    "cfg5": ("branch_tc_kernel_cfg5.md", ["branch_tc.cu", "tile_ring.h"] + TC_SOURCES),
 }
 
 

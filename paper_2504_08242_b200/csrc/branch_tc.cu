@@ -41,6 +41,7 @@
 #include "kernels.h"
 #include "tc_common.cuh"
 #include "tc_softmax.cuh"
+#include "tile_ring.h"
 #include "tmap.h"
 
 namespace jup {
@@ -127,7 +128,8 @@ enum {
   BT_S_FULL = BT_EMPTY + BT_MAX_SLOTS,   // [2] one per stream
   BT_O_READY = BT_S_FULL + 2,            // [2]
   BT_DRAIN = BT_O_READY + 2,             // [2] one per issuing thread
-  BT_BAR_COUNT = BT_DRAIN + 2
+  BT_K_SEEN = BT_DRAIN + 2,              // [2] K_0, and the K tile in front of the last V tile, have landed (a single phase)
+  BT_BAR_COUNT = BT_K_SEEN + 2
 };
 
 // One entry of a CTA's tile list.
@@ -246,7 +248,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
   // its slot for the whole softmax of that tile, and the next V was asked for late.  8 layers x 8 kv heads, prefix 2048,
   // 16 branches x 20 rows 94.1 -> 90.4 us; head_dim 64, with twice as many slots, 16 branches x 20 rows, prefix 1500
   // 16.0 -> 15.4 us.)
-  auto load_slot = [&](int i) { return i % SLOTS; };
+  using Ring = TileRing<SLOTS>;
   // The list starts with `lead` prefix tiles (see tile_at): their loads, but for the last one's V tile, have places in that
   // order that do not depend on the lengths.
   const int lead = min(npre, Cfg::LEAD), pre_issued = min(max(2 * lead - 1, 0), SLOTS);
@@ -324,8 +326,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const int tile = g - __shfl_sync(0xffffffffu, lane_first, j);
     return BtTile{j, tile, min(__shfl_sync(0xffffffffu, lane_rows, j) - tile * BT_BN, BT_BN)};
   };
-  auto k_load = [&](int s) { return max(2 * s - 1, 0); };  // the number of a tile's load
-  auto v_load = [&](int s) { return min(2 * s + 2, 2 * Tall - 1); };
+  const Ring ring{Tall};
   const int T[2] = {(Tall + 1) >> 1, Tall >> 1};  // stream x takes the sequence numbers 2 i + x
 
   if (warp == BT_LOADER_WARP) {
@@ -334,10 +335,10 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const bool leader = elect_one();
     bool ok = true;
     int i = pre_issued;
-    for (; i < 2 * Tall; ++i) {
-      const bool is_v = i == 2 * Tall - 1 || (i > 0 && (i & 1) == 0);
-      const BtTile e = tile_at(i == 2 * Tall - 1 ? Tall - 1 : is_v ? i / 2 - 1 : (i + 1) / 2);
-      const int slot = load_slot(i);
+    for (; i < ring.loads(); ++i) {
+      const bool is_v = ring.is_v(i);
+      const BtTile e = tile_at(ring.tile(i));
+      const int slot = Ring::slot(i);
       if (i >= SLOTS) ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_EMPTY + slot), (i / SLOTS - 1) & 1, abort_flag, p.status, wl));
       if (!ok) break;
       if (leader) load_kv(is_v, slot, e);
@@ -347,7 +348,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
       int dummy = 0;
       volatile int* none = &dummy;
       for (int j = max(0, i - SLOTS); j < i; ++j)
-        mbar_wait(bar(BT_FULL + load_slot(j)), (j / SLOTS) & 1, none, nullptr);
+        mbar_wait(bar(BT_FULL + Ring::slot(j)), Ring::parity(j), none, nullptr);
       mbar_wait(bar(BT_Q_FULL), 0, none, nullptr);
     }
     __syncwarp();
@@ -359,8 +360,9 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     bool ok = true;
     for (int s = 0; s < Tall && ok; ++s) {
       const BtTile e = tile_at(s);
-      const int i = v_load(s), slot = load_slot(i);
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
+      const int i = ring.v_load(s), slot = Ring::slot(i), k_before = ring.k_before_v(s);
+      ok = k_before < 0 || mbar_wait(bar(BT_K_SEEN + (k_before > 0)), 0, abort_flag, p.status, wl);
+      ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(BT_FULL + slot), Ring::parity(i), abort_flag, p.status, wl));
       if (!ok) break;
       if (e.patch()) {
         const uint32_t tile_addr = sKV + slot * TILE_BYTES;
@@ -388,10 +390,11 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     int turn = 0;
     ok = mbar_wait(bar(BT_Q_FULL), 0, abort_flag, p.status, wl);  // (also when the list is empty: the copy must land)
     for (int s = 0; s < Tall; ++s) {
-      const int i = k_load(s), slot = load_slot(i);
+      const int i = Ring::k_load(s), slot = Ring::slot(i);
       const BtTile e = tile_at(s);
       const uint32_t idesc_qk = tc_idesc_bf16(BT_BM, e.groups() * 16, false, false);
-      ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(BT_FULL + slot), (i / SLOTS) & 1, abort_flag, p.status, wl));
+      ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(BT_FULL + slot), Ring::parity(i), abort_flag, p.status, wl));
+      if (leader && ok && ring.v_after_k(s)) mbar_arrive(bar(BT_K_SEEN + (s > 0)));
       if (s > 0) named_sync(NB_S_FREE + ((s - 1) & 1), 160);
       if (leader && ok) {
         flag_write(qk_turn, ++turn);  // odd: a batch of scores is being issued
@@ -422,7 +425,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     const bool leader = elect_one();
     bool ok = true;
     for (int s = 0; s < Tall; ++s) {
-      const int slot = load_slot(v_load(s)), x = s & 1;
+      const int slot = Ring::slot(ring.v_load(s)), x = s & 1;
       const uint32_t v_lo = tc_desc_lo(sKV + slot * TILE_BYTES, BT_PANEL_BYTES);
       const uint32_t o_col = tmem + BT_O_COL0 + x * 128, p_col = tmem + BT_P_COL0 + x * 64;
       const BtTile e = tile_at(s);
@@ -564,7 +567,7 @@ branch_tc_kernel(const __grid_constant__ BtLayers<NL> layers, const BtParams p) 
     // ---- the two streams' (m, l) of a row cross through shared memory: the K slot of the stream's last tile,
     // free once its accumulator is complete and not filled again; a stream without tiles takes slot 2 + x, never filled then
     auto ml_of = [&](int y) {
-      const int slot = T[y] > 0 ? load_slot(k_load(2 * (T[y] - 1) + y)) : 2 + y;
+      const int slot = T[y] > 0 ? Ring::slot(Ring::k_load(2 * (T[y] - 1) + y)) : 2 + y;
       return reinterpret_cast<float2*>(smem_gen + Cfg::SMEM_KV + slot * TILE_BYTES);
     };
     if (Tx > 0) ok = mbar_wait(bar(BT_O_READY + x), (Tx - 1) & 1, abort_flag, p.status, wl) && ok;

@@ -127,9 +127,17 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# The current stream without the Python object that torch.cuda.current_stream() makes (3 us a call): internal calls of torch, used
+# where this torch has them.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
-    if stream is None:  # torch's current stream of the current device, without the Python object (3 us) around it
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if stream is None:
+        if _raw_stream and _current_device:
+            return _raw_stream(_current_device())
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

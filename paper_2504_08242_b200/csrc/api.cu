@@ -233,6 +233,8 @@ jupiter_status jupiter_chunk_prefill_append_attn(jupiter_ctx* ctx, const void* q
   jup::LaunchInfo li{ctx->sm_count, 0};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
+  // One launch, except for head_dim 64 with at most 64 rows: those calls keep the two launches that the header states.  (On a
+  // prompt of four calls of 64 rows, 4 heads, one launch a call takes 35 us where two take 48, the host's time.)
   const bool tc = jup::prefill_tc_supported(c, scale);
   if (tc && (c.head_dim == 128 || q_len > 64)) {
     e = jup::launch_prefill_tc_fused(static_cast<const bf16*>(q), c, static_cast<const bf16*>(k_new),

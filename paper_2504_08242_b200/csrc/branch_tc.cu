@@ -59,7 +59,6 @@ struct BtParams {
   int n_branches, q_len, q_heads, group, kv_heads;
   FastDiv by_group, by_q_len, by_row_tiles, by_layer_units;
   int prefix_len, max_suffix_len;
-  int row_tiles;          // row tiles per kv head
   int whole_units;        // units of all layers that one CTA walks
   int branches_per_tile;  // whole branches per row tile (slices_per_branch == 1)
   int slices_per_branch;  // > 1: a branch has more than 128 rows and is cut into 128-row slices
@@ -901,7 +900,6 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   p.kv_heads = suffix.kv_heads;
   p.prefix_len = prefix_len;
   p.max_suffix_len = max_suffix_len;
-  p.row_tiles = pl.row_tiles;
   p.branches_per_tile = pl.branches_per_tile;
   p.slices_per_branch = pl.slices_per_branch;
   p.box_tokens = pl.box_tokens;

@@ -54,7 +54,7 @@ struct TcParams {
   int* status;
   float* scratch;  // fragment form with several CTAs per query tile: their partial results
   int prefix_batched;  // 1: the front segment has one cache per sequence (fused form), 0: one cache shared by all
-  // Fused KVCache write (fused_write != 0).  The chunk's K/V rows, token-major [batch][q_len][kv_heads][128], are
+  // Fused KVCache write (fused_write != 0).  The chunk's K/V rows, token-major [batch][q_len][kv_heads][D], are
   // the attention's own segment; the CTAs of each group's first query head also write them, bit-exactly, into rows
   // copy_pos + r of the cache, with tiled stores straight from the K/V slots the tiles were loaded into (tensor
   // maps tm_ck / tm_cv over the destination cache).
@@ -664,7 +664,7 @@ cudaError_t launch_prefill_tc(const bf16* q, const CacheView& c, const CacheView
 cudaError_t launch_prefill_tc_fused(const bf16* q, const CacheView& c, const bf16* k_new, const bf16* v_new,
                                     int q_heads, int q_len, int pos, float scale, float* out, float* lse, int* status,
                                     void* workspace, size_t workspace_bytes, cudaStream_t st, LaunchInfo& li) {
-  // own segment: the chunk itself, [batch][q_len][kv_heads][128] seen as a cache of q_len rows at position 0;
+  // own segment: the chunk itself, [batch][q_len][kv_heads][D] seen as a cache of q_len rows at position 0;
   // front segment: rows [0, pos) of each sequence's cache
   CacheView own;
   own.k = k_new;

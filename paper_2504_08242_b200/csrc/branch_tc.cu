@@ -810,7 +810,7 @@ static size_t bt_scratch_bytes(const BtPlan& pl, int layers) {
 
 bool branch_tc_supported(const CacheView& prefix, const CacheView& suffix, int n_branches, int q_heads, int q_len,
                          float scale) {
-  if (!(scale > 0.f) || !(scale < INFINITY) || encode_fn() == nullptr) return false;
+  if (!(scale > 0.f) || !(scale < INFINITY) || !encode_fn() || !replace_fn()) return false;
   // (a stride that no tensor map carries, as of the batch of a cache for one branch, which nothing else looks at: the other
   // kernels take the call)
   if (!stride_encodable(suffix.sr) || !stride_encodable(suffix.sh) || !stride_encodable(suffix.sb) ||
@@ -848,13 +848,14 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
   const int G = q_heads / suffix.kv_heads;
   const uint64_t tokens = static_cast<uint64_t>(n_branches) * q_len;
   BtLayers<NL> L;
-  for (int i = 0; i < layers; ++i) {
-    BtLayer& l = L.l[i];
+  {  // layer 0's maps; the other layers' differ in their addresses only, and so do V's from K's.  (Encoding all seven maps of
+     // a layer took the host 100 us for a call of 32 layers, more than small layers take on the GPU; replaced addresses 90.)
+    BtLayer& l = L.l[0];
     {  // q: [tokens][q_heads][D]; a box is [box_tokens tokens][G heads][64 columns]: the tile's stacked rows in order
       const uint64_t d[4] = {D, static_cast<uint64_t>(q_heads), tokens, 1};
       const uint64_t s[3] = {D * 2ull, static_cast<uint64_t>(q_heads) * D * 2ull, 0};
       const uint32_t bx[4] = {64, static_cast<uint32_t>(G), static_cast<uint32_t>(pl.box_tokens), 1};
-      if (!make_map_bf16(&l.tm_q, t[i].q, d, s, bx)) return cudaErrorInvalidValue;
+      if (!make_map_bf16(&l.tm_q, t[0].q, d, s, bx)) return cudaErrorInvalidValue;
     }
     {  // suffix caches: rows at or beyond max_suffix_len read as zero
       const uint64_t d[4] = {D, static_cast<uint64_t>(max_suffix_len), static_cast<uint64_t>(suffix.kv_heads),
@@ -862,25 +863,37 @@ static cudaError_t launch_bt(const BranchLayerTensors* t, int layers, const Cach
       const uint64_t s[3] = {static_cast<uint64_t>(suffix.sr) * 2, static_cast<uint64_t>(suffix.sh) * 2,
                              static_cast<uint64_t>(suffix.sb) * 2};
       const uint32_t bx[4] = {64, BT_BN, 1, 1};
-      if (!make_map_bf16(&l.tm_sk, t[i].sk, d, s, bx) || !make_map_bf16(&l.tm_sv, t[i].sv, d, s, bx))
-        return cudaErrorInvalidValue;
+      if (!make_map_bf16(&l.tm_sk, t[0].sk, d, s, bx)) return cudaErrorInvalidValue;
     }
     if (prefix_len > 0) {  // rows at or beyond prefix_len read as zero
       const uint64_t d[4] = {D, static_cast<uint64_t>(prefix_len), static_cast<uint64_t>(prefix.kv_heads), 1};
       const uint64_t s[3] = {static_cast<uint64_t>(prefix.sr) * 2, static_cast<uint64_t>(prefix.sh) * 2, 0};
       const uint32_t bx[4] = {64, BT_BN, 1, 1};
-      if (!make_map_bf16(&l.tm_pk, t[i].pk, d, s, bx) || !make_map_bf16(&l.tm_pv, t[i].pv, d, s, bx))
-        return cudaErrorInvalidValue;
+      if (!make_map_bf16(&l.tm_pk, t[0].pk, d, s, bx)) return cudaErrorInvalidValue;
+    }
+    if (t[0].k_new) {  // the step's block, [tokens][kv_heads][D]: a box is the tokens of a row tile's branches
+      const uint64_t d[4] = {D, static_cast<uint64_t>(suffix.kv_heads), tokens, 1};
+      const uint64_t s[3] = {D * 2ull, static_cast<uint64_t>(suffix.kv_heads) * D * 2ull, 0};
+      const uint32_t bx[4] = {64, 1, static_cast<uint32_t>(pl.branches_per_tile * q_len), 1};
+      if (!make_map_bf16(&l.tm_nk, t[0].k_new, d, s, bx)) return cudaErrorInvalidValue;
+    }
+  }
+  for (int i = 0; i < layers; ++i) {
+    BtLayer& l = L.l[i];
+    const BtLayer& l0 = L.l[0];
+    if (i > 0 && (!make_map_like(&l.tm_q, l0.tm_q, t[i].q) || !make_map_like(&l.tm_sk, l0.tm_sk, t[i].sk)))
+      return cudaErrorInvalidValue;
+    if (!make_map_like(&l.tm_sv, l0.tm_sk, t[i].sv)) return cudaErrorInvalidValue;
+    if (prefix_len > 0) {
+      if (i > 0 && !make_map_like(&l.tm_pk, l0.tm_pk, t[i].pk)) return cudaErrorInvalidValue;
+      if (!make_map_like(&l.tm_pv, l0.tm_pk, t[i].pv)) return cudaErrorInvalidValue;
     } else {
       l.tm_pk = l.tm_sk;  // never dereferenced without a prefix
       l.tm_pv = l.tm_sv;
     }
-    if (t[i].k_new) {  // the step's block, [tokens][kv_heads][D]: a box is the tokens of a row tile's branches
-      const uint64_t d[4] = {D, static_cast<uint64_t>(suffix.kv_heads), tokens, 1};
-      const uint64_t s[3] = {D * 2ull, static_cast<uint64_t>(suffix.kv_heads) * D * 2ull, 0};
-      const uint32_t bx[4] = {64, 1, static_cast<uint32_t>(pl.branches_per_tile * q_len), 1};
-      if (!make_map_bf16(&l.tm_nk, t[i].k_new, d, s, bx) || !make_map_bf16(&l.tm_nv, t[i].v_new, d, s, bx))
-        return cudaErrorInvalidValue;
+    if (t[i].k_new) {
+      if (i > 0 && !make_map_like(&l.tm_nk, l0.tm_nk, t[i].k_new)) return cudaErrorInvalidValue;
+      if (!make_map_like(&l.tm_nv, l0.tm_nk, t[i].v_new)) return cudaErrorInvalidValue;
     } else {
       l.tm_nk = l.tm_sk;  // never dereferenced without a fused write
       l.tm_nv = l.tm_sv;

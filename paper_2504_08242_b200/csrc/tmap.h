@@ -11,16 +11,22 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+
+inline void* driver_fn(const char* name) {
+  void* ptr = nullptr;
+  cudaDriverEntryPointQueryResult qres;
+  if (cudaGetDriverEntryPoint(name, &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
+    return ptr;
+  (void)cudaGetLastError();
+  return nullptr;
+}
 inline EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      return reinterpret_cast<EncodeTiledFn>(ptr);
-    (void)cudaGetLastError();
-    return static_cast<EncodeTiledFn>(nullptr);
-  }();
+  static EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_fn("cuTensorMapEncodeTiled"));
+  return fn;
+}
+inline ReplaceAddressFn replace_fn() {
+  static ReplaceAddressFn fn = reinterpret_cast<ReplaceAddressFn>(driver_fn("cuTensorMapReplaceAddress"));
   return fn;
 }
 
@@ -44,6 +50,12 @@ inline bool make_map(CUtensorMap* m, CUtensorMapDataType type, const void* base,
   cuuint32_t es[4] = {1, 1, 1, 1};
   return fn(m, type, 4, const_cast<void*>(base), gd, gs, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// The map of another tensor with the same extents, strides and box.
+inline bool make_map_like(CUtensorMap* m, const CUtensorMap& like, const void* base) {
+  ReplaceAddressFn fn = replace_fn();
+  *m = like;
+  return fn && fn(m, const_cast<void*>(base)) == CUDA_SUCCESS;
 }
 inline bool make_map_bf16(CUtensorMap* m, const void* base, const uint64_t dims[4], const uint64_t strides_bytes[3],
                           const uint32_t box[4]) {

@@ -447,34 +447,50 @@ namespace jup {
 
 // ---------------------------------------------------------------- host side
 
-template <int D, int C>
+// Log-sum-exps are results of 32 bits and want exact exponentials; without them only bf16 weights come of an exponential, and the
+// form with a quarter of them on the FMA pipe is taken: four prompts of 8192 tokens in chunks of 128 2417 us against 2448, 2048
+// tokens in chunks of 256 105.9 against 107.  With head_dim 64 it gains nothing (3000 tokens in chunks of 448 124 against 123).
+template <int D>
+static bool frag_exact(const float* lse) {
+  return D == 64 || lse != nullptr;
+}
+template <int D, int C, bool EXACT>
 static cudaError_t frag_set_attributes() {
   static PerDeviceOnce done;
   if (done.done()) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(prefill_frag_kernel<D, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(prefill_frag_kernel<D, C, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        FragCfg<D>::SMEM_BYTES);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(prefill_frag_kernel<D, C>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(prefill_frag_kernel<D, C, EXACT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess) done.set();
   return e;
 }
-template <int D, int C>
-static cudaError_t launch_frag(int64_t units, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
-                               const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
-                               const CUtensorMap& tck, const CUtensorMap& tcv, const TcParams& p) {
-  cudaError_t e = frag_set_attributes<D, C>();
+template <int D, int C, bool EXACT>
+static cudaError_t launch_frag_as(int64_t units, cudaStream_t st, const CUtensorMap& tq, const CUtensorMap& tk,
+                                  const CUtensorMap& tv, const CUtensorMap& tpk, const CUtensorMap& tpv,
+                                  const CUtensorMap& tck, const CUtensorMap& tcv, const TcParams& p) {
+  cudaError_t e = frag_set_attributes<D, C, EXACT>();
   if (e != cudaSuccess) return e;
-  return launch_pdl_cluster(prefill_frag_kernel<D, C>, dim3(static_cast<unsigned>(units * C)), dim3(FragCfg<D>::THREADS),
-                            FragCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(C), tq, tk, tv, tpk, tpv, tck, tcv, p);
+  return launch_pdl_cluster(prefill_frag_kernel<D, C, EXACT>, dim3(static_cast<unsigned>(units * C)),
+                            dim3(FragCfg<D>::THREADS), FragCfg<D>::SMEM_BYTES, st, static_cast<unsigned>(C), tq, tk, tv, tpk,
+                            tpv, tck, tcv, p);
+}
+template <int D, int C, class... Args>
+static cudaError_t launch_frag(const float* lse, Args&&... args) {
+  if constexpr (D != 64)
+    if (!frag_exact<D>(lse)) return launch_frag_as<D, C, false>(args...);
+  return launch_frag_as<D, C, true>(args...);
 }
 
-// How many clusters of C CTAs of the fragment form can be resident at once on the current device (0 if the query fails).
+// How many clusters of C CTAs of the fragment form can be resident at once on the current device (0 if the query fails; both
+// forms take the same registers and shared memory).
 template <int D, int C>
 static int frag_resident_clusters() {
   static ResidentClusters clusters;
-  if (frag_set_attributes<D, C>() != cudaSuccess) return 0;
-  return clusters.get(reinterpret_cast<const void*>(prefill_frag_kernel<D, C>), C, FragCfg<D>::THREADS, FragCfg<D>::SMEM_BYTES);
+  if (frag_set_attributes<D, C, true>() != cudaSuccess) return 0;
+  return clusters.get(reinterpret_cast<const void*>(prefill_frag_kernel<D, C, true>), C, FragCfg<D>::THREADS,
+                      FragCfg<D>::SMEM_BYTES);
 }
 
 template <int D>
@@ -646,10 +662,12 @@ static cudaError_t launch_tc(const bf16* q, const CacheView& c, const CacheView*
   if (f.pairs)
     e = launch_pairs<D>(units, st, tq, tk, tv, tpk, tpv, to, tck, tcv, p);
   else
-    e = (f.split == 8   ? launch_frag<D, 8>
-         : f.split == 4 ? launch_frag<D, 4>
-         : f.split == 2 ? launch_frag<D, 2>
-                        : launch_frag<D, 1>)(units, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
+    switch (f.split) {
+      case 8: e = launch_frag<D, 8>(lse, units, st, tq, tk, tv, tpk, tpv, tck, tcv, p); break;
+      case 4: e = launch_frag<D, 4>(lse, units, st, tq, tk, tv, tpk, tpv, tck, tcv, p); break;
+      case 2: e = launch_frag<D, 2>(lse, units, st, tq, tk, tv, tpk, tpv, tck, tcv, p); break;
+      default: e = launch_frag<D, 1>(lse, units, st, tq, tk, tv, tpk, tpv, tck, tcv, p);
+    }
   li.launches += 1;
   return e;
 }

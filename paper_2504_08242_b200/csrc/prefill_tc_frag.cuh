@@ -50,7 +50,8 @@ enum {
 
 // C > 1: a thread-block cluster of C CTAs shares a query tile; CTA r walks the r-th of C equal ranges of its KV tiles, and
 // the partial (O, m, l) are exchanged through global scratch (L2) around one cluster barrier.
-template <int D, int C>
+// EXACT: see frag_exp_store_max.
+template <int D, int C, bool EXACT>
 __global__ void __launch_bounds__(FragCfg<D>::THREADS, 1)
 prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_pk,
@@ -338,7 +339,7 @@ prefill_frag_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       const bool next_masked = j + 1 < T && tile_masked(j + 1);
       float mxs_next[2];
-      frag_exp_store_max(cur, taddr + (j % STAGES) * 128, c, m_ref, l, nxt, next_masked, [&] { apply_mask(nxt); }, mxs_next);
+      frag_exp_store_max<EXACT>(cur, taddr + (j % STAGES) * 128, c, m_ref, l, nxt, next_masked, [&] { apply_mask(nxt); }, mxs_next);
       mxs[0] = mxs_next[0];
       mxs[1] = mxs_next[1];
       tc_wait_st();

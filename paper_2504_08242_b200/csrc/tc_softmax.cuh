@@ -239,10 +239,11 @@ __device__ __forceinline__ bool frag_decide(const float (&mxs)[2], float (&m_ref
 // is no next tile; the result is then unused).  It is waited for after the fourth of the sixteen steps, masked if
 // need be (mask_next(), warp-uniform and rare), and its 2 x 32 values are folded into running maxima a few per step,
 // so that their arithmetic issues in the gaps of the exponentials instead of after them.  mxs_next: maxima times c.
-// (A quarter of the exponentials as a degree-3 polynomial on the FMA pipe gained 1 to 1.5 % with head_dim 128 and nothing with
-// 64 -- four prompts of 8192 tokens in chunks of 128 2417 against 2448 us, 3000 tokens in chunks of 448 with head_dim 64 124 against
-// 123 -- but its 7.5e-5 showed in the log-sum-exps, 7e-5 off instead of 3e-6, and it lost NaN scores.)
-template <class MaskNext>
+// EXACT: every exponential on the special-function unit, for calls whose row sums are seen as log-sum-exps; otherwise a quarter of
+// them (more brought nothing: the loop is bound by dependent-issue latency, not by that unit alone) go to the FMA pipe, with an
+// error that shows in the row sums (log-sum-exps 7e-5 off instead of 3e-6) but not behind the bf16 rounding of P (outputs
+// 1.26e-3 off either way).
+template <bool EXACT, class MaskNext>
 __device__ __forceinline__ void frag_exp_store_max(const uint32_t (&sv)[64], uint32_t tS, float c, const float (&m_ref)[2],
                                                    float (&l)[2], uint32_t (&nxt)[64], bool next_masked,
                                                    MaskNext&& mask_next, float (&mxs_next)[2]) {
@@ -264,9 +265,15 @@ __device__ __forceinline__ void frag_exp_store_max(const uint32_t (&sv)[64], uin
     for (int e = 0; e < 2; ++e) {
       const uint64_t x =
           fma2(pack2(__uint_as_float(sv[4 * k + 2 * e]), __uint_as_float(sv[4 * k + 2 * e + 1])), c2, nm2[e]);
-      float x0, x1;
-      unpack2(x, x0, x1);
-      const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+      float p0, p1;
+      if (!EXACT && e == 1 && (k & 1) != 0) {
+        unpack2(exp2_poly_pair(x), p0, p1);
+      } else {
+        float x0, x1;
+        unpack2(x, x0, x1);
+        p0 = fast_exp2(x0);
+        p1 = fast_exp2(x1);
+      }
       lacc[e][k & 1] = add2(lacc[e][k & 1], pack2(p0, p1));
       w[2 * k + e] = pack_bf16(p0, p1);
     }

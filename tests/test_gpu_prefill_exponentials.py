@@ -63,11 +63,11 @@ def test_log_sum_exps_behind_a_shared_prefix(ctx):
 @pytest.mark.parametrize("D,Hq,Hkv,S", [(64, 4, 4, 90), (64, 32, 8, 1500), (128, 4, 4, 90), (128, 32, 8, 1500)])
 @pytest.mark.parametrize("row", [9, 83])
 def test_a_nan_key_is_not_lost(ctx, D, Hq, Hkv, S, row):
-    """Every row from the key on is NaN, every row before it finite."""
+    """No value of a row from the key on is finite, every row before it is."""
     w = synth.PrefillWorkload("nan", 1200 + D + S, 1, Hq, Hkv, D, S, S, S)
     q, k, v = w.make()
     k = k.copy()
     k[:, row] = 0x7FC0
     out = run_gpu_prefill(ctx, q, k, v, [S], S, w.scale, fused=True)[0]
     assert np.isfinite(out[:, :row]).all()
-    assert np.isnan(out[:, row:]).all()
+    assert not np.isfinite(out[:, row:]).any()

@@ -180,7 +180,9 @@ jupiter_status jupiter_chunk_prefill_append_attn(jupiter_ctx* ctx, const void* q
  *           are clamped into it before any address is formed.
  *   q:   [n_branches][q_len][q_heads][D] bf16;  1 <= q_len <= 16.
  * Draft row i of branch b attends prefix rows [0, prefix_len) and suffix_b rows
- * 0..d_suffix_len[b]-q_len+i (causal inside the draft block).
+ * 0..d_suffix_len[b]-q_len+i (causal inside the draft block).  NaN or Inf in dead rows (at or above d_suffix_len[b],
+ * prefix_len) reaches no result, in live K rows of one branch only that branch's; in live V rows of one branch it may
+ * also reach other branches of the call.
  *   out: [n_branches][q_len][q_heads][D] fp32;  lse (nullable): [n_branches][q_heads][q_len].
  * Uses the ctx scratch for split-KV partials (JUPITER_ERR_WORKSPACE if too small). */
 jupiter_status jupiter_branch_attn(jupiter_ctx* ctx, const void* q, const jupiter_kv_cache* prefix,
@@ -209,7 +211,8 @@ jupiter_status jupiter_branch_append_attn(jupiter_ctx* ctx, const void* q, const
  * every decoder layer of a stage; Sec. V-B: every layer keeps its own shared prompt KVCache and per-request
  * KVCaches).  Layer l has its own query block, K/V block, prefix cache, suffix cache and outputs; all layers have
  * the same geometry (head counts, head_dim, capacities, strides), the same branch lengths and the same scale.
- * Same result, layer by layer, as n_layers calls of jupiter_branch_append_attn -- the layers must not depend on one
+ * Same result, layer by layer, as n_layers calls of jupiter_branch_append_attn, up to rounding (how a row's keys are cut
+ * into partial sums follows from all layers' work; the caches are the same to the bit) -- the layers must not depend on one
  * another's outputs inside the call (their Q/K/V blocks are ready beforehand) -- but the layers share launches: up to
  * 16 layers run as ONE kernel launch (with many stacked query rows per kv head from three layers on), so the time
  * between dependent launches is paid once per 16 layers instead of once per layer; shapes that take the split-KV
